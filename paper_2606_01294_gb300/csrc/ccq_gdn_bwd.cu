@@ -20,6 +20,13 @@ size_t per_chunk_floats(int D) {
     return 64 * 64 + 5 * d * d + 2 * d + 6 * 64 * d + 4 * 64;
 }
 
+// The first array: the workspace is 16-byte aligned, the kernels for bf16 and D = 128 access the arrays
+// 32 bytes at a time.
+float *array_base(const GdnBwdCall &c) {
+    const uintptr_t p = reinterpret_cast<uintptr_t>(c.workspace);
+    return reinterpret_cast<float *>(c.bf16 && c.D == 128 ? (p + 31) & ~static_cast<uintptr_t>(31) : p);
+}
+
 template <typename K>
 cudaError_t allow_smem(K kernel, size_t bytes) {
     return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bytes));
@@ -61,27 +68,33 @@ cudaError_t run(gbwd::GdnBwdArgs a, cudaStream_t s) {
     constexpr bool kTc = std::is_same<Tin, __nv_bfloat16>::value;
     cudaError_t e;
     if (kTc && !(a.status = device_status_word())) return cudaErrorInvalidValue;
-    if ((e = allow_smem(gdn_bwd_prep_kernel<D, Tin>, prep_smem<D>())) != cudaSuccess) return e;
-    if ((e = allow_smem(gdn_bwd_local_kernel<D, Tin, kTc>, local_smem<D, kTc>())) != cudaSuccess) return e;
-    if ((e = allow_smem(gdn_bwd_kv_kernel<D, Tin, kTc>, kv_smem<D, kTc>())) != cudaSuccess) return e;
     const unsigned nch = static_cast<unsigned>(a.B * a.H * a.NC), bh = static_cast<unsigned>(a.B * a.H);
     const long long elems = (static_cast<long long>(D) * D + D) * a.B * a.H;
     const unsigned eblocks = static_cast<unsigned>((elems + 255) / 256);
-    if (!a.states_ready) {
+    if constexpr (kTc && D == 128) {
+        // the forward's per-chunk quantities are in the workspace (GdnBwdCall::states_ready)
+        if (!a.states_ready) return cudaErrorInvalidValue;
+        int dev = 0, sms = 0;
+        if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+        if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+        a.wave = sms;
+        if ((e = launch_gdn_local128(a, s)) != cudaSuccess) return e;
+        if ((e = launch_gdn_dstate_tc(a, a.k, s)) != cudaSuccess) return e;
+        gdn_bwd_suffix_kernel<D><<<eblocks, 256, 0, s>>>(a);
+        return launch_gdn_kv128(a, s);
+    } else {
+        if ((e = allow_smem(gdn_bwd_prep_kernel<D, Tin>, prep_smem<D>())) != cudaSuccess) return e;
+        if ((e = allow_smem(gdn_bwd_local_kernel<D, Tin, kTc>, local_smem<D, kTc>())) != cudaSuccess) return e;
+        if ((e = allow_smem(gdn_bwd_kv_kernel<D, Tin, kTc>, kv_smem<D, kTc>())) != cudaSuccess) return e;
         gdn_bwd_prep_kernel<D, Tin><<<nch, 256, prep_smem<D>(), s>>>(a);
         gdn_bwd_prefix_kernel<D><<<eblocks, 256, 0, s>>>(a);
         if ((e = launch_fstate<D, Tin>(a, bh, s)) != cudaSuccess) return e;
+        gdn_bwd_local_kernel<D, Tin, kTc><<<nch, kBwdThreads, local_smem<D, kTc>(), s>>>(a);
+        if ((e = launch_dstate<D, Tin>(a, bh, s)) != cudaSuccess) return e;
+        gdn_bwd_suffix_kernel<D><<<eblocks, 256, 0, s>>>(a);
+        gdn_bwd_kv_kernel<D, Tin, kTc><<<nch, kBwdThreads, kv_smem<D, kTc>(), s>>>(a);
+        return cudaGetLastError();
     }
-    gdn_bwd_local_kernel<D, Tin, kTc><<<nch, kBwdThreads, local_smem<D, kTc>(), s>>>(a);
-    if (D == 128 && std::is_same<Tin, __nv_bfloat16>::value && a.states_ready) {
-        // bf16, Dk = 128: the reverse state pass on tensor cores
-        if ((e = launch_gdn_dstate_tc(a, a.k, s)) != cudaSuccess) return e;
-    } else if ((e = launch_dstate<D, Tin>(a, bh, s)) != cudaSuccess) {
-        return e;
-    }
-    gdn_bwd_suffix_kernel<D><<<eblocks, 256, 0, s>>>(a);
-    gdn_bwd_kv_kernel<D, Tin, kTc><<<nch, kBwdThreads, kv_smem<D, kTc>(), s>>>(a);
-    return cudaGetLastError();
 }
 
 }  // namespace
@@ -89,7 +102,7 @@ cudaError_t run(gbwd::GdnBwdArgs a, cudaStream_t s) {
 void gdn_bwd_state_arrays(const GdnBwdCall &c, float **tt, float **sk, float **mk, float **hs) {
     const size_t chunks = static_cast<size_t>(c.B) * c.H * ((c.T + 63) / 64);
     const size_t d = static_cast<size_t>(c.D);
-    float *p = static_cast<float *>(c.workspace);
+    float *p = array_base(c);
     *tt = p;
     *sk = p + chunks * 64 * 64;
     *mk = *sk + chunks * d * d;
@@ -116,11 +129,14 @@ cudaError_t launch_gdn_bwd(const GdnBwdCall &c, cudaStream_t s) {
     a.dS0 = c.dS0; a.dC0 = c.dC0; a.dm0 = c.dm0;
     const size_t chunks = static_cast<size_t>(c.B) * c.H * a.NC;
     const size_t d = static_cast<size_t>(c.D);
-    float *p = static_cast<float *>(c.workspace);
+    float *p = array_base(c);
     auto take = [&](size_t per) { float *r = p; p += chunks * per; return r; };
     a.tt = take(64 * 64); a.sk = take(d * d); a.mk = take(d); a.hs = take(d * d); a.dh = take(d * d);
     a.dc = take(d * d); a.dm = take(d); a.x1 = take(64 * d); a.y1 = take(d * d);
-    a.qb = take(64 * d); a.qc = take(64 * d); a.u = take(64 * d); a.r = take(64 * d); a.w = take(64 * d);
+    // the bf16 kernels for D = 128 form qbar again from q: their arrays need no room for it, which
+    // leaves room for array_base()'s alignment
+    a.qb = c.bf16 && c.D == 128 ? nullptr : take(64 * d);
+    a.qc = take(64 * d); a.u = take(64 * d); a.r = take(64 * d); a.w = take(64 * d);
     a.vec = take(4 * 64);
     if (c.D == 128) return c.bf16 ? run<128, __nv_bfloat16>(a, s) : run<128, float>(a, s);
     if (c.D == 64) return c.bf16 ? run<64, __nv_bfloat16>(a, s) : run<64, float>(a, s);

@@ -37,6 +37,10 @@ void gdn_bwd_state_arrays(const GdnBwdCall &c, float **tt, float **sk, float **m
 cudaError_t launch_gdn_bwd(const GdnBwdCall &c, cudaStream_t s);
 // The reverse state pass on tensor cores (ccq_gdn_bwd_state_tc.cu): Dk = Dv = 128, bf16 keys k.
 cudaError_t launch_gdn_dstate_tc(const gbwd::GdnBwdArgs &a, const void *k, cudaStream_t s);
+// The per-chunk kernels for Dk = Dv = 128 and bf16 inputs (ccq_gdn_bwd_chunk_tc.cu); the workspace arrays
+// are 32-byte aligned.
+cudaError_t launch_gdn_local128(const gbwd::GdnBwdArgs &a, cudaStream_t s);
+cudaError_t launch_gdn_kv128(const gbwd::GdnBwdArgs &a, cudaStream_t s);
 // A 2-D tensor map over an fp32 [rows][cols] array with (box_cols x box_rows) boxes, 128-byte
 // swizzled (box_cols * 4 = 128).
 bool make_f32_rows_map(CUtensorMap *map, const void *base, long long rows, int cols, int box_cols, int box_rows);

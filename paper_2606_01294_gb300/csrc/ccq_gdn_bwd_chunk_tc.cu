@@ -1,0 +1,1221 @@
+// ccq_gdn_bwd_chunk_tc.cu -- the per-chunk kernels of the CCQ-Gated-DeltaNet backward for bf16 inputs
+// with Dk = Dv = 128: bf16 operand tiles in shared memory, accumulators in TMEM, fp32 rows in registers.
+//
+// The adjoint is the one ccq_gdn_bwd_kernels.cuh states; gdn_bwd_local128_kernel and
+// gdn_bwd_kv128_kernel stand in for its local and kv kernels.  Every product's operands are the bf16
+// roundings of the same fp32 quantities and accumulate in fp32, as there; what differs is where they live:
+//   - an operand is rounded once, into a 128-byte-swizzled tile that serves as a K-major or an MN-major
+//     operand of every product that reads it (the kernels of that file convert both operands of every
+//     product, a conversion pass and two block barriers each);
+//   - an element-wise quantity stays in the registers of the thread that owns it, from the accumulator read
+//     that makes it to the last one that needs it; row sums cross the eight threads of a row through one
+//     shuffle and four shared-memory partial sums, column sums and column prefix sums run as shuffles over
+//     the sixteen rows of a half-warp;
+//   - a seventeenth warp issues the products (six rounds in the local kernel, five in the kv one), in an
+//     order that lets the next epilogue start on the first half of a round while the rest runs.
+// What bounds them: one CTA fits an SM (about 200 KB of tiles, all of TMEM), so a chunk is the latency of its
+// load, its rounds and its epilogues.  Measured on GB300 (B = 4, H = 16, T = 4096, 4096 chunks): see the
+// two kernels below.
+//
+// Thread layout: 512 compute threads.  Warp w, lane l: TMEM quadrant qd = w % 4, column group grp = w / 4;
+// in a 64-row product the thread holds row i = 16 qd + l % 16 and, with hf = l / 16, columns
+// 64 hf + 16 grp .. + 15 of a 128-column accumulator or 32 hf + 8 grp .. + 7 of a 64-column one; in a
+// 128-row product row 32 qd + l, columns 32 grp .. + 31.
+#include <cuda_bf16.h>
+#include <cuda_runtime.h>
+#include <stdint.h>
+
+#include "ccq_gdn_bwd.h"
+#include "ccq_gdn_bwd_kernels.cuh"
+#include "ccq_internal.h"
+#include "sm100_ptx.cuh"
+
+namespace ccq {
+
+namespace {
+
+using gbwd::GdnBwdArgs;
+
+constexpr int kC = 64, kD = 128;
+constexpr int kCompute = 512, kAll = kCompute + 32;
+
+constexpr uint32_t ID_64x64_KK = make_idesc(64, 64, 0, 0), ID_64x64_MM = make_idesc(64, 64, 1, 1);
+constexpr uint32_t ID_64x128_KK = make_idesc(64, 128, 0, 0), ID_64x128_KM = make_idesc(64, 128, 0, 1);
+constexpr uint32_t ID_64x128_MM = make_idesc(64, 128, 1, 1), ID_128x128_MM = make_idesc(128, 128, 1, 1);
+
+__device__ __forceinline__ void compute_sync() { named_bar(1, kCompute); }
+// The compute threads' tiles and TMEM reads of a round are done: release the issuing warp.
+__device__ __forceinline__ void signal_issue(int id) {
+    fence_proxy_async_smem();
+    tc_fence_before();
+    named_bar_arrive(id, kAll);
+}
+
+// 256-bit global accesses: a thread's rows of 16 or 32 floats are 32-byte sectors of their own (32-byte
+// aligned; the workspace arrays are).
+__device__ __forceinline__ void st_global8(float *p, const float *v) {
+    asm volatile("st.global.v8.f32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(p), "f"(v[0]), "f"(v[1]), "f"(v[2]),
+                 "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7])
+                 : "memory");
+}
+__device__ __forceinline__ void ld_global8(const float *p, float *v) {
+    asm volatile("ld.global.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                 : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7])
+                 : "l"(p));
+}
+
+// Accumulator columns of a 64-row product, without the wait: NR values at columns [c, c + NR) for lanes
+// 0-15 and [c + OFF, c + OFF + NR) for lanes 16-31 (the same sixteen rows).
+__device__ __forceinline__ void acc_ld16(uint32_t taddr, float (&v)[16]) {  // OFF = 64
+    uint32_t r[16];
+    asm volatile(
+        "tcgen05.ld.sync.aligned.16x32bx2.x16.b32 "
+        "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16], 64;\n\t"
+        "tcgen05.wait::ld.sync.aligned;"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+        : "r"(taddr)
+        : "memory");
+#pragma unroll
+    for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
+}
+__device__ __forceinline__ void acc_ld8(uint32_t taddr, float (&v)[8]) {  // OFF = 32
+    uint32_t r[8];
+    asm volatile(
+        "tcgen05.ld.sync.aligned.16x32bx2.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8], 32;\n\t"
+        "tcgen05.wait::ld.sync.aligned;"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+        : "r"(taddr)
+        : "memory");
+#pragma unroll
+    for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[i]);
+}
+
+__device__ __forceinline__ uint4 pack8(const float *f) {
+    return make_uint4(pack_bf16(f[0], f[1]), pack_bf16(f[2], f[3]), pack_bf16(f[4], f[5]), pack_bf16(f[6], f[7]));
+}
+// The thread's 16 columns of a [64][128] tile (two T64 tiles 8 KB apart) / 8 columns of a [64][64] one: the
+// eight lanes of a quarter-warp write one chunk of eight consecutive rows, swizzled apart (no bank conflict).
+__device__ __forceinline__ void put16(uint8_t *tile, int i, int hf, int grp, const float (&f)[16]) {
+    *reinterpret_cast<uint4 *>(tile + hf * 8192 + t64_chunk(i, 2 * grp)) = pack8(f);
+    *reinterpret_cast<uint4 *>(tile + hf * 8192 + t64_chunk(i, 2 * grp + 1)) = pack8(f + 8);
+}
+__device__ __forceinline__ void put8(uint8_t *tile, int i, int hf, int grp, const float (&f)[8]) {
+    *reinterpret_cast<uint4 *>(tile + t64_chunk(i, 4 * hf + grp)) = pack8(f);
+}
+
+// 16 consecutive values of a token row (zero past the sequence).
+struct Raw16 {
+    uint4 a, b;
+};
+__device__ __forceinline__ Raw16 load_raw16(const void *base, size_t row, int c0, bool valid) {
+    Raw16 x{make_uint4(0u, 0u, 0u, 0u), make_uint4(0u, 0u, 0u, 0u)};
+    if (valid) {
+        const uint4 *p = reinterpret_cast<const uint4 *>(static_cast<const __nv_bfloat16 *>(base) + row * kD + c0);
+        x.a = p[0];
+        x.b = p[1];
+    }
+    return x;
+}
+__device__ __forceinline__ void unpack16(const Raw16 &x, float (&f)[16]) {
+    float lo[8], hi[8];
+    unpack_bf16x8(x.a, lo);
+    unpack_bf16x8(x.b, hi);
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+        f[e] = lo[e];
+        f[8 + e] = hi[e];
+    }
+}
+__device__ __forceinline__ void store_row16(void *base, size_t row, int c0, const float (&f)[16]) {
+    uint4 *p = reinterpret_cast<uint4 *>(static_cast<__nv_bfloat16 *>(base) + row * kD + c0);
+    p[0] = pack8(f);
+    p[1] = pack8(f + 8);
+}
+
+// The fp32 chunk tiles that one kernel writes and the other reads in the same thread layout (R, U, W):
+// 32 bytes a thread, consecutive threads consecutive in memory.
+__device__ __forceinline__ void st_own16(float *tile, int tid, const float (&f)[16]) {
+    st_global8(tile + 8 * tid, f);
+    st_global8(tile + 8 * (kCompute + tid), f + 8);
+}
+__device__ __forceinline__ void ld_own16(const float *tile, int tid, float (&f)[16]) {
+    ld_global8(tile + 8 * tid, f);
+    ld_global8(tile + 8 * (kCompute + tid), f + 8);
+}
+
+// An fp32 [128][128] array as a bf16 operand tile (two T64 tiles of 128 rows, 16 KB apart).
+__device__ __forceinline__ void stage_square(uint8_t *tile, const float *src, int tid) {
+    float f[4][8];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) ld_global8(src + 8 * (tid + kCompute * u), f[u]);
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        const int it = tid + kCompute * u, row = it >> 4, ch = it & 15;
+        *reinterpret_cast<uint4 *>(tile + (ch >> 3) * 16384 + t64_chunk(row, ch & 7)) = pack8(f[u]);
+    }
+}
+
+// Sums over the sixteen rows of a half-warp of N columns: leaves in v[0] the sum of column lane & 15 (N = 16)
+// or (lane >> 1) & 7 (N = 8).
+template <int N>
+__device__ __forceinline__ void col_sums(float (&v)[N], int lane) {
+    int m = N;
+#pragma unroll
+    for (int o = 8; o >= 1; o >>= 1) {
+        if (m > 1) {
+            m >>= 1;
+            const bool up = (lane & o) != 0;
+#pragma unroll
+            for (int e = 0; e < N / 2; ++e)
+                if (e < m) {
+                    const float send = up ? v[e] : v[e + m], keep = up ? v[e + m] : v[e];
+                    v[e] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+                }
+        } else {
+            v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+        }
+    }
+}
+
+// Row sums: the eight threads of row i add up (two by shuffle, four through red[4][64]).
+__device__ __forceinline__ void row_part(float *red, int grp, int i, int hf, float x) {
+    x += __shfl_xor_sync(0xffffffffu, x, 16);
+    if (hf == 0) red[grp * kC + i] = x;
+}
+__device__ __forceinline__ float row_total(const float *red, int i) {
+    return (red[i] + red[kC + i]) + (red[2 * kC + i] + red[3 * kC + i]);
+}
+
+// The scalars of the chunk's tokens, by the issuing warp (two tokens a lane): in-chunk cumulative log
+// decay gc (held past the sequence; summed token by token, one lane), E = e^{gc}, 1 / t, beta, lambda.
+__device__ __forceinline__ void token_scalars(const GdnBwdArgs &a, int b, int h, int r, int lane, float *gc, float *E,
+                                              float *be, float *tinv, float *lam) {
+    const int t0 = r * kC + 2 * lane;
+    const bool v0 = t0 < a.T, v1 = t0 + 1 < a.T;
+    const size_t r0 = (static_cast<size_t>(b) * a.T + (v0 ? t0 : 0)) * a.H + h;
+    const size_t r1 = (static_cast<size_t>(b) * a.T + (v1 ? t0 + 1 : 0)) * a.H + h;
+    *reinterpret_cast<float2 *>(gc + 2 * lane) = make_float2(v0 ? a.g[r0] : 0.f, v1 ? a.g[r1] : 0.f);
+    be[2 * lane] = v0 ? a.beta[r0] : 0.f;
+    be[2 * lane + 1] = v1 ? a.beta[r1] : 0.f;
+    if (lam) {
+        lam[2 * lane] = v0 ? a.lambda[r0] : 0.f;
+        lam[2 * lane + 1] = v1 ? a.lambda[r1] : 0.f;
+    }
+    const float ts = static_cast<float>((a.t0 ? a.t0[b] : 0) + static_cast<int64_t>(r) * kC);
+    tinv[2 * lane] = 1.f / (ts + 1.f + static_cast<float>(2 * lane));
+    tinv[2 * lane + 1] = 1.f / (ts + 1.f + static_cast<float>(2 * lane + 1));
+    __syncwarp();
+    if (lane == 0) {
+        float acc = 0.f;
+#pragma unroll
+        for (int q = 0; q < kC / 4; ++q) {
+            float4 x = *reinterpret_cast<const float4 *>(gc + 4 * q);
+            x.x = acc + x.x;
+            x.y = x.x + x.y;
+            x.z = x.y + x.z;
+            acc = x.w = x.z + x.w;
+            *reinterpret_cast<float4 *>(gc + 4 * q) = x;
+        }
+    }
+    __syncwarp();
+    E[2 * lane] = expf(gc[2 * lane]);
+    E[2 * lane + 1] = expf(gc[2 * lane + 1]);
+}
+
+// Sums over a row's columns in eight interleaved parts (columns p, p + 8, ..., each summed in order, then
+// the parts in order): four neighbouring threads take two parts each.  The order is that of row_sums() in
+// ccq_gdn_bwd_kernels.cuh, so that a row rounds to the same bf16 operands in either kernel.
+__device__ __forceinline__ float parts_total(float p0, float p1, int lane) {
+    float s = 0.f;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        s += __shfl_sync(0xffffffffu, p0, (lane & 28) + q);
+        s += __shfl_sync(0xffffffffu, p1, (lane & 28) + q);
+    }
+    return s;
+}
+// Columns 2 qtr, 2 qtr + 1 of every 16-byte chunk of row `row` of a raw [64][128] tile.
+__device__ __forceinline__ void load_parts(const uint8_t *tile, int row, int qtr, uint32_t (&w)[16]) {
+#pragma unroll
+    for (int c = 0; c < 16; ++c)
+        w[c] = *reinterpret_cast<const uint32_t *>(tile + (c >> 3) * 8192 + t64_chunk(row, c & 7) + 4 * qtr);
+}
+__device__ __forceinline__ float lo_bf16(uint32_t w) { return __uint_as_float(w << 16); }
+__device__ __forceinline__ float hi_bf16(uint32_t w) { return __uint_as_float(w & 0xffff0000u); }
+// 1 / |row| of the raw q (threads 0-255) and k (256-511) tiles: row (tid % 256) / 4, the row's four
+// threads return the same value; w keeps the values read.
+__device__ __forceinline__ float row_norms(const uint8_t *qt, const uint8_t *kt, int tid, int l2norm, uint32_t (&w)[16]) {
+    load_parts(tid < 256 ? qt : kt, (tid & 255) >> 2, tid & 3, w);
+    float p0 = 0.f, p1 = 0.f;
+#pragma unroll
+    for (int c = 0; c < 16; ++c) {
+        p0 = fmaf(lo_bf16(w[c]), lo_bf16(w[c]), p0);
+        p1 = fmaf(hi_bf16(w[c]), hi_bf16(w[c]), p1);
+    }
+    return gbwd::rnorm_of(parts_total(p0, p1, tid & 31), l2norm);
+}
+__device__ __forceinline__ void put_raw16(uint8_t *tile, int i, int hf, int grp, const Raw16 &x) {
+    *reinterpret_cast<uint4 *>(tile + hf * 8192 + t64_chunk(i, 2 * grp)) = x.a;
+    *reinterpret_cast<uint4 *>(tile + hf * 8192 + t64_chunk(i, 2 * grp + 1)) = x.b;
+}
+
+// K = 64 or 128 products over T64 tiles.  A and B: descriptors of the first K = 16 step; K-major operands
+// advance 32 B a step and `*blk` (tile bytes >> 4) every 64, MN-major ones 2 KB a step.
+template <int K, bool AM, bool BM>
+__device__ __forceinline__ void mma_k(uint32_t d, uint64_t A, int ablk, uint64_t B, int bblk, uint32_t id, bool acc) {
+#pragma unroll
+    for (int k = 0; k < K / 16; ++k)
+        mma_bf16(d, A + (AM ? k * 128 : (k >> 2) * ablk + (k & 3) * 2), B + (BM ? k * 128 : (k >> 2) * bblk + (k & 3) * 2),
+                 id, (acc || k > 0) ? 1u : 0u);
+}
+
+// The chunk one wave later finds its strided token rows in L2 (one 128-byte line a thread).
+__device__ __forceinline__ void prefetch_rows(const void *t0, const void *t1, const void *t2, const void *t3,
+                                              const GdnBwdArgs &a, int ch, int tid) {
+    const int r = ch % a.NC, bh = ch / a.NC, b = bh / a.H, h = bh % a.H;
+    const int row = (tid >> 1) & 63, which = tid >> 7, t = r * kC + row;
+    if (t >= a.T) return;
+    const void *src = which == 0 ? t0 : which == 1 ? t1 : which == 2 ? t2 : t3;
+    const __nv_bfloat16 *p = static_cast<const __nv_bfloat16 *>(src) +
+                             ((static_cast<size_t>(b) * a.T + t) * a.H + h) * kD + 64 * (tid & 1);
+    asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
+}
+
+// =====================================================================================
+// gdn_bwd_local128_kernel: one CTA per (sequence, head, chunk)
+// =====================================================================================
+namespace lk {
+constexpr uint32_t OFF_Q = 0;        // qbar
+constexpr uint32_t OFF_K = 16384;    // kbar
+constexpr uint32_t OFF_SK = 32768;   // S^K_r (32 KB)
+constexpr uint32_t OFF_H = 65536;    // H_r (32 KB)
+constexpr uint32_t OFF_R = 98304;    // R, then W
+constexpr uint32_t OFF_U = 114688;   // U
+constexpr uint32_t OFF_QC = 131072;  // q_clean
+constexpr uint32_t OFF_D = 147456;   // D = scale dO
+constexpr uint32_t OFF_ED = 163840;  // diag(E) D
+constexpr uint32_t OFF_TB = 180224;  // Tt diag(beta), then dP
+constexpr uint32_t OFF_SA = 188416;  // (Qbar Kbar^T) o causal, then P, then (W Kbar^T) o causal
+constexpr uint32_t OFF_MISC = 196608;
+constexpr int F_GC = 0, F_E = 64, F_BE = 128, F_TI = 192, F_LAM = 256, F_M = 320, F_SEG = 448, F_DM = 960,
+              F_RN = 1088, F_CQ = 1216, F_RED = 1280, kReds = 4, kFloats = F_RED + kReds * 256;
+constexpr int LS = 72;               // row stride (floats) of the fp32 copy of masked Sc in U's and q_clean's place
+constexpr uint32_t M_BAR = kFloats * 4, M_TMEM = M_BAR + 80, M_ABORT = M_TMEM + 4;
+constexpr uint32_t kSmem = OFF_MISC + M_ABORT + 4 + 1024;
+static_assert(kSmem <= 232448, "exceeds the 227 KB per-CTA limit");
+enum { B1 = 0, B2, B2B, B3, B3B, B4, B5, B5B, B6, kBars };
+static_assert(8 * kBars <= 80, "barriers reach the TMEM slot");
+static_assert(OFF_QC == OFF_U + 16384 && 64 * LS * 4 <= 32768, "the fp32 staging spans U and q_clean");
+// TMEM columns: Sc, then P | dP, then dP Kbar, then W Kbar^T | KH, U, Y1, DC | z, X1, the dqbar terms | (E D) H^T
+constexpr uint32_t TM_A = 0, TM_A2 = 64, TM_B = 128, TM_C = 256, TM_D = 384;
+}  // namespace lk
+
+// Per chunk, everything that does not need dH.  Rounds (products, then the epilogue they feed):
+//   1  Sc = Qbar Kbar^T, KH = Kbar H | Z = Qbar S^K     masked Sc, cq, R = V - E KH
+//   2  U = Tb R | Z += Sc Kbar                           U, z, q_clean
+//   3  P = Qc Kbar^T, dP = D U^T | (E D) H^T, Y1 = Qc^T (E D)   P, dP; E rowsum((Qc H) o D); Y1
+//   4  dP Kbar, X1 = P^T D                               dqc, dlambda, W; X1
+//   5  Wk = W Kbar^T | W S^K, DC = W^T Qbar              masked Wk, cz; DC
+//   6  += Wk Kbar                                        dqbar, dq, the Dm increment
+__global__ void __launch_bounds__(kAll, 1) gdn_bwd_local128_kernel(const GdnBwdArgs a) {
+    using namespace lk;
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t *sm = smem_align1024(smem_raw);
+    const uint32_t sb = smem_addr(sm);
+    float *fm = reinterpret_cast<float *>(sm + OFF_MISC);
+    float *gc = fm + F_GC, *E = fm + F_E, *be = fm + F_BE, *tinv = fm + F_TI, *lam = fm + F_LAM, *M = fm + F_M;
+    float *segs = fm + F_SEG, *dMs = fm + F_DM, *rn = fm + F_RN, *cqs = fm + F_CQ, *red = fm + F_RED;
+    uint64_t *bar = reinterpret_cast<uint64_t *>(sm + OFF_MISC + M_BAR);
+    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(sm + OFF_MISC + M_TMEM);
+    volatile int *abort_flag = reinterpret_cast<volatile int *>(sm + OFF_MISC + M_ABORT);
+
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int ch = blockIdx.x, r = ch % a.NC, bh = ch / a.NC, b = bh / a.H, h = bh % a.H;
+    const int n = min(kC, a.T - r * kC);
+    const size_t t64 = static_cast<size_t>(ch) * kC * kD, sq = static_cast<size_t>(ch) * kD * kD;
+    int *status = a.status;
+
+    if (warp == kCompute / 32) {
+        // ---- the issuing warp
+        if (lane == 0) {
+            for (int i = 0; i < kBars; ++i) mbar_init(&bar[i], 1);
+            *abort_flag = 0;
+            fence_barrier_init();
+        }
+        token_scalars(a, b, h, r, lane, gc, E, be, tinv, lam);
+        __syncthreads();  // scalars, partial norms, M, TMEM
+        const uint32_t tb = *tmem_slot;
+        const uint64_t dQ = make_desc(sb + OFF_Q, 16, 1024), dQm = make_desc(sb + OFF_Q, 8192, 1024);
+        const uint64_t dK = make_desc(sb + OFF_K, 16, 1024), dKm = make_desc(sb + OFF_K, 8192, 1024);
+        const uint64_t dSKm = make_desc(sb + OFF_SK, 16384, 1024);
+        const uint64_t dH = make_desc(sb + OFF_H, 16, 1024), dHm = make_desc(sb + OFF_H, 16384, 1024);
+        const uint64_t dR = make_desc(sb + OFF_R, 16, 1024), dRm = make_desc(sb + OFF_R, 8192, 1024);
+        const uint64_t dU = make_desc(sb + OFF_U, 16, 1024);
+        const uint64_t dQC = make_desc(sb + OFF_QC, 16, 1024), dQCm = make_desc(sb + OFF_QC, 8192, 1024);
+        const uint64_t dD = make_desc(sb + OFF_D, 16, 1024), dDm = make_desc(sb + OFF_D, 8192, 1024);
+        const uint64_t dED = make_desc(sb + OFF_ED, 16, 1024), dEDm = make_desc(sb + OFF_ED, 8192, 1024);
+        const uint64_t dTB = make_desc(sb + OFF_TB, 16, 1024);
+        const uint64_t dSA = make_desc(sb + OFF_SA, 16, 1024), dSAm = make_desc(sb + OFF_SA, 8192, 1024);
+        int last = -1;  // the last committed round, for the drain after a give-up
+        auto go = [&] { return lane == 0 && !*abort_flag; };
+        named_bar(2, kAll);
+        tc_fence_after();
+        if (go()) {
+            mma_k<128, false, false>(tb + TM_A, dQ, 512, dK, 512, ID_64x64_KK, false);
+            mma_k<128, false, true>(tb + TM_B, dK, 512, dHm, 0, ID_64x128_KM, false);
+            mma_commit(&bar[B1]);
+            mma_k<128, false, true>(tb + TM_C, dQ, 512, dSKm, 0, ID_64x128_KM, false);
+            last = B1;
+        }
+        {
+            // the chunk one wave later finds its inputs in L2
+            const int nx = ch + a.wave;
+            if (lane == 0 && a.wave > 0 && nx < static_cast<int>(gridDim.x)) {
+                bulk_prefetch_l2(a.hs + static_cast<size_t>(nx) * kD * kD, kD * kD * 4);
+                bulk_prefetch_l2(a.sk + static_cast<size_t>(nx) * kD * kD, kD * kD * 4);
+                bulk_prefetch_l2(a.tt + static_cast<size_t>(nx) * kC * kC, kC * kC * 4);
+            }
+        }
+        named_bar(3, kAll);
+        tc_fence_after();
+        if (go()) {
+            mma_k<64, false, true>(tb + TM_B, dTB, 0, dRm, 0, ID_64x128_KM, false);
+            mma_commit(&bar[B2]);
+            mma_k<64, false, true>(tb + TM_C, dSA, 0, dKm, 0, ID_64x128_KM, true);
+            mma_commit(&bar[B2B]);
+            last = B2B;
+        }
+        named_bar(2, kAll);
+        tc_fence_after();
+        if (go()) {
+            mma_k<128, false, false>(tb + TM_A, dQC, 512, dK, 512, ID_64x64_KK, false);
+            mma_k<128, false, false>(tb + TM_A2, dD, 512, dU, 512, ID_64x64_KK, false);
+            mma_commit(&bar[B3]);
+            mma_k<128, false, false>(tb + TM_D, dED, 512, dH, 1024, ID_64x128_KK, false);
+            mma_k<64, true, true>(tb + TM_B, dQCm, 0, dEDm, 0, ID_128x128_MM, false);
+            mma_commit(&bar[B3B]);
+            last = B3B;
+        }
+        named_bar(3, kAll);
+        tc_fence_after();
+        if (go()) {
+            mma_k<64, false, true>(tb + TM_A, dTB, 0, dKm, 0, ID_64x128_KM, false);
+            mma_k<64, true, true>(tb + TM_C, dSAm, 0, dDm, 0, ID_64x128_MM, false);
+            mma_commit(&bar[B4]);
+            last = B4;
+        }
+        named_bar(2, kAll);
+        tc_fence_after();
+        if (go()) {
+            mma_k<128, false, false>(tb + TM_A, dR, 512, dK, 512, ID_64x64_KK, false);
+            mma_commit(&bar[B5]);
+            mma_k<128, false, true>(tb + TM_C, dR, 512, dSKm, 0, ID_64x128_KM, false);
+            mma_k<64, true, true>(tb + TM_B, dRm, 0, dQm, 0, ID_128x128_MM, false);
+            mma_commit(&bar[B5B]);
+            last = B5B;
+        }
+        named_bar(3, kAll);
+        tc_fence_after();
+        if (go()) {
+            mma_k<64, false, true>(tb + TM_C, dSA, 0, dKm, 0, ID_64x128_KM, true);
+            mma_commit(&bar[B6]);
+            last = B6;
+        }
+        if (lane == 0 && *abort_flag && last >= 0) mbar_drain(&bar[last], 0);
+        __syncthreads();
+        return;
+    }
+
+    // ---- the compute threads
+    const int qd = warp & 3, grp = warp >> 2, hf = lane >> 4, i = 16 * qd + (lane & 15);
+    const int c0 = 64 * hf + 16 * grp, s0 = 32 * hf + 8 * grp;
+    if (warp == 0) tmem_alloc(tmem_slot, 512);
+    const bool valid = i < n;
+    const size_t row = (static_cast<size_t>(b) * a.T + r * kC + (valid ? i : 0)) * a.H + h;
+    const Raw16 qr = load_raw16(a.q, row, c0, valid), kr = load_raw16(a.k, row, c0, valid);
+    const Raw16 vr = load_raw16(a.v, row, c0, valid), dr = load_raw16(a.dout, row, c0, valid);
+    if (tid < kD) {
+        M[tid] = a.mk[static_cast<size_t>(ch) * kD + tid];
+        dMs[tid] = 0.f;
+    }
+    put_raw16(sm + OFF_Q, i, hf, grp, qr);
+    put_raw16(sm + OFF_K, i, hf, grp, kr);
+    stage_square(sm + OFF_H, a.hs + sq, tid);
+    if (a.wave > 0 && ch + a.wave < static_cast<int>(gridDim.x)) prefetch_rows(a.q, a.k, a.v, a.dout, a, ch + a.wave, tid);
+    __syncthreads();
+    const uint32_t tb = *tmem_slot, tq = tb + (static_cast<uint32_t>(32 * qd) << 16);
+    // row norms, and (threads 0-255) the M . qbar terms of cq in the same interleaved parts
+    float m0 = 0.f, m1 = 0.f;
+    {
+        uint32_t w[16];
+        const float rr = row_norms(sm + OFF_Q, sm + OFF_K, tid, a.l2norm, w);
+        if ((tid & 3) == 0) rn[tid >> 2] = rr;
+        if (tid < 256) {
+#pragma unroll
+            for (int c = 0; c < 16; ++c) {
+                const float2 mm = *reinterpret_cast<const float2 *>(M + 8 * c + 2 * (tid & 3));
+                m0 = fmaf(mm.x, lo_bf16(w[c]) * rr, m0);
+                m1 = fmaf(mm.y, hi_bf16(w[c]) * rr, m1);
+            }
+        }
+    }
+    compute_sync();
+    const float rq = rn[i], rk = rn[kC + i];
+    float qb[16], x[16], cum[16];
+    float4 *fst = reinterpret_cast<float4 *>(sm + OFF_U);  // fp32 [64][128], 16-byte chunks c ^ (row & 7)
+    unpack16(qr, qb);
+    unpack16(kr, x);
+#pragma unroll
+    for (int e = 0; e < 16; ++e) {
+        qb[e] *= rq;
+        x[e] *= rk;
+    }
+    put16(sm + OFF_Q, i, hf, grp, qb);
+    put16(sm + OFF_K, i, hf, grp, x);
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+        fst[i * 32 + ((c0 / 4 + q) ^ (i & 7))] = make_float4(x[4 * q], x[4 * q + 1], x[4 * q + 2], x[4 * q + 3]);
+    {
+        float d[16];
+        unpack16(dr, d);
+#pragma unroll
+        for (int e = 0; e < 16; ++e) d[e] *= a.scale;
+        put16(sm + OFF_D, i, hf, grp, d);
+#pragma unroll
+        for (int e = 0; e < 16; ++e) d[e] *= E[i];
+        put16(sm + OFF_ED, i, hf, grp, d);
+    }
+    {
+        // Tt diag(beta): row tid / 8, columns 8 (tid % 8) .. + 7
+        float t[8];
+        ld_global8(a.tt + static_cast<size_t>(ch) * kC * kC + 8 * tid, t);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) t[e] *= be[8 * (tid & 7) + e];
+        *reinterpret_cast<uint4 *>(sm + OFF_TB + t64_chunk(tid >> 3, tid & 7)) = pack8(t);
+    }
+    stage_square(sm + OFF_SK, a.sk + sq, tid);
+    signal_issue(2);
+    // while round 1 runs: CumK_i = M + sum_{j <= i} kbar_j, a thread per column and sixteen rows
+    compute_sync();
+    {
+        const int j = tid & 127, sg = tid >> 7;
+        float *col = reinterpret_cast<float *>(fst) + (j & 3);
+        float kv[16], acc = 0.f;
+#pragma unroll
+        for (int l = 0; l < 16; ++l) kv[l] = col[(16 * sg + l) * 128 + 4 * ((j >> 2) ^ (l & 7))];
+#pragma unroll
+        for (int l = 0; l < 16; ++l) acc += kv[l];
+        segs[sg * kD + j] = acc;
+        compute_sync();
+        float c = M[j];
+        for (int s = 0; s < sg; ++s) c += segs[s * kD + j];
+#pragma unroll
+        for (int l = 0; l < 16; ++l) {
+            c += kv[l];
+            col[(16 * sg + l) * 128 + 4 * ((j >> 2) ^ (l & 7))] = c;
+        }
+    }
+    compute_sync();
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const float4 y = fst[i * 32 + ((c0 / 4 + q) ^ (i & 7))];
+        cum[4 * q] = y.x;
+        cum[4 * q + 1] = y.y;
+        cum[4 * q + 2] = y.z;
+        cum[4 * q + 3] = y.w;
+    }
+    compute_sync();
+
+    // ---- round 1: masked Sc, cq, R
+    mbar_wait(&bar[B1], 0, abort_flag, status);
+    tc_fence_after();
+    float *scf = reinterpret_cast<float *>(sm + OFF_U);  // [64][LS]
+    {
+        float s[8];
+        acc_ld8(tq + TM_A + 8 * grp, s);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) s[e] = s0 + e <= i ? s[e] : 0.f;
+        put8(sm + OFF_SA, i, hf, grp, s);
+        *reinterpret_cast<float4 *>(scf + i * LS + s0) = make_float4(s[0], s[1], s[2], s[3]);
+        *reinterpret_cast<float4 *>(scf + i * LS + s0 + 4) = make_float4(s[4], s[5], s[6], s[7]);
+        float v[16];
+        unpack16(vr, v);
+        acc_ld16(tq + TM_B + 16 * grp, x);
+        const float ei = E[i];
+#pragma unroll
+        for (int e = 0; e < 16; ++e) x[e] = fmaf(-ei, x[e], v[e]);
+        put16(sm + OFF_R, i, hf, grp, x);
+        signal_issue(3);
+        st_own16(a.r + t64, tid, x);
+    }
+    compute_sync();
+    if (tid < 256) {
+        // cq_i = CumK_i . qbar_i = M . qbar_i + sum_{j <= i} Sc_ij
+        const float *sr = scf + (tid >> 2) * LS + 2 * (tid & 3);
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+            const float2 y = *reinterpret_cast<const float2 *>(sr + 8 * c);
+            m0 += y.x;
+            m1 += y.y;
+        }
+        const float t = parts_total(m0, m1, lane);
+        if ((tid & 3) == 0) cqs[tid >> 2] = t;
+    }
+    compute_sync();
+    const float cf = a.centered ? 1.f : 0.f, ti = tinv[i];
+    const float cq = cqs[i];
+    // ---- round 2: U, z, q_clean
+    mbar_wait(&bar[B2], 0, abort_flag, status);
+    tc_fence_after();
+    acc_ld16(tq + TM_B + 16 * grp, x);
+    put16(sm + OFF_U, i, hf, grp, x);
+    st_own16(a.u + t64, tid, x);
+    mbar_wait(&bar[B2B], 0, abort_flag, status);
+    tc_fence_after();
+    float z[16];
+    acc_ld16(tq + TM_C + 16 * grp, z);
+    {
+        const float li = lam[i];
+#pragma unroll
+        for (int e = 0; e < 16; ++e) {
+            z[e] = z[e] * ti - cf * cum[e] * cq * ti * ti;
+            x[e] = qb[e] - li * z[e];
+        }
+    }
+    put16(sm + OFF_QC, i, hf, grp, x);
+    signal_issue(2);
+    {
+        // q_clean as the kv kernel's operand tile
+        uint8_t *img = reinterpret_cast<uint8_t *>(a.qc + t64) + hf * 8192;
+        *reinterpret_cast<uint4 *>(img + t64_chunk(i, 2 * grp)) = pack8(x);
+        *reinterpret_cast<uint4 *>(img + t64_chunk(i, 2 * grp + 1)) = pack8(x + 8);
+    }
+    // ---- round 3: P, dP; E rowsum((Qc H) o D); Y1
+    float gam[8];  // Gamma o causal
+    {
+        const float gi = gc[i];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) gam[e] = s0 + e <= i ? expf(gi - gc[s0 + e]) : 0.f;
+    }
+    mbar_wait(&bar[B3], 0, abort_flag, status);
+    tc_fence_after();
+    {
+        float p[8];
+        acc_ld8(tq + TM_A + 8 * grp, p);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) p[e] = s0 + e <= i ? p[e] * gam[e] : 0.f;
+        put8(sm + OFF_SA, i, hf, grp, p);
+        acc_ld8(tq + TM_A2 + 8 * grp, p);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) p[e] = s0 + e <= i ? p[e] * gam[e] : 0.f;
+        put8(sm + OFF_TB, i, hf, grp, p);
+    }
+    signal_issue(3);
+    mbar_wait(&bar[B3B], 0, abort_flag, status);
+    tc_fence_after();
+    float dqc[16];
+    acc_ld16(tq + TM_D + 16 * grp, dqc);
+    {
+        float part = 0.f;
+#pragma unroll
+        for (int e = 0; e < 16; ++e) part = fmaf(x[e], dqc[e], part);
+        row_part(red, grp, i, hf, part);
+        float y[32];
+        tmem_ld32(tq + TM_B + 32 * grp, y);
+        float *Y1 = a.y1 + sq + (32 * qd + lane) * kD + 32 * grp;
+#pragma unroll
+        for (int e = 0; e < 32; e += 8) st_global8(Y1 + e, y + e);
+    }
+    // ---- round 4: dqc, dlambda, W; X1
+    mbar_wait(&bar[B4], 0, abort_flag, status);
+    tc_fence_after();
+    acc_ld16(tq + TM_A + 16 * grp, x);
+    float mw = 0.f;
+    {
+        float part = 0.f;
+        const float li = lam[i];
+#pragma unroll
+        for (int e = 0; e < 16; ++e) {
+            dqc[e] = x[e] + dqc[e];
+            part = fmaf(z[e], dqc[e], part);
+            z[e] = -li * dqc[e] * ti;  // W = dz / t from here on
+            mw = fmaf(M[c0 + e], z[e], mw);
+        }
+        put16(sm + OFF_R, i, hf, grp, z);
+        row_part(red + 256, grp, i, hf, part);
+        acc_ld16(tq + TM_C + 16 * grp, x);
+    }
+    signal_issue(2);
+    {
+        float *X1 = a.x1 + t64 + i * kD + c0;
+        st_global8(X1, x);
+        st_global8(X1 + 8, x + 8);
+    }
+    st_own16(a.w + t64, tid, z);
+    // ---- round 5: masked W Kbar^T, cz; DC
+    mbar_wait(&bar[B5], 0, abort_flag, status);
+    tc_fence_after();
+    {
+        float s[8], part = mw;
+        acc_ld8(tq + TM_A + 8 * grp, s);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+            s[e] = s0 + e <= i ? s[e] : 0.f;
+            part += s[e];
+        }
+        put8(sm + OFF_SA, i, hf, grp, s);
+        row_part(red + 512, grp, i, hf, part);
+    }
+    signal_issue(3);
+    compute_sync();
+    const float cz = row_total(red + 512, i) / ti;
+    if (grp == 0 && hf == 0) {
+        float *vec = a.vec + static_cast<size_t>(ch) * 4 * kC;
+        vec[i] = cq;
+        vec[kC + i] = cz;
+        vec[2 * kC + i] = valid ? row_total(red, i) : 0.f;
+        if (valid && a.dlambda) a.dlambda[row] = -row_total(red + 256, i);
+    }
+    mbar_wait(&bar[B5B], 0, abort_flag, status);
+    tc_fence_after();
+    {
+        float y[32];
+        tmem_ld32(tq + TM_B + 32 * grp, y);
+        float *dC = a.dc + sq + (32 * qd + lane) * kD + 32 * grp;
+#pragma unroll
+        for (int e = 0; e < 32; e += 8) st_global8(dC + e, y + e);
+    }
+    {
+        // the Dm increment: sum_i (W_i cq_i t_i + qbar_i cz_i) / t_i^2
+        const float ct = cq / ti, t2 = ti * ti;
+#pragma unroll
+        for (int e = 0; e < 16; ++e) z[e] = (z[e] * ct + qb[e] * cz) * t2;
+        col_sums<16>(z, lane);
+        atomicAdd(&dMs[c0 + (lane & 15)], z[0]);
+    }
+    // ---- round 6: dqbar, dq
+    mbar_wait(&bar[B6], 0, abort_flag, status);
+    tc_fence_after();
+    acc_ld16(tq + TM_C + 16 * grp, x);
+    {
+        float part = 0.f;
+        const float k2 = cf * cz * ti * ti;
+#pragma unroll
+        for (int e = 0; e < 16; ++e) {
+            dqc[e] = dqc[e] + x[e] - cum[e] * k2;
+            part = fmaf(qb[e], dqc[e], part);
+        }
+        row_part(red + 768, grp, i, hf, part);
+    }
+    tc_fence_before();
+    compute_sync();
+    if (valid) {
+        const float rdot = a.l2norm ? row_total(red + 768, i) : 0.f;
+#pragma unroll
+        for (int e = 0; e < 16; ++e) x[e] = (dqc[e] - qb[e] * rdot) * rq;
+        store_row16(a.dq, row, c0, x);
+    }
+    if (tid < kD) a.dm[static_cast<size_t>(ch) * kD + tid] = -cf * dMs[tid];
+    __syncthreads();
+    if (warp == 0) {
+        tc_fence_after();
+        tmem_dealloc(tb, 512);
+    }
+}
+
+// =====================================================================================
+// gdn_bwd_kv128_kernel: one CTA per (sequence, head, chunk)
+// =====================================================================================
+namespace kk {
+constexpr uint32_t OFF_K = 0;        // kbar
+constexpr uint32_t OFF_Q = 16384;    // qbar
+constexpr uint32_t OFF_W = 32768;    // W
+constexpr uint32_t OFF_D = 49152;    // D = scale dO, then R, then dR
+constexpr uint32_t OFF_DU = 65536;   // dU
+constexpr uint32_t OFF_QC = 81920;   // q_clean, then (with U) the staging of dKK^T
+constexpr uint32_t OFF_U = 98304;    // U
+constexpr uint32_t OFF_DH = 114688;  // dH (32 KB), then DC + DC^T
+constexpr uint32_t OFF_H = 147456;   // H_r (32 KB)
+constexpr uint32_t OFF_TT = 180224;  // Tt
+constexpr uint32_t OFF_DP = 188416;  // dP, then M2
+constexpr uint32_t OFF_QK = 196608;  // (Qbar Kbar^T) o causal
+constexpr uint32_t OFF_WK = 204800;  // (W Kbar^T) o causal
+constexpr uint32_t OFF_DT = 212992;  // dTb, then dKK + dKK^T
+constexpr uint32_t OFF_MISC = 221184;
+constexpr int F_GC = 0, F_E = 64, F_BE = 128, F_TI = 192, F_PCS = 256, F_CS = 320, F_DB = 384, F_SCAL = 448,
+              F_SEG = 452, F_RN = 964, F_RED = 1092, kReds = 5, kFloats = F_RED + kReds * 256;
+constexpr uint32_t M_BAR = kFloats * 4, M_TMEM = M_BAR + 64, M_ABORT = M_TMEM + 4;
+constexpr uint32_t kSmem = OFF_MISC + M_ABORT + 4 + 1024;
+static_assert(kSmem <= 232448, "exceeds the 227 KB per-CTA limit");
+static_assert(OFF_U == OFF_QC + 16384 && 64 * 65 * 4 <= 32768, "the dKK staging spans q_clean and U");
+static_assert(M_BAR % 8 == 0, "barrier alignment");
+enum { BIN = 0, B1, B1B, B2, B2B, B3, B4, B5, kBars };
+static_assert(8 * kBars <= 64, "barriers reach the TMEM slot");
+// TMEM columns: t, then dR, then dR H^T | S, dP, then U dH^T | KK | QK, WK, then the sum of dk's other
+// products | dTb, then M2, then dA
+constexpr uint32_t TM_T = 0, TM_S = 128, TM_P = 192, TM_KK = 256, TM_ACC = 320, TM_WK = 384, TM_X = 448;
+constexpr int LS = 65;  // row stride of the dKK staging (floats)
+}  // namespace kk
+
+// Per chunk: dv, dk, dbeta, dg.  Rounds:
+//   1  t = Kbar dH, S = Qc Kbar^T, dP = D U^T | QK, WK, KK       dU, dP, sums of dP o S; masked QK, WK
+//   2  Tt^T dU, dTb = dU R^T | dP^T Qc + QK^T W + WK^T Qbar, U dH^T     dR = dv, dTb
+//   3  M2 = Tt^T dTb | dR H^T                                    M2 diag(beta)
+//   4  dA = M2 Tt^T                                              dKK + dKK^T
+//   5  += (dKK + dKK^T) Kbar + Kbar (DC + DC^T)                  dk
+__global__ void __launch_bounds__(kAll, 1) gdn_bwd_kv128_kernel(const GdnBwdArgs a) {
+    using namespace kk;
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t *sm = smem_align1024(smem_raw);
+    const uint32_t sb = smem_addr(sm);
+    float *fm = reinterpret_cast<float *>(sm + OFF_MISC);
+    float *gc = fm + F_GC, *E = fm + F_E, *be = fm + F_BE, *tinv = fm + F_TI, *pcs = fm + F_PCS, *cs = fm + F_CS;
+    float *db1 = fm + F_DB, *scal = fm + F_SCAL, *segs = fm + F_SEG, *rn = fm + F_RN, *red = fm + F_RED;
+    uint64_t *bar = reinterpret_cast<uint64_t *>(sm + OFF_MISC + M_BAR);
+    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(sm + OFF_MISC + M_TMEM);
+    volatile int *abort_flag = reinterpret_cast<volatile int *>(sm + OFF_MISC + M_ABORT);
+
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int ch = blockIdx.x, r = ch % a.NC, bh = ch / a.NC, b = bh / a.H, h = bh % a.H;
+    const int n = min(kC, a.T - r * kC);
+    const size_t t64 = static_cast<size_t>(ch) * kC * kD, sq = static_cast<size_t>(ch) * kD * kD;
+    const float *vec = a.vec + static_cast<size_t>(ch) * 4 * kC;
+    const float cf = a.centered ? 1.f : 0.f;
+    int *status = a.status;
+
+    if (warp == kCompute / 32) {
+        // ---- the issuing warp
+        if (lane == 0) {
+            for (int i = 0; i < kBars; ++i) mbar_init(&bar[i], 1);
+            *abort_flag = 0;
+            fence_barrier_init();
+            mbar_arrive_expect_tx(&bar[BIN], 16384);
+            bulk_load(sm + OFF_QC, a.qc + t64, 16384, &bar[BIN]);
+        }
+        token_scalars(a, b, h, r, lane, gc, E, be, tinv, nullptr);
+        __syncthreads();
+        const uint32_t tb = *tmem_slot;
+        const uint64_t dK = make_desc(sb + OFF_K, 16, 1024), dKm = make_desc(sb + OFF_K, 8192, 1024);
+        const uint64_t dQ = make_desc(sb + OFF_Q, 16, 1024), dQm = make_desc(sb + OFF_Q, 8192, 1024);
+        const uint64_t dW = make_desc(sb + OFF_W, 16, 1024), dWm = make_desc(sb + OFF_W, 8192, 1024);
+        const uint64_t dD = make_desc(sb + OFF_D, 16, 1024);  // D, R, dR
+        const uint64_t dDU = make_desc(sb + OFF_DU, 16, 1024), dDUm = make_desc(sb + OFF_DU, 8192, 1024);
+        const uint64_t dQC = make_desc(sb + OFF_QC, 16, 1024), dQCm = make_desc(sb + OFF_QC, 8192, 1024);
+        const uint64_t dU = make_desc(sb + OFF_U, 16, 1024);
+        const uint64_t dDH = make_desc(sb + OFF_DH, 16, 1024), dDHm = make_desc(sb + OFF_DH, 16384, 1024);
+        const uint64_t dH = make_desc(sb + OFF_H, 16, 1024);
+        const uint64_t dTT = make_desc(sb + OFF_TT, 16, 1024), dTTm = make_desc(sb + OFF_TT, 8192, 1024);
+        const uint64_t dDP = make_desc(sb + OFF_DP, 16, 1024), dDPm = make_desc(sb + OFF_DP, 8192, 1024);
+        const uint64_t dQKm = make_desc(sb + OFF_QK, 8192, 1024), dWKm = make_desc(sb + OFF_WK, 8192, 1024);
+        const uint64_t dDT = make_desc(sb + OFF_DT, 16, 1024), dDTm = make_desc(sb + OFF_DT, 8192, 1024);
+        int last = -1;
+        auto go = [&] { return lane == 0 && !*abort_flag; };
+        named_bar(2, kAll);
+        mbar_wait(&bar[BIN], 0, abort_flag, status);
+        tc_fence_after();
+        if (go()) {
+            mma_k<128, false, true>(tb + TM_T, dK, 512, dDHm, 0, ID_64x128_KM, false);
+            mma_k<128, false, false>(tb + TM_S, dQC, 512, dK, 512, ID_64x64_KK, false);
+            mma_k<128, false, false>(tb + TM_P, dD, 512, dU, 512, ID_64x64_KK, false);
+            mma_commit(&bar[B1]);
+            mma_k<128, false, false>(tb + TM_ACC, dQ, 512, dK, 512, ID_64x64_KK, false);
+            mma_k<128, false, false>(tb + TM_WK, dW, 512, dK, 512, ID_64x64_KK, false);
+            mma_k<128, false, false>(tb + TM_KK, dK, 512, dK, 512, ID_64x64_KK, false);
+            mma_commit(&bar[B1B]);
+            last = B1B;
+        }
+        {
+            const int nx = ch + a.wave;
+            if (lane == 0 && a.wave > 0 && nx < static_cast<int>(gridDim.x)) {
+                const size_t nsq = static_cast<size_t>(nx) * kD * kD, n64 = static_cast<size_t>(nx) * kC * kD;
+                bulk_prefetch_l2(a.dh + nsq, kD * kD * 4);
+                bulk_prefetch_l2(a.u + n64, kC * kD * 4);
+                bulk_prefetch_l2(a.w + n64, kC * kD * 4);
+                bulk_prefetch_l2(a.qc + n64, kC * kD * 2);
+                bulk_prefetch_l2(a.tt + static_cast<size_t>(nx) * kC * kC, kC * kC * 4);
+                bulk_prefetch_l2(a.hs + nsq, kD * kD * 4);
+                bulk_prefetch_l2(a.r + n64, kC * kD * 4);
+                bulk_prefetch_l2(a.x1 + n64, kC * kD * 4);
+                bulk_prefetch_l2(a.dc + nsq, kD * kD * 4);
+            }
+        }
+        named_bar(3, kAll);
+        tc_fence_after();
+        if (go()) {
+            mma_k<64, true, true>(tb + TM_T, dTTm, 0, dDUm, 0, ID_64x128_MM, false);
+            mma_k<128, false, false>(tb + TM_X, dDU, 512, dD, 512, ID_64x64_KK, false);
+            mma_commit(&bar[B2]);
+            last = B2;
+        }
+        named_bar(2, kAll);
+        tc_fence_after();
+        if (go()) {
+            mma_k<64, true, true>(tb + TM_ACC, dDPm, 0, dQCm, 0, ID_64x128_MM, false);
+            mma_k<64, true, true>(tb + TM_ACC, dQKm, 0, dWm, 0, ID_64x128_MM, true);
+            mma_k<64, true, true>(tb + TM_ACC, dWKm, 0, dQm, 0, ID_64x128_MM, true);
+            mma_k<128, false, false>(tb + TM_S, dU, 512, dDH, 1024, ID_64x128_KK, false);
+            mma_commit(&bar[B2B]);
+            last = B2B;
+        }
+        named_bar(3, kAll);
+        tc_fence_after();
+        if (go()) {
+            mma_k<64, true, true>(tb + TM_X, dTTm, 0, dDTm, 0, ID_64x64_MM, false);
+            mma_commit(&bar[B3]);
+            mma_k<128, false, false>(tb + TM_T, dD, 512, dH, 1024, ID_64x128_KK, false);
+            last = B3;
+        }
+        named_bar(2, kAll);
+        tc_fence_after();
+        if (go()) {
+            mma_k<64, false, false>(tb + TM_X, dDP, 0, dTT, 0, ID_64x64_KK, false);
+            mma_commit(&bar[B4]);
+            last = B4;
+        }
+        named_bar(3, kAll);
+        tc_fence_after();
+        if (go()) {
+            mma_k<64, false, true>(tb + TM_ACC, dDT, 0, dKm, 0, ID_64x128_KM, true);
+            mma_k<128, false, true>(tb + TM_ACC, dK, 512, dDHm, 0, ID_64x128_KM, true);
+            mma_commit(&bar[B5]);
+            last = B5;
+        }
+        if (lane == 0 && *abort_flag) {
+            mbar_drain(&bar[BIN], 0);
+            if (last >= 0) mbar_drain(&bar[last], 0);
+        }
+        __syncthreads();  // the row sums below are complete
+        if (warp == kCompute / 32) {
+            // dg: the in-chunk reverse cumulative sum of dgc, two tokens a lane; dbeta
+            float d[2];
+            float kd_all = 0.f;
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                const int j = 2 * lane + u;
+                const float rs = row_total(red + 256, j), kd = row_total(red + 512, j);
+                const float prs = row_total(red + 768, j), gkh = row_total(red + 1024, j);
+                kd_all += kd;
+                d[u] = j < n ? be[j] * rs - cs[j] + prs - pcs[j] + vec[2 * kC + j] - kd - gkh : 0.f;
+                if (j < n) a.dbeta[(static_cast<size_t>(b) * a.T + r * kC + j) * a.H + h] = db1[j] + rs;
+            }
+#pragma unroll
+            for (int o = 16; o >= 1; o >>= 1) kd_all += __shfl_xor_sync(0xffffffffu, kd_all, o);
+            // e^{gc_last} <dH, H> + sum_i kd_i at the last row
+#pragma unroll
+            for (int u = 0; u < 2; ++u)
+                if (2 * lane + u == n - 1) d[u] += E[kC - 1] * scal[0] + kd_all;
+            float p = d[0] + d[1];
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const float y = __shfl_down_sync(0xffffffffu, p, o);
+                if (lane + o < 32) p += y;
+            }
+            const size_t out = (static_cast<size_t>(b) * a.T + r * kC + 2 * lane) * a.H + h;
+            if (2 * lane < n) a.dg[out] = p;
+            if (2 * lane + 1 < n) a.dg[out + a.H] = p - d[0];
+        }
+        return;
+    }
+
+    // ---- the compute threads
+    const int qd = warp & 3, grp = warp >> 2, hf = lane >> 4, i = 16 * qd + (lane & 15);
+    const int c0 = 64 * hf + 16 * grp, s0 = 32 * hf + 8 * grp;
+    if (warp == 0) tmem_alloc(tmem_slot, 512);
+    const bool valid = i < n;
+    const size_t row = (static_cast<size_t>(b) * a.T + r * kC + (valid ? i : 0)) * a.H + h;
+    const Raw16 kr = load_raw16(a.k, row, c0, valid), qr = load_raw16(a.q, row, c0, valid);
+    const Raw16 dr = load_raw16(a.dout, row, c0, valid), vr = load_raw16(a.v, row, c0, valid);
+    float u[16], x[16];
+    ld_own16(a.u + t64, tid, u);
+    if (tid < kC) pcs[tid] = cs[tid] = db1[tid] = 0.f;
+    if (tid == 0) scal[0] = 0.f;
+    put_raw16(sm + OFF_Q, i, hf, grp, qr);
+    put_raw16(sm + OFF_K, i, hf, grp, kr);
+    stage_square(sm + OFF_DH, a.dh + sq, tid);
+    put16(sm + OFF_U, i, hf, grp, u);
+    ld_own16(a.w + t64, tid, x);
+    put16(sm + OFF_W, i, hf, grp, x);
+    {
+        float t[8];
+        ld_global8(a.tt + static_cast<size_t>(ch) * kC * kC + 8 * tid, t);
+        *reinterpret_cast<uint4 *>(sm + OFF_TT + t64_chunk(tid >> 3, tid & 7)) = pack8(t);
+        unpack16(dr, x);
+#pragma unroll
+        for (int e = 0; e < 16; ++e) x[e] *= a.scale;
+        put16(sm + OFF_D, i, hf, grp, x);
+    }
+    if (a.wave > 0 && ch + a.wave < static_cast<int>(gridDim.x)) prefetch_rows(a.q, a.k, a.v, a.dout, a, ch + a.wave, tid);
+    __syncthreads();
+    const uint32_t tb = *tmem_slot, tq = tb + (static_cast<uint32_t>(32 * qd) << 16);
+    {
+        uint32_t w[16];
+        const float rr = row_norms(sm + OFF_Q, sm + OFF_K, tid, a.l2norm, w);
+        if ((tid & 3) == 0) rn[tid >> 2] = rr;
+    }
+    compute_sync();
+    const float rq = rn[i], rk = rn[kC + i];
+    unpack16(qr, x);
+#pragma unroll
+    for (int e = 0; e < 16; ++e) x[e] *= rq;
+    put16(sm + OFF_Q, i, hf, grp, x);
+    unpack16(kr, x);
+#pragma unroll
+    for (int e = 0; e < 16; ++e) x[e] *= rk;
+    put16(sm + OFF_K, i, hf, grp, x);
+    signal_issue(2);
+    // while round 1 runs: H's tile and <dH, H>, R, X1
+    {
+        float part = 0.f;
+#pragma unroll
+        for (int s = 0; s < 4; s += 2) {
+            float f[2][8], g[2][8];
+#pragma unroll
+            for (int v = 0; v < 2; ++v) {
+                ld_global8(a.hs + sq + 8 * (tid + kCompute * (s + v)), f[v]);
+                ld_global8(a.dh + sq + 8 * (tid + kCompute * (s + v)), g[v]);
+            }
+#pragma unroll
+            for (int v = 0; v < 2; ++v) {
+                const int it = tid + kCompute * (s + v), rw = it >> 4, cc = it & 15;
+                *reinterpret_cast<uint4 *>(sm + OFF_H + (cc >> 3) * 16384 + t64_chunk(rw, cc & 7)) = pack8(f[v]);
+#pragma unroll
+                for (int e = 0; e < 8; ++e) part = fmaf(f[v][e], g[v][e], part);
+            }
+        }
+#pragma unroll
+        for (int o = 16; o >= 1; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
+        if (lane == 0) atomicAdd(&scal[0], part);
+    }
+    float du[16], rr[16];
+    ld_global8(a.x1 + t64 + i * kD + c0, du);
+    ld_global8(a.x1 + t64 + i * kD + c0 + 8, du + 8);
+    ld_own16(a.r + t64, tid, rr);
+    float gam[8];
+    {
+        const float gi = gc[i];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) gam[e] = s0 + e <= i ? expf(gi - gc[s0 + e]) : 0.f;
+    }
+    const float ed = expf(gc[kC - 1] - gc[i]);
+    // ---- round 1: dU, dP
+    mbar_wait(&bar[B1], 0, abort_flag, status);
+    tc_fence_after();
+    put16(sm + OFF_D, i, hf, grp, rr);  // R in D's place
+    {
+        acc_ld16(tq + TM_T + 16 * grp, x);
+        float part = 0.f;
+#pragma unroll
+        for (int e = 0; e < 16; ++e) {
+            part = fmaf(u[e], ed * x[e], part);
+            du[e] = fmaf(ed, x[e], du[e]);
+        }
+        put16(sm + OFF_DU, i, hf, grp, du);
+        row_part(red + 512, grp, i, hf, part);
+        float s[8], p[8];
+        acc_ld8(tq + TM_S + 8 * grp, s);
+        acc_ld8(tq + TM_P + 8 * grp, p);
+        part = 0.f;
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+            p[e] = s0 + e <= i ? p[e] * gam[e] : 0.f;
+            s[e] *= p[e];
+            part += s[e];
+        }
+        put8(sm + OFF_DP, i, hf, grp, p);
+        signal_issue(3);
+        row_part(red + 768, grp, i, hf, part);
+        col_sums<8>(s, lane);
+        if (!(lane & 1)) atomicAdd(&pcs[s0 + ((lane >> 1) & 7)], s[0]);
+    }
+    mbar_wait(&bar[B1B], 0, abort_flag, status);
+    tc_fence_after();
+    {
+        float s[8];
+        acc_ld8(tq + TM_ACC + 8 * grp, s);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) s[e] = s0 + e <= i ? s[e] : 0.f;
+        put8(sm + OFF_QK, i, hf, grp, s);
+        acc_ld8(tq + TM_WK + 8 * grp, s);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) s[e] = s0 + e <= i ? s[e] : 0.f;
+        put8(sm + OFF_WK, i, hf, grp, s);
+    }
+    signal_issue(2);
+    // ---- round 2: dR = dv, dTb
+    float tt[8];
+    ld_global8(a.tt + static_cast<size_t>(ch) * kC * kC + i * kC + s0, tt);
+    mbar_wait(&bar[B2], 0, abort_flag, status);
+    tc_fence_after();
+    {
+        acc_ld16(tq + TM_T + 16 * grp, x);
+        float v[16], part = 0.f;
+        unpack16(vr, v);
+        const float bi = be[i];
+#pragma unroll
+        for (int e = 0; e < 16; ++e) {
+            x[e] *= bi;
+            part = fmaf(v[e] - rr[e], x[e], part);
+        }
+        put16(sm + OFF_D, i, hf, grp, x);  // dR in R's place
+        float t[8];
+        acc_ld8(tq + TM_X + 8 * grp, t);
+        put8(sm + OFF_DT, i, hf, grp, t);
+        signal_issue(3);
+        if (valid) store_row16(a.dv, row, c0, x);
+        row_part(red + 1024, grp, i, hf, part);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) t[e] *= tt[e];
+        col_sums<8>(t, lane);
+        if (!(lane & 1)) atomicAdd(&db1[s0 + ((lane >> 1) & 7)], t[0]);
+    }
+    // the reverse sums G_i = sum_{l >= i} (W_l cq_l t_l + qbar_l cz_l) / t_l^2: sixteen rows by shuffle, the
+    // quadrants' totals through segs
+    float g[16];
+    {
+        ld_own16(a.w + t64, tid, g);
+        unpack16(qr, x);
+        const float ti = tinv[i], ct = vec[i] / ti, cz = vec[kC + i], t2 = ti * ti;
+#pragma unroll
+        for (int e = 0; e < 16; ++e) g[e] = (g[e] * ct + x[e] * rq * cz) * t2;
+#pragma unroll
+        for (int o = 1; o < 16; o <<= 1)
+#pragma unroll
+            for (int e = 0; e < 16; ++e) {
+                const float y = __shfl_down_sync(0xffffffffu, g[e], o, 16);
+                if ((lane & 15) + o < 16) g[e] += y;
+            }
+        if ((lane & 15) == 0)
+#pragma unroll
+            for (int e = 0; e < 16; ++e) segs[qd * kD + c0 + e] = g[e];
+    }
+    // ---- round 3: M2
+    mbar_wait(&bar[B2B], 0, abort_flag, status);
+    mbar_wait(&bar[B3], 0, abort_flag, status);
+    tc_fence_after();
+    {
+        float m[8];
+        acc_ld8(tq + TM_X + 8 * grp, m);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) m[e] *= be[s0 + e];
+        put8(sm + OFF_DP, i, hf, grp, m);
+    }
+    signal_issue(2);
+    // DC + DC^T in dH's place: a warp takes 32 rows and 8 columns at a time
+    {
+        const float *DC = a.dc + sq;
+#pragma unroll
+        for (int s = 0; s < 4; s += 2) {
+            float f[2][8], t[2][8];
+#pragma unroll
+            for (int v = 0; v < 2; ++v) {
+                const int it = warp + 16 * (s + v), p = 32 * (it & 3) + lane, j0 = 8 * (it >> 2);
+                ld_global8(DC + p * kD + j0, f[v]);
+#pragma unroll
+                for (int e = 0; e < 8; ++e) t[v][e] = DC[(j0 + e) * kD + p];
+            }
+#pragma unroll
+            for (int v = 0; v < 2; ++v) {
+                const int it = warp + 16 * (s + v), p = 32 * (it & 3) + lane, cc = it >> 2;
+#pragma unroll
+                for (int e = 0; e < 8; ++e) f[v][e] += t[v][e];
+                *reinterpret_cast<uint4 *>(sm + OFF_DH + (cc >> 3) * 16384 + t64_chunk(p, cc & 7)) = pack8(f[v]);
+            }
+        }
+    }
+    // ---- round 4: dKK + dKK^T
+    float *stage = reinterpret_cast<float *>(sm + OFF_QC);
+    mbar_wait(&bar[B4], 0, abort_flag, status);
+    tc_fence_after();
+    {
+        float da[8], kk2[8];
+        acc_ld8(tq + TM_X + 8 * grp, da);
+        acc_ld8(tq + TM_KK + 8 * grp, kk2);
+        float part = 0.f;
+        const float bi = be[i];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+            const int j = s0 + e;
+            const float y = j < i ? -da[e] : 0.f;
+            const float xx = y * gam[e] * kk2[e];
+            part += xx;
+            da[e] = y * bi * gam[e];  // dKK
+            kk2[e] = bi * xx;
+            stage[i * LS + j] = da[e];
+        }
+        row_part(red + 256, grp, i, hf, part);
+        col_sums<8>(kk2, lane);
+        if (!(lane & 1)) atomicAdd(&cs[s0 + ((lane >> 1) & 7)], kk2[0]);
+        tc_fence_before();
+        compute_sync();
+#pragma unroll
+        for (int e = 0; e < 8; ++e) da[e] += stage[(s0 + e) * LS + i];
+        put8(sm + OFF_DT, i, hf, grp, da);
+    }
+    signal_issue(3);
+    float dmv[16];
+    ld_global8(a.dm + static_cast<size_t>(ch) * kD + c0, dmv);
+    ld_global8(a.dm + static_cast<size_t>(ch) * kD + c0 + 8, dmv + 8);
+#pragma unroll
+    for (int e = 0; e < 16; ++e) {
+        float off = 0.f;
+        for (int s = qd + 1; s < 4; ++s) off += segs[s * kD + c0 + e];
+        dmv[e] -= cf * (g[e] + off);
+    }
+    // ---- round 5: dk
+    mbar_wait(&bar[B5], 0, abort_flag, status);
+    tc_fence_after();
+    {
+        const float ei = E[i];
+        acc_ld16(tq + TM_ACC + 16 * grp, x);
+#pragma unroll
+        for (int e = 0; e < 16; ++e) dmv[e] += x[e];
+        acc_ld16(tq + TM_S + 16 * grp, x);
+#pragma unroll
+        for (int e = 0; e < 16; ++e) dmv[e] = fmaf(ed, x[e], dmv[e]);
+        acc_ld16(tq + TM_T + 16 * grp, x);
+#pragma unroll
+        for (int e = 0; e < 16; ++e) dmv[e] = fmaf(-ei, x[e], dmv[e]);
+        unpack16(kr, x);
+        float part = 0.f;
+#pragma unroll
+        for (int e = 0; e < 16; ++e) {
+            x[e] *= rk;
+            part = fmaf(x[e], dmv[e], part);
+        }
+        row_part(red, grp, i, hf, part);
+    }
+    tc_fence_before();
+    compute_sync();
+    if (valid) {
+        const float rdot = a.l2norm ? row_total(red, i) : 0.f;
+#pragma unroll
+        for (int e = 0; e < 16; ++e) x[e] = (dmv[e] - x[e] * rdot) * rk;
+        store_row16(a.dk, row, c0, x);
+    }
+    __syncthreads();
+    if (warp == 0) {
+        tc_fence_after();
+        tmem_dealloc(tb, 512);
+    }
+}
+
+}  // namespace
+
+cudaError_t launch_gdn_local128(const gbwd::GdnBwdArgs &a, cudaStream_t s) {
+    cudaError_t e = cudaFuncSetAttribute(gdn_bwd_local128_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         static_cast<int>(lk::kSmem));
+    if (e != cudaSuccess) return e;
+    gdn_bwd_local128_kernel<<<static_cast<unsigned>(a.B * a.H * a.NC), kAll, lk::kSmem, s>>>(a);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_gdn_kv128(const gbwd::GdnBwdArgs &a, cudaStream_t s) {
+    cudaError_t e = cudaFuncSetAttribute(gdn_bwd_kv128_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         static_cast<int>(kk::kSmem));
+    if (e != cudaSuccess) return e;
+    gdn_bwd_kv128_kernel<<<static_cast<unsigned>(a.B * a.H * a.NC), kAll, kk::kSmem, s>>>(a);
+    return cudaGetLastError();
+}
+
+}  // namespace ccq

@@ -97,6 +97,8 @@ struct GdnBwdArgs {
                           // (sequence, head) runs as nsplit CTAs of D / nsplit columns
     int states_ready = 0; // tt, sk, mk, hs already hold Tt, S^K_r, M_r, H_r (from the forward)
     int *status = nullptr; // status word of the tensor-core products' bounded waits (TC kernels)
+    int wave = 0;          // chunk CTAs resident at once: each prefetches into L2 the inputs of the
+                           // chunk one wave after its own (ccq_gdn_bwd_chunk_tc.cu)
 };
 
 __device__ __forceinline__ size_t tok_row(const GdnBwdArgs &a, int b, int t, int h) {
