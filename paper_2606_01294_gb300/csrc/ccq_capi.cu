@@ -532,11 +532,9 @@ ccq_status ccq_gdn_workspace_size(int B, int T, int H, int Dk, int Dv, ccq_dtype
     return CCQ_OK;
 }
 
-// Per-chunk fp32 arrays of the CCQ-Gated-DeltaNet backward that the tensor-core forward can
-// fill (ChunkArgs::tt_out and the rest); with them the forward writes no output.
-struct GdnDumps {
-    float *tt, *sk, *mk, *hs;
-};
+// Per-chunk arrays of the CCQ-Gated-DeltaNet backward that the tensor-core forward can fill
+// (ChunkArgs::tt_out and the rest); with them the forward writes no output.
+using GdnDumps = GdnStateArrays;
 
 // The Gated DeltaNet forward behind ccq_gdn_fwd; `dry` runs every argument check and
 // returns before the first CUDA call.
@@ -588,7 +586,8 @@ static ccq_status gdn_fwd_impl(const void *q, const void *k, const void *v, cons
         a.o = static_cast<__nv_bfloat16 *>(o);
         a.ST = ST; a.CT = CT; a.mT = mT;
         if (dumps) {
-            a.tt_out = dumps->tt; a.sk_out = dumps->sk; a.mk_out = dumps->mk; a.hs_out = dumps->hs;
+            a.tt_out = dumps->tt; a.mk_out = dumps->mk; a.hs_out = dumps->hs;
+            a.hs_img = dumps->hs_img; a.sk_img = dumps->sk_img;
             a.skip_o = 1;
         }
         a.status = device_status_word();
@@ -711,7 +710,7 @@ ccq_status ccq_gdn_bwd(const void *q, const void *k, const void *v, const float 
         // Tt, S^K_r, M_r and H_r of every chunk from the tensor-core forward (no output written:
         // dq stands in for the output tensor, which the forward must be given)
         GdnDumps d;
-        gdn_bwd_state_arrays(a, &d.tt, &d.sk, &d.mk, &d.hs);
+        gdn_bwd_state_arrays(a, &d);
         const ccq_params fp = gdn_bwd_forward_params(c.p);
         const size_t off = gdn_bwd_forward_offset(B, T, H, Dk);
         st = gdn_fwd_impl(q, k, v, g, beta, lambda, in_dtype, S0, C0, m0, t0, dq, nullptr, nullptr, nullptr,

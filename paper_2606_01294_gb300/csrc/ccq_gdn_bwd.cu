@@ -68,21 +68,19 @@ cudaError_t run(gbwd::GdnBwdArgs a, cudaStream_t s) {
     constexpr bool kTc = std::is_same<Tin, __nv_bfloat16>::value;
     cudaError_t e;
     if (kTc && !(a.status = device_status_word())) return cudaErrorInvalidValue;
-    const unsigned nch = static_cast<unsigned>(a.B * a.H * a.NC), bh = static_cast<unsigned>(a.B * a.H);
-    const long long elems = (static_cast<long long>(D) * D + D) * a.B * a.H;
-    const unsigned eblocks = static_cast<unsigned>((elems + 255) / 256);
     if constexpr (kTc && D == 128) {
-        // the forward's per-chunk quantities are in the workspace (GdnBwdCall::states_ready)
-        if (!a.states_ready) return cudaErrorInvalidValue;
         int dev = 0, sms = 0;
         if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
         if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
         a.wave = sms;
         if ((e = launch_gdn_local128(a, s)) != cudaSuccess) return e;
         if ((e = launch_gdn_dstate_tc(a, a.k, s)) != cudaSuccess) return e;
-        gdn_bwd_suffix_kernel<D><<<eblocks, 256, 0, s>>>(a);
+        if ((e = launch_gdn_suffix128(a, s)) != cudaSuccess) return e;
         return launch_gdn_kv128(a, s);
     } else {
+        const unsigned nch = static_cast<unsigned>(a.B * a.H * a.NC), bh = static_cast<unsigned>(a.B * a.H);
+        const long long elems = (static_cast<long long>(D) * D + D) * a.B * a.H;
+        const unsigned eblocks = static_cast<unsigned>((elems + 255) / 256);
         if ((e = allow_smem(gdn_bwd_prep_kernel<D, Tin>, prep_smem<D>())) != cudaSuccess) return e;
         if ((e = allow_smem(gdn_bwd_local_kernel<D, Tin, kTc>, local_smem<D, kTc>())) != cudaSuccess) return e;
         if ((e = allow_smem(gdn_bwd_kv_kernel<D, Tin, kTc>, kv_smem<D, kTc>())) != cudaSuccess) return e;
@@ -99,14 +97,23 @@ cudaError_t run(gbwd::GdnBwdArgs a, cudaStream_t s) {
 
 }  // namespace
 
-void gdn_bwd_state_arrays(const GdnBwdCall &c, float **tt, float **sk, float **mk, float **hs) {
-    const size_t chunks = static_cast<size_t>(c.B) * c.H * ((c.T + 63) / 64);
-    const size_t d = static_cast<size_t>(c.D);
+// The workspace arrays of bf16 inputs with D = 128 (floats a chunk; 482 KB in all, within the size that
+// per_chunk_floats() reports).
+static void arrays128(const GdnBwdCall &c, gbwd::GdnBwdArgs &a) {
+    const size_t chunks = static_cast<size_t>(c.B) * c.H * ((c.T + 63) / 64), sq = 128 * 128, t64 = 64 * 128;
     float *p = array_base(c);
-    *tt = p;
-    *sk = p + chunks * 64 * 64;
-    *mk = *sk + chunks * d * d;
-    *hs = *mk + chunks * d;
+    auto take = [&](size_t per) { float *r = p; p += chunks * per; return r; };
+    auto take_img = [&] { return reinterpret_cast<uint8_t *>(take(sq / 2)); };
+    a.tt = take(64 * 64); a.mk = take(128); a.hs = take(sq);
+    a.hs_img = take_img(); a.sk_img = take_img(); a.dh_img = take_img(); a.dcs_img = take_img();
+    a.dc = take(sq); a.dm = take(128); a.x1 = take(t64); a.y1 = take(sq);
+    a.qc = take(t64 / 2); a.u = take(t64); a.r = take(t64); a.w = take(t64); a.vec = take(4 * 64);
+}
+
+void gdn_bwd_state_arrays(const GdnBwdCall &c, GdnStateArrays *d) {
+    gbwd::GdnBwdArgs a{};
+    arrays128(c, a);
+    *d = {a.tt, a.mk, a.hs, const_cast<uint8_t *>(a.hs_img), const_cast<uint8_t *>(a.sk_img)};
 }
 
 size_t gdn_bwd_workspace_bytes(int B, int T, int H, int D) {
@@ -118,7 +125,6 @@ cudaError_t launch_gdn_bwd(const GdnBwdCall &c, cudaStream_t s) {
     gbwd::GdnBwdArgs a{};
     a.B = c.B; a.T = c.T; a.H = c.H; a.NC = (c.T + 63) / 64;
     a.nsplit = gbwd::seq_split(c.B, c.H);
-    a.states_ready = c.states_ready;
     a.l2norm = c.l2norm; a.centered = c.centered; a.scale = c.scale;
     a.q = c.q; a.k = c.k; a.v = c.v; a.dout = c.dout;
     a.g = c.g; a.beta = c.beta; a.lambda = c.lambda;
@@ -127,18 +133,21 @@ cudaError_t launch_gdn_bwd(const GdnBwdCall &c, cudaStream_t s) {
     a.dq = c.dq; a.dk = c.dk; a.dv = c.dv;
     a.dg = c.dg; a.dbeta = c.dbeta; a.dlambda = c.dlambda;
     a.dS0 = c.dS0; a.dC0 = c.dC0; a.dm0 = c.dm0;
+    if (c.bf16 && c.D == 128) {
+        // the forward's per-chunk quantities are in these arrays
+        if (!c.states_ready) return cudaErrorInvalidValue;
+        arrays128(c, a);
+        return run<128, __nv_bfloat16>(a, s);
+    }
     const size_t chunks = static_cast<size_t>(c.B) * c.H * a.NC;
     const size_t d = static_cast<size_t>(c.D);
-    float *p = array_base(c);
+    float *p = static_cast<float *>(c.workspace);
     auto take = [&](size_t per) { float *r = p; p += chunks * per; return r; };
     a.tt = take(64 * 64); a.sk = take(d * d); a.mk = take(d); a.hs = take(d * d); a.dh = take(d * d);
     a.dc = take(d * d); a.dm = take(d); a.x1 = take(64 * d); a.y1 = take(d * d);
-    // the bf16 kernels for D = 128 form qbar again from q: their arrays need no room for it, which
-    // leaves room for array_base()'s alignment
-    a.qb = c.bf16 && c.D == 128 ? nullptr : take(64 * d);
-    a.qc = take(64 * d); a.u = take(64 * d); a.r = take(64 * d); a.w = take(64 * d);
+    a.qb = take(64 * d); a.qc = take(64 * d); a.u = take(64 * d); a.r = take(64 * d); a.w = take(64 * d);
     a.vec = take(4 * 64);
-    if (c.D == 128) return c.bf16 ? run<128, __nv_bfloat16>(a, s) : run<128, float>(a, s);
+    if (c.D == 128) return run<128, float>(a, s);
     if (c.D == 64) return c.bf16 ? run<64, __nv_bfloat16>(a, s) : run<64, float>(a, s);
     return cudaErrorInvalidValue;
 }

@@ -27,19 +27,25 @@ struct GdnBwdCall {
     float *dg, *dbeta, *dlambda, *dS0, *dC0, *dm0;
     void *workspace;
     // 1: the forward's per-chunk quantities (Tt, S^K_r, M_r, H_r) are already in the workspace
-    // arrays that gdn_bwd_state_arrays() names (written by the tensor-core forward); the three
-    // launches that would compute them are skipped.
+    // arrays that gdn_bwd_state_arrays() names (written by the tensor-core forward), as bf16 inputs
+    // with D = 128 need; other inputs compute them in three launches of their own.
     int states_ready = 0;
 };
 size_t gdn_bwd_workspace_bytes(int B, int T, int H, int D);
-// The workspace arrays of the forward's per-chunk quantities (layout: ChunkArgs::tt_out etc.).
-void gdn_bwd_state_arrays(const GdnBwdCall &c, float **tt, float **sk, float **mk, float **hs);
+// The workspace arrays of the forward's per-chunk quantities (bf16 inputs with D = 128; layout:
+// ChunkArgs::tt_out etc.).
+struct GdnStateArrays {
+    float *tt, *mk, *hs;
+    uint8_t *hs_img, *sk_img;
+};
+void gdn_bwd_state_arrays(const GdnBwdCall &c, GdnStateArrays *d);
 cudaError_t launch_gdn_bwd(const GdnBwdCall &c, cudaStream_t s);
 // The reverse state pass on tensor cores (ccq_gdn_bwd_state_tc.cu): Dk = Dv = 128, bf16 keys k.
 cudaError_t launch_gdn_dstate_tc(const gbwd::GdnBwdArgs &a, const void *k, cudaStream_t s);
 // The per-chunk kernels for Dk = Dv = 128 and bf16 inputs (ccq_gdn_bwd_chunk_tc.cu); the workspace arrays
 // are 32-byte aligned.
 cudaError_t launch_gdn_local128(const gbwd::GdnBwdArgs &a, cudaStream_t s);
+cudaError_t launch_gdn_suffix128(const gbwd::GdnBwdArgs &a, cudaStream_t s);
 cudaError_t launch_gdn_kv128(const gbwd::GdnBwdArgs &a, cudaStream_t s);
 // A 2-D tensor map over an fp32 [rows][cols] array with (box_cols x box_rows) boxes, 128-byte
 // swizzled (box_cols * 4 = 128).

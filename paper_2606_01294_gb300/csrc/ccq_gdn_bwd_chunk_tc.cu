@@ -144,18 +144,6 @@ __device__ __forceinline__ void ld_own16(const float *tile, int tid, float (&f)[
     ld_global8(tile + 8 * (kCompute + tid), f + 8);
 }
 
-// An fp32 [128][128] array as a bf16 operand tile (two T64 tiles of 128 rows, 16 KB apart).
-__device__ __forceinline__ void stage_square(uint8_t *tile, const float *src, int tid) {
-    float f[4][8];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) ld_global8(src + 8 * (tid + kCompute * u), f[u]);
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-        const int it = tid + kCompute * u, row = it >> 4, ch = it & 15;
-        *reinterpret_cast<uint4 *>(tile + (ch >> 3) * 16384 + t64_chunk(row, ch & 7)) = pack8(f[u]);
-    }
-}
-
 // Sums over the sixteen rows of a half-warp of N columns: leaves in v[0] the sum of column lane & 15 (N = 16)
 // or (lane >> 1) & 7 (N = 8).
 template <int N>
@@ -304,7 +292,7 @@ constexpr int LS = 72;               // row stride (floats) of the fp32 copy of 
 constexpr uint32_t M_BAR = kFloats * 4, M_TMEM = M_BAR + 80, M_ABORT = M_TMEM + 4;
 constexpr uint32_t kSmem = OFF_MISC + M_ABORT + 4 + 1024;
 static_assert(kSmem <= 232448, "exceeds the 227 KB per-CTA limit");
-enum { B1 = 0, B2, B2B, B3, B3B, B4, B5, B5B, B6, kBars };
+enum { BIN = 0, B1, B2, B2B, B3, B3B, B4, B5, B5B, B6, kBars };
 static_assert(8 * kBars <= 80, "barriers reach the TMEM slot");
 static_assert(OFF_QC == OFF_U + 16384 && 64 * LS * 4 <= 32768, "the fp32 staging spans U and q_clean");
 // TMEM columns: Sc, then P | dP, then dP Kbar, then W Kbar^T | KH, U, Y1, DC | z, X1, the dqbar terms | (E D) H^T
@@ -342,6 +330,9 @@ __global__ void __launch_bounds__(kAll, 1) gdn_bwd_local128_kernel(const GdnBwdA
             for (int i = 0; i < kBars; ++i) mbar_init(&bar[i], 1);
             *abort_flag = 0;
             fence_barrier_init();
+            mbar_arrive_expect_tx(&bar[BIN], 65536);
+            bulk_load(sm + OFF_H, a.hs_img + static_cast<size_t>(ch) * 32768, 32768, &bar[BIN]);
+            bulk_load(sm + OFF_SK, a.sk_img + static_cast<size_t>(ch) * 32768, 32768, &bar[BIN]);
         }
         token_scalars(a, b, h, r, lane, gc, E, be, tinv, lam);
         __syncthreads();  // scalars, partial norms, M, TMEM
@@ -360,6 +351,7 @@ __global__ void __launch_bounds__(kAll, 1) gdn_bwd_local128_kernel(const GdnBwdA
         int last = -1;  // the last committed round, for the drain after a give-up
         auto go = [&] { return lane == 0 && !*abort_flag; };
         named_bar(2, kAll);
+        mbar_wait(&bar[BIN], 0, abort_flag, status);
         tc_fence_after();
         if (go()) {
             mma_k<128, false, false>(tb + TM_A, dQ, 512, dK, 512, ID_64x64_KK, false);
@@ -372,8 +364,8 @@ __global__ void __launch_bounds__(kAll, 1) gdn_bwd_local128_kernel(const GdnBwdA
             // the chunk one wave later finds its inputs in L2
             const int nx = ch + a.wave;
             if (lane == 0 && a.wave > 0 && nx < static_cast<int>(gridDim.x)) {
-                bulk_prefetch_l2(a.hs + static_cast<size_t>(nx) * kD * kD, kD * kD * 4);
-                bulk_prefetch_l2(a.sk + static_cast<size_t>(nx) * kD * kD, kD * kD * 4);
+                bulk_prefetch_l2(a.hs_img + static_cast<size_t>(nx) * 32768, 32768);
+                bulk_prefetch_l2(a.sk_img + static_cast<size_t>(nx) * 32768, 32768);
                 bulk_prefetch_l2(a.tt + static_cast<size_t>(nx) * kC * kC, kC * kC * 4);
             }
         }
@@ -422,7 +414,10 @@ __global__ void __launch_bounds__(kAll, 1) gdn_bwd_local128_kernel(const GdnBwdA
             mma_commit(&bar[B6]);
             last = B6;
         }
-        if (lane == 0 && *abort_flag && last >= 0) mbar_drain(&bar[last], 0);
+        if (lane == 0 && *abort_flag) {
+            mbar_drain(&bar[BIN], 0);
+            if (last >= 0) mbar_drain(&bar[last], 0);
+        }
         __syncthreads();
         return;
     }
@@ -441,7 +436,6 @@ __global__ void __launch_bounds__(kAll, 1) gdn_bwd_local128_kernel(const GdnBwdA
     }
     put_raw16(sm + OFF_Q, i, hf, grp, qr);
     put_raw16(sm + OFF_K, i, hf, grp, kr);
-    stage_square(sm + OFF_H, a.hs + sq, tid);
     if (a.wave > 0 && ch + a.wave < static_cast<int>(gridDim.x)) prefetch_rows(a.q, a.k, a.v, a.dout, a, ch + a.wave, tid);
     __syncthreads();
     const uint32_t tb = *tmem_slot, tq = tb + (static_cast<uint32_t>(32 * qd) << 16);
@@ -494,7 +488,6 @@ __global__ void __launch_bounds__(kAll, 1) gdn_bwd_local128_kernel(const GdnBwdA
         for (int e = 0; e < 8; ++e) t[e] *= be[8 * (tid & 7) + e];
         *reinterpret_cast<uint4 *>(sm + OFF_TB + t64_chunk(tid >> 3, tid & 7)) = pack8(t);
     }
-    stage_square(sm + OFF_SK, a.sk + sq, tid);
     signal_issue(2);
     // while round 1 runs: CumK_i = M + sum_{j <= i} kbar_j, a thread per column and sixteen rows
     compute_sync();
@@ -587,7 +580,7 @@ __global__ void __launch_bounds__(kAll, 1) gdn_bwd_local128_kernel(const GdnBwdA
     signal_issue(2);
     {
         // q_clean as the kv kernel's operand tile
-        uint8_t *img = reinterpret_cast<uint8_t *>(a.qc + t64) + hf * 8192;
+        uint8_t *img = reinterpret_cast<uint8_t *>(a.qc + t64 / 2) + hf * 8192;
         *reinterpret_cast<uint4 *>(img + t64_chunk(i, 2 * grp)) = pack8(x);
         *reinterpret_cast<uint4 *>(img + t64_chunk(i, 2 * grp + 1)) = pack8(x + 8);
     }
@@ -735,7 +728,7 @@ constexpr uint32_t OFF_D = 49152;    // D = scale dO, then R, then dR
 constexpr uint32_t OFF_DU = 65536;   // dU
 constexpr uint32_t OFF_QC = 81920;   // q_clean, then (with U) the staging of dKK^T
 constexpr uint32_t OFF_U = 98304;    // U
-constexpr uint32_t OFF_DH = 114688;  // dH (32 KB), then DC + DC^T
+constexpr uint32_t OFF_DH = 114688;  // dH (32 KB), then DC_{r+1} + DC_{r+1}^T
 constexpr uint32_t OFF_H = 147456;   // H_r (32 KB)
 constexpr uint32_t OFF_TT = 180224;  // Tt
 constexpr uint32_t OFF_DP = 188416;  // dP, then M2
@@ -743,15 +736,15 @@ constexpr uint32_t OFF_QK = 196608;  // (Qbar Kbar^T) o causal
 constexpr uint32_t OFF_WK = 204800;  // (W Kbar^T) o causal
 constexpr uint32_t OFF_DT = 212992;  // dTb, then dKK + dKK^T
 constexpr uint32_t OFF_MISC = 221184;
-constexpr int F_GC = 0, F_E = 64, F_BE = 128, F_TI = 192, F_PCS = 256, F_CS = 320, F_DB = 384, F_SCAL = 448,
-              F_SEG = 452, F_RN = 964, F_RED = 1092, kReds = 5, kFloats = F_RED + kReds * 256;
-constexpr uint32_t M_BAR = kFloats * 4, M_TMEM = M_BAR + 64, M_ABORT = M_TMEM + 4;
+constexpr int F_GC = 0, F_E = 64, F_BE = 128, F_TI = 192, F_PCS = 256, F_CS = 320, F_DB = 384, F_SEG = 448,
+              F_RN = 960, F_RED = 1088, kReds = 5, kFloats = F_RED + kReds * 256;
+constexpr uint32_t M_BAR = kFloats * 4, M_TMEM = M_BAR + 80, M_ABORT = M_TMEM + 4;
 constexpr uint32_t kSmem = OFF_MISC + M_ABORT + 4 + 1024;
 static_assert(kSmem <= 232448, "exceeds the 227 KB per-CTA limit");
 static_assert(OFF_U == OFF_QC + 16384 && 64 * 65 * 4 <= 32768, "the dKK staging spans q_clean and U");
 static_assert(M_BAR % 8 == 0, "barrier alignment");
-enum { BIN = 0, B1, B1B, B2, B2B, B3, B4, B5, kBars };
-static_assert(8 * kBars <= 64, "barriers reach the TMEM slot");
+enum { BIN = 0, BDC, B1, B1B, B2, B2B, B3, B4, B5, kBars };
+static_assert(8 * kBars <= 80, "barriers reach the TMEM slot");
 // TMEM columns: t, then dR, then dR H^T | S, dP, then U dH^T | KK | QK, WK, then the sum of dk's other
 // products | dTb, then M2, then dA
 constexpr uint32_t TM_T = 0, TM_S = 128, TM_P = 192, TM_KK = 256, TM_ACC = 320, TM_WK = 384, TM_X = 448;
@@ -771,7 +764,7 @@ __global__ void __launch_bounds__(kAll, 1) gdn_bwd_kv128_kernel(const GdnBwdArgs
     const uint32_t sb = smem_addr(sm);
     float *fm = reinterpret_cast<float *>(sm + OFF_MISC);
     float *gc = fm + F_GC, *E = fm + F_E, *be = fm + F_BE, *tinv = fm + F_TI, *pcs = fm + F_PCS, *cs = fm + F_CS;
-    float *db1 = fm + F_DB, *scal = fm + F_SCAL, *segs = fm + F_SEG, *rn = fm + F_RN, *red = fm + F_RED;
+    float *db1 = fm + F_DB, *segs = fm + F_SEG, *rn = fm + F_RN, *red = fm + F_RED;
     uint64_t *bar = reinterpret_cast<uint64_t *>(sm + OFF_MISC + M_BAR);
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(sm + OFF_MISC + M_TMEM);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(sm + OFF_MISC + M_ABORT);
@@ -779,7 +772,7 @@ __global__ void __launch_bounds__(kAll, 1) gdn_bwd_kv128_kernel(const GdnBwdArgs
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int ch = blockIdx.x, r = ch % a.NC, bh = ch / a.NC, b = bh / a.H, h = bh % a.H;
     const int n = min(kC, a.T - r * kC);
-    const size_t t64 = static_cast<size_t>(ch) * kC * kD, sq = static_cast<size_t>(ch) * kD * kD;
+    const size_t t64 = static_cast<size_t>(ch) * kC * kD;
     const float *vec = a.vec + static_cast<size_t>(ch) * 4 * kC;
     const float cf = a.centered ? 1.f : 0.f;
     int *status = a.status;
@@ -790,8 +783,11 @@ __global__ void __launch_bounds__(kAll, 1) gdn_bwd_kv128_kernel(const GdnBwdArgs
             for (int i = 0; i < kBars; ++i) mbar_init(&bar[i], 1);
             *abort_flag = 0;
             fence_barrier_init();
-            mbar_arrive_expect_tx(&bar[BIN], 16384);
-            bulk_load(sm + OFF_QC, a.qc + t64, 16384, &bar[BIN]);
+            const size_t img = static_cast<size_t>(ch) * 32768;
+            mbar_arrive_expect_tx(&bar[BIN], 16384 + 65536);
+            bulk_load(sm + OFF_DH, a.dh_img + img, 32768, &bar[BIN]);
+            bulk_load(sm + OFF_QC, a.qc + t64 / 2, 16384, &bar[BIN]);
+            bulk_load(sm + OFF_H, a.hs_img + img, 32768, &bar[BIN]);
         }
         token_scalars(a, b, h, r, lane, gc, E, be, tinv, nullptr);
         __syncthreads();
@@ -828,16 +824,16 @@ __global__ void __launch_bounds__(kAll, 1) gdn_bwd_kv128_kernel(const GdnBwdArgs
         {
             const int nx = ch + a.wave;
             if (lane == 0 && a.wave > 0 && nx < static_cast<int>(gridDim.x)) {
-                const size_t nsq = static_cast<size_t>(nx) * kD * kD, n64 = static_cast<size_t>(nx) * kC * kD;
-                bulk_prefetch_l2(a.dh + nsq, kD * kD * 4);
+                const size_t nimg = static_cast<size_t>(nx) * 32768, n64 = static_cast<size_t>(nx) * kC * kD;
+                bulk_prefetch_l2(a.dh_img + nimg, 32768);
                 bulk_prefetch_l2(a.u + n64, kC * kD * 4);
                 bulk_prefetch_l2(a.w + n64, kC * kD * 4);
-                bulk_prefetch_l2(a.qc + n64, kC * kD * 2);
+                bulk_prefetch_l2(a.qc + n64 / 2, kC * kD * 2);
                 bulk_prefetch_l2(a.tt + static_cast<size_t>(nx) * kC * kC, kC * kC * 4);
-                bulk_prefetch_l2(a.hs + nsq, kD * kD * 4);
+                bulk_prefetch_l2(a.hs_img + nimg, 32768);
                 bulk_prefetch_l2(a.r + n64, kC * kD * 4);
                 bulk_prefetch_l2(a.x1 + n64, kC * kD * 4);
-                bulk_prefetch_l2(a.dc + nsq, kD * kD * 4);
+                bulk_prefetch_l2(a.dcs_img + nimg, 32768);
             }
         }
         named_bar(3, kAll);
@@ -866,6 +862,13 @@ __global__ void __launch_bounds__(kAll, 1) gdn_bwd_kv128_kernel(const GdnBwdArgs
             mma_k<128, false, false>(tb + TM_T, dD, 512, dH, 1024, ID_64x128_KK, false);
             last = B3;
         }
+        // dH's last reader is done: DC + DC^T into its place
+        mbar_wait(&bar[B2B], 0, abort_flag, status);
+        const bool dcs = go();
+        if (dcs) {
+            mbar_arrive_expect_tx(&bar[BDC], 32768);
+            bulk_load(sm + OFF_DH, a.dcs_img + static_cast<size_t>(ch) * 32768, 32768, &bar[BDC]);
+        }
         named_bar(2, kAll);
         tc_fence_after();
         if (go()) {
@@ -874,6 +877,7 @@ __global__ void __launch_bounds__(kAll, 1) gdn_bwd_kv128_kernel(const GdnBwdArgs
             last = B4;
         }
         named_bar(3, kAll);
+        mbar_wait(&bar[BDC], 0, abort_flag, status);
         tc_fence_after();
         if (go()) {
             mma_k<64, false, true>(tb + TM_ACC, dDT, 0, dKm, 0, ID_64x128_KM, true);
@@ -883,6 +887,7 @@ __global__ void __launch_bounds__(kAll, 1) gdn_bwd_kv128_kernel(const GdnBwdArgs
         }
         if (lane == 0 && *abort_flag) {
             mbar_drain(&bar[BIN], 0);
+            if (dcs) mbar_drain(&bar[BDC], 0);
             if (last >= 0) mbar_drain(&bar[last], 0);
         }
         __syncthreads();  // the row sums below are complete
@@ -904,7 +909,7 @@ __global__ void __launch_bounds__(kAll, 1) gdn_bwd_kv128_kernel(const GdnBwdArgs
             // e^{gc_last} <dH, H> + sum_i kd_i at the last row
 #pragma unroll
             for (int u = 0; u < 2; ++u)
-                if (2 * lane + u == n - 1) d[u] += E[kC - 1] * scal[0] + kd_all;
+                if (2 * lane + u == n - 1) d[u] += E[kC - 1] * (vec[3 * kC] + vec[3 * kC + 1]) + kd_all;
             float p = d[0] + d[1];
 #pragma unroll
             for (int o = 1; o < 32; o <<= 1) {
@@ -929,10 +934,8 @@ __global__ void __launch_bounds__(kAll, 1) gdn_bwd_kv128_kernel(const GdnBwdArgs
     float u[16], x[16];
     ld_own16(a.u + t64, tid, u);
     if (tid < kC) pcs[tid] = cs[tid] = db1[tid] = 0.f;
-    if (tid == 0) scal[0] = 0.f;
     put_raw16(sm + OFF_Q, i, hf, grp, qr);
     put_raw16(sm + OFF_K, i, hf, grp, kr);
-    stage_square(sm + OFF_DH, a.dh + sq, tid);
     put16(sm + OFF_U, i, hf, grp, u);
     ld_own16(a.w + t64, tid, x);
     put16(sm + OFF_W, i, hf, grp, x);
@@ -964,29 +967,7 @@ __global__ void __launch_bounds__(kAll, 1) gdn_bwd_kv128_kernel(const GdnBwdArgs
     for (int e = 0; e < 16; ++e) x[e] *= rk;
     put16(sm + OFF_K, i, hf, grp, x);
     signal_issue(2);
-    // while round 1 runs: H's tile and <dH, H>, R, X1
-    {
-        float part = 0.f;
-#pragma unroll
-        for (int s = 0; s < 4; s += 2) {
-            float f[2][8], g[2][8];
-#pragma unroll
-            for (int v = 0; v < 2; ++v) {
-                ld_global8(a.hs + sq + 8 * (tid + kCompute * (s + v)), f[v]);
-                ld_global8(a.dh + sq + 8 * (tid + kCompute * (s + v)), g[v]);
-            }
-#pragma unroll
-            for (int v = 0; v < 2; ++v) {
-                const int it = tid + kCompute * (s + v), rw = it >> 4, cc = it & 15;
-                *reinterpret_cast<uint4 *>(sm + OFF_H + (cc >> 3) * 16384 + t64_chunk(rw, cc & 7)) = pack8(f[v]);
-#pragma unroll
-                for (int e = 0; e < 8; ++e) part = fmaf(f[v][e], g[v][e], part);
-            }
-        }
-#pragma unroll
-        for (int o = 16; o >= 1; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
-        if (lane == 0) atomicAdd(&scal[0], part);
-    }
+    // while round 1 runs: R, X1
     float du[16], rr[16];
     ld_global8(a.x1 + t64 + i * kD + c0, du);
     ld_global8(a.x1 + t64 + i * kD + c0 + 8, du + 8);
@@ -1101,28 +1082,6 @@ __global__ void __launch_bounds__(kAll, 1) gdn_bwd_kv128_kernel(const GdnBwdArgs
         put8(sm + OFF_DP, i, hf, grp, m);
     }
     signal_issue(2);
-    // DC + DC^T in dH's place: a warp takes 32 rows and 8 columns at a time
-    {
-        const float *DC = a.dc + sq;
-#pragma unroll
-        for (int s = 0; s < 4; s += 2) {
-            float f[2][8], t[2][8];
-#pragma unroll
-            for (int v = 0; v < 2; ++v) {
-                const int it = warp + 16 * (s + v), p = 32 * (it & 3) + lane, j0 = 8 * (it >> 2);
-                ld_global8(DC + p * kD + j0, f[v]);
-#pragma unroll
-                for (int e = 0; e < 8; ++e) t[v][e] = DC[(j0 + e) * kD + p];
-            }
-#pragma unroll
-            for (int v = 0; v < 2; ++v) {
-                const int it = warp + 16 * (s + v), p = 32 * (it & 3) + lane, cc = it >> 2;
-#pragma unroll
-                for (int e = 0; e < 8; ++e) f[v][e] += t[v][e];
-                *reinterpret_cast<uint4 *>(sm + OFF_DH + (cc >> 3) * 16384 + t64_chunk(p, cc & 7)) = pack8(f[v]);
-            }
-        }
-    }
     // ---- round 4: dKK + dKK^T
     float *stage = reinterpret_cast<float *>(sm + OFF_QC);
     mbar_wait(&bar[B4], 0, abort_flag, status);
@@ -1200,6 +1159,100 @@ __global__ void __launch_bounds__(kAll, 1) gdn_bwd_kv128_kernel(const GdnBwdArgs
     }
 }
 
+// =====================================================================================
+// gdn_bwd_suffix128_kernel: exclusive suffix over the chunks of a sequence and head of the increments of
+// DC and Dm
+// =====================================================================================
+// acc = dC_T + sum_{s > r} dc[s] per element; DC_{r+1} + DC_{r+1}^T goes out as the kv kernel's bf16
+// operand tile (half the bytes of the fp32 array, and no transposed reads there), the full sum is dC0.  A
+// CTA walks the chunks with one pair of 32 x 32 blocks (bi, bj), (bj, bi) in registers (four elements of
+// each a thread), the partner block through shared memory; loads run four chunks ahead.  HBM-bound: 96 KB a
+// chunk.  The last CTA of a sequence and head does Dm.
+constexpr int kSufPairs = 10, kSufAhead = 4;
+__global__ void __launch_bounds__(256) gdn_bwd_suffix128_kernel(const GdnBwdArgs a) {
+    __shared__ float tile[2][2][32][33];
+    const int bh = blockIdx.x / (kSufPairs + 1), pr = blockIdx.x % (kSufPairs + 1), tid = threadIdx.x, NC = a.NC;
+    const size_t ch0 = static_cast<size_t>(bh) * NC;
+    if (pr == kSufPairs) {
+        if (tid >= kD) return;
+        float acc = a.dmT ? a.dmT[static_cast<size_t>(bh) * kD + tid] : 0.f;
+        for (int r0 = NC - 1; r0 >= 0; r0 -= 8) {
+            float x[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) x[u] = r0 - u >= 0 ? a.dm[(ch0 + r0 - u) * kD + tid] : 0.f;
+#pragma unroll
+            for (int u = 0; u < 8; ++u)
+                if (r0 - u >= 0) {
+                    a.dm[(ch0 + r0 - u) * kD + tid] = acc;
+                    acc += x[u];
+                }
+        }
+        if (a.dm0) a.dm0[static_cast<size_t>(bh) * kD + tid] = acc;
+        return;
+    }
+    // pair pr of blocks bi <= bj: (0,0) (0,1) (0,2) (0,3) (1,1) (1,2) (1,3) (2,2) (2,3) (3,3)
+    const int bi = pr < 4 ? 0 : pr < 7 ? 1 : pr < 9 ? 2 : 3;
+    const int bj = pr < 4 ? pr : pr < 7 ? pr - 3 : pr < 9 ? pr - 5 : 3;
+    const int y = tid >> 3, x4 = 4 * (tid & 7);
+    const size_t eA = static_cast<size_t>(32 * bi + y) * kD + 32 * bj + x4;  // block (bi, bj): row y, columns x4 ..
+    const size_t eB = static_cast<size_t>(32 * bj + y) * kD + 32 * bi + x4;  // block (bj, bi)
+    const size_t st = static_cast<size_t>(bh) * kD * kD;
+    float A[4] = {0.f, 0.f, 0.f, 0.f}, Bv[4] = {0.f, 0.f, 0.f, 0.f};
+    auto ld4 = [](const float *p, float (&v)[4]) {
+        const float4 f = *reinterpret_cast<const float4 *>(p);
+        v[0] = f.x; v[1] = f.y; v[2] = f.z; v[3] = f.w;
+    };
+    if (a.dCT) {
+        ld4(a.dCT + st + eA, A);
+        ld4(a.dCT + st + eB, Bv);
+    }
+    float qa[kSufAhead][4], qb[kSufAhead][4];
+    auto fetch = [&](int u, int r) {
+        if (r < 0) return;
+        ld4(a.dc + (ch0 + r) * kD * kD + eA, qa[u]);
+        ld4(a.dc + (ch0 + r) * kD * kD + eB, qb[u]);
+    };
+#pragma unroll
+    for (int u = 0; u < kSufAhead; ++u) fetch(u, NC - 1 - u);
+    auto out4 = [&](int r, int row, int col, const float (&v)[4]) {
+        uint8_t *img = a.dcs_img + (ch0 + r) * 32768 + (col >> 6) * 16384;
+        *reinterpret_cast<uint2 *>(img + t64_offset(row, col & 63)) = make_uint2(pack_bf16(v[0], v[1]), pack_bf16(v[2], v[3]));
+    };
+    for (int rb = NC - 1; rb >= 0; rb -= kSufAhead) {
+#pragma unroll
+        for (int u = 0; u < kSufAhead; ++u) {
+            const int r = rb - u;
+            if (r < 0) break;
+            float (*tA)[33] = tile[u & 1][0], (*tB)[33] = tile[u & 1][1];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                tA[y][x4 + e] = A[e];
+                tB[y][x4 + e] = Bv[e];
+            }
+            __syncthreads();
+            float v[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) v[e] = A[e] + tB[x4 + e][y];
+            out4(r, 32 * bi + y, 32 * bj + x4, v);
+            if (bi != bj) {
+#pragma unroll
+                for (int e = 0; e < 4; ++e) v[e] = Bv[e] + tA[x4 + e][y];
+                out4(r, 32 * bj + y, 32 * bi + x4, v);
+            }
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                A[e] += qa[u][e];
+                Bv[e] += qb[u][e];
+            }
+            fetch(u, r - kSufAhead);
+        }
+    }
+    if (a.dC0) {
+        *reinterpret_cast<float4 *>(a.dC0 + st + eA) = make_float4(A[0], A[1], A[2], A[3]);
+        if (bi != bj) *reinterpret_cast<float4 *>(a.dC0 + st + eB) = make_float4(Bv[0], Bv[1], Bv[2], Bv[3]);
+    }
+}
+
 }  // namespace
 
 cudaError_t launch_gdn_local128(const gbwd::GdnBwdArgs &a, cudaStream_t s) {
@@ -1207,6 +1260,11 @@ cudaError_t launch_gdn_local128(const gbwd::GdnBwdArgs &a, cudaStream_t s) {
                                          static_cast<int>(lk::kSmem));
     if (e != cudaSuccess) return e;
     gdn_bwd_local128_kernel<<<static_cast<unsigned>(a.B * a.H * a.NC), kAll, lk::kSmem, s>>>(a);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_gdn_suffix128(const gbwd::GdnBwdArgs &a, cudaStream_t s) {
+    gdn_bwd_suffix128_kernel<<<static_cast<unsigned>(a.B * a.H * (kSufPairs + 1)), 256, 0, s>>>(a);
     return cudaGetLastError();
 }
 

@@ -95,7 +95,11 @@ struct GdnBwdArgs {
     int nsplit = 1;       // value-column blocks of the sequential passes (a divisor of D): the
                           // delta rule acts on the columns of H independently, so each
                           // (sequence, head) runs as nsplit CTAs of D / nsplit columns
-    int states_ready = 0; // tt, sk, mk, hs already hold Tt, S^K_r, M_r, H_r (from the forward)
+    // bf16 inputs with D = 128 (ccq_gdn_bwd_chunk_tc.cu): [D][D] quantities of which the products read
+    // the bf16 rounding, as the byte images of their operand tiles (two T64 tiles of 128 rows, 32 KB a
+    // chunk): H_r and S^K_r (from the forward), dH (the state pass), DC_{r+1} + DC_{r+1}^T (the suffix)
+    const uint8_t *hs_img = nullptr, *sk_img = nullptr;
+    uint8_t *dh_img = nullptr, *dcs_img = nullptr;
     int *status = nullptr; // status word of the tensor-core products' bounded waits (TC kernels)
     int wave = 0;          // chunk CTAs resident at once: each prefetches into L2 the inputs of the
                            // chunk one wave after its own (ccq_gdn_bwd_chunk_tc.cu)

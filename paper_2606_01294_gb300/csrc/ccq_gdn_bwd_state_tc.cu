@@ -11,8 +11,9 @@
 //   dU  = X1 + diag(ed) Kbar dH                       (MMA1, 64 x 64 per column half, K = Dk)
 //   dR' = diag(E beta) Tt^T dU                        (MMA2, K = 64)
 //   dH <- e^{gc_last} dH + Y1 - Kbar^T dR'            (MMA3 accumulating into TMEM, K = 64)
-// and stores dH_{r+1} (the adjoint of the state leaving chunk r) for the per-chunk key/value
-// kernel; after chunk 0, dH is dS0.  The delta rule acts on the value columns of the state
+// and stores, for the per-chunk key/value kernel, the bf16 operand tile of dH_{r+1} (the adjoint of the
+// state leaving chunk r; the tile MMA1 reads, one bulk copy) and this half's <dH_{r+1}, H_r> in fp32;
+// after chunk 0, dH is dS0.  The delta rule acts on the value columns of the state
 // independently, so each (sequence, head) runs as two CTAs, one per half of the value columns.
 //
 // Layout: dH lives in TMEM as fp32 (128 lanes = key dim, 64 columns = this CTA's value
@@ -49,7 +50,7 @@ constexpr uint32_t OFF_DHB = OFF_TB + 8192;  // 172032: bf16 dH [128][64]
 constexpr uint32_t OFF_DUB = OFF_DHB + 16384;  // 188416: bf16 dU [64][64]
 constexpr uint32_t OFF_DRB = OFF_DUB + 8192;   // 196608: bf16 -dR' [64][64]
 constexpr uint32_t OFF_MISC = OFF_DRB + 8192;  // 204800
-constexpr uint32_t M_GC = 0, M_ED = 256, M_EB = 512, M_EL = 768, M_BAR = 832, M_TMEM = 896, M_ABORT = 900;
+constexpr uint32_t M_GC = 0, M_ED = 256, M_EB = 512, M_EL = 768, M_RED = 784, M_BAR = 832, M_TMEM = 896, M_ABORT = 900;
 constexpr uint32_t kMisc = 1280;
 constexpr uint32_t kSmem = OFF_MISC + kMisc + 1024;
 static_assert(kSmem <= 232448, "exceeds the 227 KB per-CTA limit");
@@ -85,6 +86,7 @@ gdn_bwd_state_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_
     float *eds = reinterpret_cast<float *>(misc + M_ED);  // e^{gc_last - gc_i}
     float *ebs = reinterpret_cast<float *>(misc + M_EB);  // E_i beta_i
     float *els = reinterpret_cast<float *>(misc + M_EL);  // e^{gc_last}
+    float *red = reinterpret_cast<float *>(misc + M_RED);  // [8] the warps' parts of <dH, H>
     uint64_t *bar = reinterpret_cast<uint64_t *>(misc + M_BAR);
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(misc + M_TMEM);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(misc + M_ABORT);
@@ -141,6 +143,15 @@ gdn_bwd_state_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_
         const size_t ci = chunk0 + r;
         uint8_t *base = sm + buf * BUF_BYTES;
         const uint32_t bsb = sb + buf * BUF_BYTES;
+        float hv[32];  // this thread's part of H_r, in flight until dH_{r+1} is read
+        {
+            const float4 *src = reinterpret_cast<const float4 *>(a.hs + (ci * kD + row) * kD + 64 * half + 32 * th);
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                const float4 v = src[e];
+                hv[4 * e] = v.x; hv[4 * e + 1] = v.y; hv[4 * e + 2] = v.z; hv[4 * e + 3] = v.w;
+            }
+        }
         if (it > 0) {
             // chunk r+1's three products are done: dH is updated, the shared tiles and buffer
             // buf ^ 1 are free; load chunk r-1 into that buffer
@@ -215,9 +226,12 @@ gdn_bwd_state_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_
         {
             float x[32];
             tmem_ld32(tq + TM_DH + 32 * th, x);
-            float4 *dst = reinterpret_cast<float4 *>(a.dh + (ci * kD + row) * kD + 64 * half + 32 * th);
+            float dot = 0.f;
 #pragma unroll
-            for (int e = 0; e < 8; ++e) dst[e] = make_float4(x[4 * e], x[4 * e + 1], x[4 * e + 2], x[4 * e + 3]);
+            for (int e = 0; e < 32; ++e) dot = fmaf(x[e], hv[e], dot);
+#pragma unroll
+            for (int o = 16; o >= 1; o >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, o);
+            if (lane == 0) red[warp] = dot;
 #pragma unroll
             for (int q = 0; q < 4; ++q) put_bf16x8(sm + OFF_DHB, row, 4 * th + q, x + 8 * q);
             const float el = *els;
@@ -236,6 +250,11 @@ gdn_bwd_state_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_
         fence_proxy_async_smem();
         tc_fence_before();
         __syncthreads();
+        if (tid == kThreads - 1) {
+            float dot = 0.f;
+            for (int w = 0; w < kThreads / 32; ++w) dot += red[w];
+            a.vec[ci * 4 * kC + 3 * kC + half] = dot;
+        }
         if (tid == 0 && !*abort_flag) {
             tc_fence_after();
             // MMA1: Kbar dH (M = 64 tokens, N = 64 columns, K = 128 key dims)
@@ -244,6 +263,8 @@ gdn_bwd_state_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_
             for (int k = 0; k < 8; ++k)
                 mma_bf16(tbase + TM_A1, dK + (k >> 2) * 512 + (k & 3) * 2, dH + k * 128, ID_M1, k != 0);
             mma_commit(&bar[BAR_M1]);
+            bulk_store(a.dh_img + ci * 32768 + half * 16384, sm + OFF_DHB, 16384);
+            tma_store_commit();
         }
         // ---- dU = X1 + diag(ed) Kbar dH (warps 0-3: row i, columns 32 hf .. + 31)
         mbar_wait(&bar[BAR_M1], it & 1, abort_flag, status);
@@ -299,6 +320,7 @@ gdn_bwd_state_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_
             const uint64_t dR = make_desc(sb + OFF_DRB, 8192, 1024);
             for (int k = 0; k < 4; ++k) mma_bf16(tbase + TM_DH, dKm + k * 128, dR + k * 128, ID_M3, 1);
             mma_commit(&bar[BAR_M3]);
+            tma_store_wait_read();  // before the barrier that lets the next chunk's dH over the tile
         }
     }
     // dS0 = dH after chunk 0

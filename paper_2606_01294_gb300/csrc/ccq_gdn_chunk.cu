@@ -407,6 +407,32 @@ constexpr uint32_t ID_64x128_KM = make_idesc(64, 128, 0, 1);
 constexpr uint32_t ID_128x128_MM = make_idesc(128, 128, 1, 1);
 constexpr uint32_t ID_128x64_MK = make_idesc(128, 64, 1, 0);
 
+// 32 columns [32 cc, 32 cc + 32) of row `row` as bf16 pairs, into a T64 tile in shared memory / into the
+// byte image of one in global memory, where two neighbouring 16-byte chunks are one 32-byte sector (the
+// swizzle swaps them in odd rows).
+__device__ __forceinline__ void put_row32(uint8_t *tile, int row, int cc, const uint32_t (&w)[16]) {
+#pragma unroll
+    for (int q4 = 0; q4 < 4; ++q4)
+        *reinterpret_cast<uint4 *>(tile + t64_chunk(row, 4 * cc + q4)) =
+            make_uint4(w[4 * q4], w[4 * q4 + 1], w[4 * q4 + 2], w[4 * q4 + 3]);
+}
+__device__ __forceinline__ void img_row32(uint8_t *img, int row, int cc, const uint32_t (&w)[16]) {
+    const bool odd = row & 1;
+#pragma unroll
+    for (int q8 = 0; q8 < 2; ++q8) {
+        uint32_t y[8];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            y[e] = odd ? w[8 * q8 + 4 + e] : w[8 * q8 + e];
+            y[4 + e] = odd ? w[8 * q8 + e] : w[8 * q8 + 4 + e];
+        }
+        asm volatile("st.global.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(
+                         img + (t64_chunk(row, 4 * cc + 2 * q8) & ~31u)),
+                     "r"(y[0]), "r"(y[1]), "r"(y[2]), "r"(y[3]), "r"(y[4]), "r"(y[5]), "r"(y[6]), "r"(y[7])
+                     : "memory");
+    }
+}
+
 __global__ void __launch_bounds__(kThreads, 1)
 gdn_chunk_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                  const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CUtensorMap map_tb,
@@ -546,23 +572,20 @@ gdn_chunk_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         const int i = 16 * (warp & 3) + (lane & 15);
         const int hf = lane >> 4;
         const int row = 32 * (warp & 3) + lane;  // state row of the M = 128 layout
-        // (with a.sk_out / a.hs_out the snapshots of chunk ch of this sequence also write the
-        // fp32 states to the backward's arrays)
+        // (with a.sk_img / a.hs_img the snapshots of chunk ch of this sequence also write the operand
+        // tiles they make to the backward's arrays, with a.hs_out the fp32 H)
+        auto state_img = [&](int ch) { return (static_cast<size_t>(bh) * NCt + ch) * 32768; };
         auto snap_sk = [&](int ch) {
             tc_fence_after();
 #pragma unroll
             for (int cc = 0; cc < 2; ++cc) {
                 float x[32];
                 tmem_ld32(tq + TM_SK + 64 * grp + 32 * cc, x);
-                if (a.sk_out) {
-                    float4 *dst = reinterpret_cast<float4 *>(
-                        a.sk_out + ((static_cast<size_t>(bh) * NCt + ch) * kD + row) * kD + 64 * grp + 32 * cc);
+                uint32_t w[16];
 #pragma unroll
-                    for (int e = 0; e < 8; ++e) dst[e] = make_float4(x[4 * e], x[4 * e + 1], x[4 * e + 2], x[4 * e + 3]);
-                }
-#pragma unroll
-                for (int q4 = 0; q4 < 4; ++q4)
-                    store_row_chunk(sm + OFF_SK + grp * 16384, row, 4 * cc + q4, x + 8 * q4);
+                for (int e = 0; e < 16; ++e) w[e] = pack_bf16(x[2 * e], x[2 * e + 1]);
+                put_row32(sm + OFF_SK + grp * 16384, row, cc, w);
+                if (a.sk_img) img_row32(a.sk_img + state_img(ch) + grp * 16384, row, cc, w);
             }
             fence_proxy_async_smem();
             tc_fence_before();
@@ -592,10 +615,8 @@ gdn_chunk_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
                     x[2 * e] = y.x;
                     x[2 * e + 1] = y.y;
                 }
-#pragma unroll
-                for (int q4 = 0; q4 < 4; ++q4)
-                    *reinterpret_cast<uint4 *>(sm + OFF_HB + grp * 16384 + t64_chunk(row, 4 * cc + q4)) =
-                        make_uint4(w[4 * q4], w[4 * q4 + 1], w[4 * q4 + 2], w[4 * q4 + 3]);
+                put_row32(sm + OFF_HB + grp * 16384, row, cc, w);
+                if (a.hs_img) img_row32(a.hs_img + state_img(ch) + grp * 16384, row, cc, w);
                 tmem_st32(tq + TM_S + 64 * grp + 32 * cc, x);
             }
             tmem_wait_st();

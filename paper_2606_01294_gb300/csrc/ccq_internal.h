@@ -72,10 +72,13 @@ struct ChunkArgs {
     const int *chunk_seq = nullptr;
     int vl_chunks = 0;  // cbase[B]: the packed chunk count
     // Gated DeltaNet, for the backward (no packed sequences): when set, the forward writes per
-    // chunk ch = (b H + h) NC + r of every (sequence, head), in fp32, what the backward reads:
-    // tt_out[ch][64][64] = Tt = (I + A)^{-1} (the WY kernel), and the states entering the chunk
-    // hs_out[ch][Dk][Dv] = H_r, sk_out[ch][Dk][Dk] = S^K_r, mk_out[ch][Dk] = M_r (the chunk kernel).
-    float *tt_out = nullptr, *hs_out = nullptr, *sk_out = nullptr, *mk_out = nullptr;
+    // chunk ch = (b H + h) NC + r of every (sequence, head) what the backward reads: in fp32
+    // tt_out[ch][64][64] = Tt = (I + A)^{-1} (the WY kernel), and of the states entering the chunk
+    // hs_out[ch][Dk][Dv] = H_r and mk_out[ch][Dk] = M_r (the chunk kernel); and as the byte images of
+    // its bf16 operand tiles (two T64 tiles of 128 rows, 32 KB a chunk, 32-byte aligned) hs_img = H_r
+    // and sk_img = S^K_r.
+    float *tt_out = nullptr, *hs_out = nullptr, *mk_out = nullptr;
+    uint8_t *hs_img = nullptr, *sk_img = nullptr;
 };
 
 // Per (sequence, segment) workspace: S [128][128], C [128][128], m [128], D [128].
