@@ -8,7 +8,8 @@
 
 namespace ccq {
 
-// Arguments of the token-by-token kernel (ccq_recurrent.cu).  dtype codes
+// Arguments of the decode step (ccq_recurrent.cu) and of the fp32 forward over a sequence
+// (ccq_recurrent_block.cu).  dtype codes
 // follow ccq_dtype (0 = bf16, 1 = fp32).
 struct RecurrentArgs {
     int backbone;  // 0 GLA, 1 Gated DeltaNet
@@ -24,7 +25,9 @@ struct RecurrentArgs {
     float *ST, *CT, *mT;
 };
 
+// T = 1: the decode step; else launch_recurrent_block.
 cudaError_t launch_recurrent(const RecurrentArgs &a, cudaStream_t s);
+cudaError_t launch_recurrent_block(const RecurrentArgs &a, cudaStream_t s);
 
 // tT[b] = t0[b] + T (t0 NULL: T), one thread per batch row.  The kernels leave
 // the final count to this launch, enqueued after them: tT may alias t0, and
