@@ -9,6 +9,7 @@ tensor is not on a CUDA device, the call raises.
 from __future__ import annotations
 
 import ctypes
+import functools
 import os
 import re
 from dataclasses import dataclass
@@ -150,8 +151,60 @@ def params(*, l2norm: bool = True, scale: Optional[float] = None, centered: bool
     return p
 
 
+# The calls below cost more on the host than a small case does on the GPU, so what depends on values alone
+# is formed once per value: the parameter block (never written by the library) and the workspace sizes
+# (bounded caches).  Addresses go to ctypes as plain integers, and a tensor that is as required passes _req on one
+# expression.  Measured on GB300's host: a decode step of two sequences 30 us before.
+@functools.lru_cache(maxsize=64)
+def _params_of(items):
+    p = params(**dict(items))
+    return p, ctypes.byref(p)
+
+
+def _items(kw):
+    """The keyword arguments as a cache key, or None when a value is not a plain one (a tensor, say)."""
+    if not kw:
+        return ()
+    if all(v is None or isinstance(v, (bool, int, float, str)) for v in kw.values()):
+        return tuple(sorted(kw.items()))
+    return None
+
+
+def _pref(kw):
+    """(block, reference) of the parameters ``kw``; the reference is good while the block is held."""
+    items = _items(kw)
+    if items is not None:
+        return _params_of(items)
+    p = params(**kw)
+    return p, ctypes.byref(p)
+
+
+def _query(fn, args, pref):
+    need = ctypes.c_size_t(0)
+    _check(getattr(load_library(), fn)(*args, pref, ctypes.byref(need)))
+    return need.value
+
+
+@functools.lru_cache(maxsize=256)
+def _size_of(fn, device, args, items):
+    return _query(fn, args, _params_of(items)[1])
+
+
+def _workspace_bytes(fn, args, kw):
+    """Workspace bytes from the library function ``fn``: a function of the sizes, the parameters and the current
+    device's SM count (the split of long sequences)."""
+    items = _items(kw)
+    if items is None:
+        return _query(fn, args, _pref(kw)[1])
+    try:
+        device = torch.cuda.current_device()
+    except (RuntimeError, AssertionError):  # no GPU: the library answers with a default SM count
+        device = -1
+    return _size_of(fn, device, args, items)
+
+
 def _ptr(x: Optional[torch.Tensor]):
-    return None if x is None else ctypes.c_void_p(x.data_ptr())
+    return None if x is None else x.data_ptr()
 
 
 def _dtype_code(t: torch.Tensor) -> int:
@@ -163,6 +216,9 @@ def _dtype_code(t: torch.Tensor) -> int:
 
 
 def _req(t, name, device, dtype=None, shape=None):
+    if (isinstance(t, torch.Tensor) and t.device == device and device.type == "cuda" and t.is_contiguous()
+            and (dtype is None or t.dtype == dtype) and (shape is None or t.shape == shape)):
+        return t
     if t is None:
         raise ValueError(f"{name} is required")
     if not isinstance(t, torch.Tensor) or t.device.type != "cuda":
@@ -178,9 +234,13 @@ def _req(t, name, device, dtype=None, shape=None):
     return t
 
 
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _stream(device, stream):
-    s = stream if stream is not None else torch.cuda.current_stream(device)
-    return ctypes.c_void_p(s.cuda_stream)
+    if stream is None and _raw_stream is not None and device.index is not None:
+        return _raw_stream(device.index)
+    return (stream if stream is not None else torch.cuda.current_stream(device)).cuda_stream
 
 
 @dataclass
@@ -201,10 +261,11 @@ class CCQState:
 
     @staticmethod
     def empty(B, H, Dk, Dv, device):
-        return CCQState(torch.empty(B, H, Dk, Dv, device=device),
-                        torch.empty(B, H, Dk, Dk, device=device),
-                        torch.empty(B, H, Dk, device=device),
-                        torch.empty(B, dtype=torch.int64, device=device))
+        f32 = torch.float32
+        return CCQState(torch.empty((B, H, Dk, Dv), dtype=f32, device=device),
+                        torch.empty((B, H, Dk, Dk), dtype=f32, device=device),
+                        torch.empty((B, H, Dk), dtype=f32, device=device),
+                        torch.empty((B,), dtype=torch.int64, device=device))
 
 
 def _state_in(state, B, H, Dk, Dv, device):
@@ -241,21 +302,19 @@ def gla_fwd(q, k, v, gk, lam, state: Optional[CCQState] = None, *, out=None,
     fs = final_state
     if fs is None and return_state:
         fs = CCQState.empty(B, H, Dk, Dv, dev)
-    p = params(**kw)
+    p, pref = _pref(kw)
     lib = load_library()
     if workspace is None:
-        need = ctypes.c_size_t(0)
-        _check(lib.ccq_gla_workspace_size(B, T, H, Dk, Dv, _dtype_code(q), ctypes.byref(p),
-                                          ctypes.byref(need)))
-        if need.value:
-            workspace = torch.empty(need.value, dtype=torch.uint8, device=dev)
+        need = _workspace_bytes("ccq_gla_workspace_size", (B, T, H, Dk, Dv, _dtype_code(q)), kw)
+        if need:
+            workspace = torch.empty(need, dtype=torch.uint8, device=dev)
     ws_bytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
     st = lib.ccq_gla_fwd(
         _ptr(q), _ptr(k), _ptr(v), _ptr(gk), _ptr(lam), _dtype_code(q), _dtype_code(gk),
         _ptr(S0), _ptr(C0), _ptr(m0), _ptr(t0), _ptr(o),
         _ptr(fs.S if fs else None), _ptr(fs.C if fs else None), _ptr(fs.m if fs else None),
         _ptr(fs.t if fs else None), B, T, H, Dk, Dv, _ptr(workspace), ws_bytes,
-        ctypes.byref(p), _stream(dev, stream))
+        pref, _stream(dev, stream))
     _check(st)
     return (o, fs) if return_state else o
 
@@ -290,33 +349,28 @@ def gla_fwd_save(q, k, v, gk, lam, state: Optional[CCQState] = None, *, ckpt=Non
     if ckpt is None:
         ckpt = torch.empty(gla_ckpt_size(B, T, H, Dk, Dv), dtype=torch.uint8, device=dev)
     _req(ckpt, "ckpt", dev, torch.uint8)
-    p = params(**kw)
+    p, pref = _pref(kw)
     lib = load_library()
     if workspace is None:
-        need = ctypes.c_size_t(0)
-        _check(lib.ccq_gla_workspace_size(B, T, H, Dk, Dv, _dtype_code(q), ctypes.byref(p),
-                                          ctypes.byref(need)))
-        if need.value:
-            workspace = torch.empty(need.value, dtype=torch.uint8, device=dev)
+        need = _workspace_bytes("ccq_gla_workspace_size", (B, T, H, Dk, Dv, _dtype_code(q)), kw)
+        if need:
+            workspace = torch.empty(need, dtype=torch.uint8, device=dev)
     ws_bytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
     st = lib.ccq_gla_fwd_save(
         _ptr(q), _ptr(k), _ptr(v), _ptr(gk), _ptr(lam), _dtype_code(q), _dtype_code(gk),
         _ptr(S0), _ptr(C0), _ptr(m0), _ptr(t0), _ptr(o),
         _ptr(fs.S if fs else None), _ptr(fs.C if fs else None), _ptr(fs.m if fs else None),
         _ptr(fs.t if fs else None), B, T, H, Dk, Dv, _ptr(workspace), ws_bytes,
-        _ptr(ckpt), ckpt.numel(), ctypes.byref(p), _stream(dev, stream))
+        _ptr(ckpt), ckpt.numel(), pref, _stream(dev, stream))
     _check(st)
     return o, fs, ckpt
 
 
 def gla_bwd_workspace(B, T, H, Dk, Dv, device, *, with_ckpt: bool, dtype=torch.bfloat16, **kw):
     """Allocate the workspace ccq_gla_bwd needs (None if none)."""
-    p = params(**kw)
-    need = ctypes.c_size_t(0)
     code = BF16 if dtype == torch.bfloat16 else FP32
-    _check(load_library().ccq_gla_bwd_workspace_size(B, T, H, Dk, Dv, code, int(bool(with_ckpt)),
-                                                      ctypes.byref(p), ctypes.byref(need)))
-    return torch.empty(need.value, dtype=torch.uint8, device=device) if need.value else None
+    need = _workspace_bytes("ccq_gla_bwd_workspace_size", (B, T, H, Dk, Dv, code, int(bool(with_ckpt))), kw)
+    return torch.empty(need, dtype=torch.uint8, device=device) if need else None
 
 
 def gla_bwd(q, k, v, gk, lam, dout, state: Optional[CCQState] = None, *, dST=None, dCT=None,
@@ -353,7 +407,7 @@ def gla_bwd(q, k, v, gk, lam, dout, state: Optional[CCQState] = None, *, dST=Non
         if g.get(name) is None:
             g[name] = torch.empty(shape, dtype=dt, device=dev)
         _req(g[name], name, dev, dt, shape)
-    p = params(**kw)
+    p, pref = _pref(kw)
     lib = load_library()
     if workspace is None:
         workspace = gla_bwd_workspace(B, T, H, Dk, Dv, dev, with_ckpt=ckpt is not None,
@@ -364,7 +418,7 @@ def gla_bwd(q, k, v, gk, lam, dout, state: Optional[CCQState] = None, *, dST=Non
         _ptr(S0), _ptr(C0), _ptr(m0), _ptr(t0), _ptr(dout), _ptr(dST), _ptr(dCT), _ptr(dmT),
         _ptr(ckpt), _ptr(g["dq"]), _ptr(g["dk"]), _ptr(g["dv"]), _ptr(g["dgk"]),
         _ptr(g["dlambda"]), _ptr(g["dS0"]), _ptr(g["dC0"]), _ptr(g["dm0"]),
-        B, T, H, Dk, Dv, _ptr(workspace), ws_bytes, ctypes.byref(p), _stream(dev, stream))
+        B, T, H, Dk, Dv, _ptr(workspace), ws_bytes, pref, _stream(dev, stream))
     _check(st)
     return g
 
@@ -390,20 +444,18 @@ def gdn_fwd(q, k, v, g, beta, lam, state: Optional[CCQState] = None, *, out=None
     fs = final_state
     if fs is None and return_state:
         fs = CCQState.empty(B, H, Dk, Dv, dev)
-    p = params(**kw)
+    p, pref = _pref(kw)
     lib = load_library()
-    need = ctypes.c_size_t(0)
-    _check(lib.ccq_gdn_workspace_size(B, T, H, Dk, Dv, _dtype_code(q), ctypes.byref(p),
-                                      ctypes.byref(need)))
-    if workspace is None and need.value:
-        workspace = torch.empty(need.value, dtype=torch.uint8, device=dev)
+    need = _workspace_bytes("ccq_gdn_workspace_size", (B, T, H, Dk, Dv, _dtype_code(q)), kw)
+    if workspace is None and need:
+        workspace = torch.empty(need, dtype=torch.uint8, device=dev)
     ws_bytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
     st = lib.ccq_gdn_fwd(
         _ptr(q), _ptr(k), _ptr(v), _ptr(g), _ptr(beta), _ptr(lam), _dtype_code(q),
         _ptr(S0), _ptr(C0), _ptr(m0), _ptr(t0), _ptr(o),
         _ptr(fs.S if fs else None), _ptr(fs.C if fs else None), _ptr(fs.m if fs else None),
         _ptr(fs.t if fs else None), B, T, H, Dk, Dv, _ptr(workspace), ws_bytes,
-        ctypes.byref(p), _stream(dev, stream))
+        pref, _stream(dev, stream))
     _check(st)
     return (o, fs) if return_state else o
 
@@ -442,20 +494,18 @@ def gdn_bwd(q, k, v, g, beta, lam, dout, state: Optional[CCQState] = None, *, dS
         if grads.get(name) is None:
             grads[name] = torch.empty(shape, dtype=dt, device=dev)
         _req(grads[name], name, dev, dt, shape)
-    p = params(**kw)
+    p, pref = _pref(kw)
     lib = load_library()
-    need = ctypes.c_size_t(0)
-    _check(lib.ccq_gdn_bwd_workspace_size(B, T, H, Dk, Dv, _dtype_code(q), ctypes.byref(p),
-                                          ctypes.byref(need)))
-    if workspace is None and need.value:
-        workspace = torch.empty(need.value, dtype=torch.uint8, device=dev)
+    need = _workspace_bytes("ccq_gdn_bwd_workspace_size", (B, T, H, Dk, Dv, _dtype_code(q)), kw)
+    if workspace is None and need:
+        workspace = torch.empty(need, dtype=torch.uint8, device=dev)
     ws_bytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
     st = lib.ccq_gdn_bwd(
         _ptr(q), _ptr(k), _ptr(v), _ptr(g), _ptr(beta), _ptr(lam), _dtype_code(q),
         _ptr(S0), _ptr(C0), _ptr(m0), _ptr(t0), _ptr(dout), _ptr(dST), _ptr(dCT), _ptr(dmT),
         _ptr(grads["dq"]), _ptr(grads["dk"]), _ptr(grads["dv"]), _ptr(grads["dg"]),
         _ptr(grads["dbeta"]), _ptr(grads["dlambda"]), _ptr(grads["dS0"]), _ptr(grads["dC0"]),
-        _ptr(grads["dm0"]), B, T, H, Dk, Dv, _ptr(workspace), ws_bytes, ctypes.byref(p),
+        _ptr(grads["dm0"]), B, T, H, Dk, Dv, _ptr(workspace), ws_bytes, pref,
         _stream(dev, stream))
     _check(st)
     return grads
@@ -494,20 +544,18 @@ def gdn_fwd_decayed(q, k, v, g, beta, lam, *, S0=None, C0=None, m0=None, n0=None
               "C": torch.empty(B, H, Dk, Dk, dtype=torch.float32, device=dev),
               "m": torch.empty(B, H, Dk, dtype=torch.float32, device=dev),
               "n": torch.empty(B, H, dtype=torch.float32, device=dev)}
-    p = params(**kw)
+    p, pref = _pref(kw)
     lib = load_library()
-    need = ctypes.c_size_t(0)
-    _check(lib.ccq_gdn_decayed_workspace_size(B, T, H, Dk, Dv, _dtype_code(q), ctypes.byref(p),
-                                              ctypes.byref(need)))
-    if workspace is None and need.value:
-        workspace = torch.empty(need.value, dtype=torch.uint8, device=dev)
+    need = _workspace_bytes("ccq_gdn_decayed_workspace_size", (B, T, H, Dk, Dv, _dtype_code(q)), kw)
+    if workspace is None and need:
+        workspace = torch.empty(need, dtype=torch.uint8, device=dev)
     ws_bytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
     st = lib.ccq_gdn_fwd_spectral(
         _ptr(q), _ptr(k), _ptr(v), _ptr(g), _ptr(beta), _ptr(lam), _dtype_code(q),
         _ptr(S0), _ptr(C0), _ptr(m0), _ptr(n0), _ptr(o),
         _ptr(fs["S"] if fs else None), _ptr(fs["C"] if fs else None), _ptr(fs["m"] if fs else None),
         _ptr(fs["n"] if fs else None), B, T, H, Dk, Dv, CONTRACTION[contraction], int(bool(decayed)),
-        _ptr(workspace), ws_bytes, ctypes.byref(p), _stream(dev, stream))
+        _ptr(workspace), ws_bytes, pref, _stream(dev, stream))
     _check(st)
     return (o, fs) if return_state else o
 
@@ -559,11 +607,11 @@ def fwd_varlen(backbone, q, k, v, gate, lam, cu_seqlens, *, beta=None, state: Op
     if fs is not None:
         _state_in(fs, ns, H, Dk, Dv, dev)
     cu_arr = (ctypes.c_int64 * len(cu))(*cu)
-    p = params(**kw)
+    p, pref = _pref(kw)
     lib = load_library()
     need = ctypes.c_size_t(0)
     _check(lib.ccq_fwd_varlen_workspace_size(int(backbone), ctypes.cast(cu_arr, _VP), ns, H, Dk, Dv,
-                                             _dtype_code(q), ctypes.byref(p), ctypes.byref(need)))
+                                             _dtype_code(q), pref, ctypes.byref(need)))
     if workspace is None and need.value:
         workspace = torch.empty(need.value, dtype=torch.uint8, device=dev)
     ws_bytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
@@ -571,39 +619,30 @@ def fwd_varlen(backbone, q, k, v, gate, lam, cu_seqlens, *, beta=None, state: Op
         int(backbone), _ptr(q), _ptr(k), _ptr(v), _ptr(gate), _ptr(beta), _ptr(lam), _dtype_code(q),
         _dtype_code(gate), ctypes.cast(cu_arr, _VP), ns, _ptr(S0), _ptr(C0), _ptr(m0), _ptr(t0), _ptr(o),
         _ptr(fs.S if fs else None), _ptr(fs.C if fs else None), _ptr(fs.m if fs else None),
-        _ptr(fs.t if fs else None), H, Dk, Dv, _ptr(workspace), ws_bytes, ctypes.byref(p), _stream(dev, stream))
+        _ptr(fs.t if fs else None), H, Dk, Dv, _ptr(workspace), ws_bytes, pref, _stream(dev, stream))
     _check(st)
     return (o, fs) if return_state else o
 
 
 def gla_workspace(B, T, H, Dk, Dv, device, dtype=torch.bfloat16, **kw):
     """Allocate the workspace ccq_gla_fwd needs for these sizes (None if none)."""
-    p = params(**kw)
-    need = ctypes.c_size_t(0)
     code = BF16 if dtype == torch.bfloat16 else FP32
-    _check(load_library().ccq_gla_workspace_size(B, T, H, Dk, Dv, code, ctypes.byref(p),
-                                                  ctypes.byref(need)))
-    return torch.empty(need.value, dtype=torch.uint8, device=device) if need.value else None
+    need = _workspace_bytes("ccq_gla_workspace_size", (B, T, H, Dk, Dv, code), kw)
+    return torch.empty(need, dtype=torch.uint8, device=device) if need else None
 
 
 def gdn_workspace(B, T, H, Dk, Dv, device, dtype=torch.bfloat16, **kw):
     """Allocate the workspace ccq_gdn_fwd needs for these sizes (None if none)."""
-    p = params(**kw)
-    need = ctypes.c_size_t(0)
     code = BF16 if dtype == torch.bfloat16 else FP32
-    _check(load_library().ccq_gdn_workspace_size(B, T, H, Dk, Dv, code, ctypes.byref(p),
-                                                  ctypes.byref(need)))
-    return torch.empty(need.value, dtype=torch.uint8, device=device) if need.value else None
+    need = _workspace_bytes("ccq_gdn_workspace_size", (B, T, H, Dk, Dv, code), kw)
+    return torch.empty(need, dtype=torch.uint8, device=device) if need else None
 
 
 def gdn_bwd_workspace(B, T, H, Dk, Dv, device, dtype=torch.bfloat16, **kw):
     """Allocate the workspace ccq_gdn_bwd needs for these sizes (None if none)."""
-    p = params(**kw)
-    need = ctypes.c_size_t(0)
     code = BF16 if dtype == torch.bfloat16 else FP32
-    _check(load_library().ccq_gdn_bwd_workspace_size(B, T, H, Dk, Dv, code, ctypes.byref(p),
-                                                      ctypes.byref(need)))
-    return torch.empty(need.value, dtype=torch.uint8, device=device) if need.value else None
+    need = _workspace_bytes("ccq_gdn_bwd_workspace_size", (B, T, H, Dk, Dv, code), kw)
+    return torch.empty(need, dtype=torch.uint8, device=device) if need else None
 
 
 def decode_step(backbone: int, q, k, v, gate, lam, state: CCQState, beta=None, *,
@@ -624,11 +663,11 @@ def decode_step(backbone: int, q, k, v, gate, lam, state: CCQState, beta=None, *
     S, C, m, t = _state_in(state, B, H, Dk, Dv, dev)
     o = out if out is not None else torch.empty(B, H, Dv, dtype=q.dtype, device=dev)
     _req(o, "out", dev, q.dtype, (B, H, Dv))
-    p = params(**kw)
+    p, pref = _pref(kw)
     st = load_library().ccq_decode_step(
         int(backbone), _ptr(q), _ptr(k), _ptr(v), _ptr(gate), _ptr(beta), _ptr(lam),
         _dtype_code(q), _dtype_code(gate), _ptr(S), _ptr(C), _ptr(m), _ptr(t), _ptr(o),
-        B, H, Dk, Dv, ctypes.byref(p), _stream(dev, stream))
+        B, H, Dk, Dv, pref, _stream(dev, stream))
     _check(st)
     return o
 

@@ -60,10 +60,10 @@ struct Shape {
     static constexpr int V = RPT < 4 ? RPT : 4; // consecutive rows a thread
     static constexpr int NV = RPT / V;
     static constexpr int LT = kL / NS;          // tokens whose scores a CTA forms
-    static constexpr int LD = D + 4;            // row stride of qbar, kbar (16-byte reads of a row a lane)
+    static constexpr int LD = D + 4;            // row stride of qbar, kbar, q_clean (16-byte accesses of a row a lane)
     static constexpr int NQ = kL * D / 4 / kThreads;
     static constexpr int NVV = (kL * DS / 4 + kThreads - 1) / kThreads;
-    static constexpr int F_Q = 0, F_K = F_Q + kL * LD, F_A = F_K + kL * LD, F_QC = F_A + kL * D, F_V = F_QC + kL * D,
+    static constexpr int F_Q = 0, F_K = F_Q + kL * LD, F_A = F_K + kL * LD, F_QC = F_A + kL * D, F_V = F_QC + kL * LD,
                          F_C = F_V + kL * DS, F_SC = F_C + DS * D, F_M = F_SC + kL * (kL + 1), F_CQ = F_M + D,
                          F_LAM = F_CQ + kL, F_G = F_LAM + kL, F_B = F_G + kL, F_QK = F_B + kL, kFloats = F_QK + kL;
     static_assert(TPC >= 2 && TPC <= 32 && RPT >= 2, "a column's threads share a warp");
@@ -143,6 +143,7 @@ __global__ void __launch_bounds__(kThreads, 1) recurrent_block_kernel(const Recu
             if (i < kL * DS / 4 && t < a.T)
                 pv[u] = load4(a.v, ((static_cast<size_t>(b) * a.T + t) * a.H + h) * D + col, a.in_dtype);
         }
+        pl = ps = pb = 0.f;  // past the sequence: lambda = 0, a decay of 1 and beta = 0
         if (tid < kL && tb + tid < a.T) {
             const size_t e = (static_cast<size_t>(b) * a.T + tb + tid) * a.H + h;
             pl = a.lambda[e];
@@ -252,34 +253,34 @@ __global__ void __launch_bounds__(kThreads, 1) recurrent_block_kernel(const Recu
         // ---- q_clean columns of this CTA's rows of C: lane = token, warp = rows d
         {
             const float tinv = 1.f / static_cast<float>(t0 + tb + lane + 1);
-            float cs = cq[lane];  // m_t . qbar_t
-#pragma unroll 8
-            for (int j = 0; j < kL; ++j) cs += sc[lane * LSC + j];
-            const float lt = lam[lane];
+            const float mq = cq[lane], lt = lam[lane];
             constexpr int U = DS / kWarps < 4 ? DS / kWarps : 4;  // rows at a time
             for (int u0 = 0; u0 < DS / kWarps; u0 += U) {
-                float z[U], ms[U];
+                float z[U], z4[U][4], ms[U], cs = mq;  // four chains a row for C qbar; cs = m_t . qbar_t
                 const int dl = warp * (DS / kWarps) + u0;  // local rows dl .. dl + U - 1
 #pragma unroll
                 for (int u = 0; u < U; ++u) {
-                    z[u] = 0.f;
+                    z4[u][0] = z4[u][1] = z4[u][2] = z4[u][3] = 0.f;
                     ms[u] = m[d0 + dl + u];
                 }
-#pragma unroll 4
+#pragma unroll(U <= 2 ? 16 : 4)
                 for (int x = 0; x < D; x += 4) {
                     const float4 qv = *reinterpret_cast<const float4 *>(qn + lane * LD + x);
 #pragma unroll
                     for (int u = 0; u < U; ++u) {
                         const float4 cv = *reinterpret_cast<const float4 *>(C + (dl + u) * D + x);
-                        z[u] = fmaf(cv.x, qv.x, z[u]);
-                        z[u] = fmaf(cv.y, qv.y, z[u]);
-                        z[u] = fmaf(cv.z, qv.z, z[u]);
-                        z[u] = fmaf(cv.w, qv.w, z[u]);
+                        z4[u][0] = fmaf(cv.x, qv.x, z4[u][0]);
+                        z4[u][1] = fmaf(cv.y, qv.y, z4[u][1]);
+                        z4[u][2] = fmaf(cv.z, qv.z, z4[u][2]);
+                        z4[u][3] = fmaf(cv.w, qv.w, z4[u][3]);
                     }
                 }
-#pragma unroll 4
+#pragma unroll
+                for (int u = 0; u < U; ++u) z[u] = (z4[u][0] + z4[u][1]) + (z4[u][2] + z4[u][3]);
+#pragma unroll(U <= 2 ? 16 : 8)
                 for (int j = 0; j < kL; ++j) {
                     const float w = sc[lane * LSC + j];
+                    cs += w;
 #pragma unroll
                     for (int u = 0; u < U; ++u) {
                         const float kv = kn[j * LD + d0 + dl + u];
@@ -292,10 +293,17 @@ __global__ void __launch_bounds__(kThreads, 1) recurrent_block_kernel(const Recu
                     const int d = d0 + dl + u;
                     float sig = z[u] * tinv;
                     if (a.centered) sig -= ms[u] * cs * tinv * tinv;
-                    const float x = qn[lane * LD + d] - lt * sig;
-#pragma unroll
-                    for (int p = 0; p < NS; ++p) *peer(qc + lane * D + d, p) = x;
+                    qc[lane * LD + d] = qn[lane * LD + d] - lt * sig;
                 }
+            }
+        }
+        if constexpr (NS > 1) {
+            // to the other CTAs, 16 bytes a store
+            __syncthreads();
+            constexpr int per = kL * DS / 4;
+            for (int i = tid; i < per * (NS - 1); i += kThreads) {
+                const int p = (s + 1 + i / per) % NS, x = i % per, off = (x / (DS / 4)) * LD + d0 + 4 * (x % (DS / 4));
+                *reinterpret_cast<float4 *>(peer(qc + off, p)) = *reinterpret_cast<const float4 *>(qc + off);
             }
         }
         sync_cluster();
@@ -310,7 +318,7 @@ __global__ void __launch_bounds__(kThreads, 1) recurrent_block_kernel(const Recu
                 float4 acc[U];
 #pragma unroll
                 for (int u = 0; u < U; ++u) acc[u] = *reinterpret_cast<const float4 *>(C + (r0 + RG * u) * D + p4);
-#pragma unroll 4
+#pragma unroll 8
                 for (int j = 0; j < kL; ++j) {
                     const float4 kv = *reinterpret_cast<const float4 *>(kn + j * LD + p4);
 #pragma unroll
@@ -339,65 +347,88 @@ __global__ void __launch_bounds__(kThreads, 1) recurrent_block_kernel(const Recu
                 float x = 0.f;
 #pragma unroll
                 for (int e = 0; e < D / 32; ++e)
-                    x = fmaf(qc[(warp + 8 * r) * D + lane + 32 * e], kn[(warp + 8 * r) * LD + lane + 32 * e], x);
+                    x = fmaf(qc[(warp + 8 * r) * LD + lane + 32 * e], kn[(warp + 8 * r) * LD + lane + 32 * e], x);
                 x = warp_sum(x);
                 if (lane == 0) qk[warp + 8 * r] = x;
             }
             __syncthreads();
         }
-        // ---- the backbone, token by token; o takes v's place
-        if (BB == 0) {
-#pragma unroll 4
-            for (int t = 0; t < n; ++t) {
-                const float vv = vs[t * DS + c];
-                float po = 0.f;
+        // ---- the backbone, token by token; o takes v's place.  The reads of a group of G tokens come
+        // before its stores (rows past the sequence have kbar = 0, a decay of 1 and beta = 0: no change)
+        constexpr int G = P::RPT > 8 ? (BB == 0 ? 4 : 2) : (BB == 0 ? 8 : 4);
+        constexpr bool kKeep = P::RPT <= 16;  // delta rule: a token's kbar rows stay in registers
+        for (int t0g = 0; t0g < n; t0g += G) {
+            float vv[G], r0[G], r1[G];  // GLA: q_clean . S in r0; GDN: kbar . S, q_clean . S
 #pragma unroll
-                for (int u = 0; u < P::NV; ++u) {
-                    const int r = P::V * (tl + P::TPC * u);
-                    float av[P::V], kv[P::V], qv[P::V];
-                    ldv<P::V>(al + t * D + r, av);
-                    ldv<P::V>(kn + t * LD + r, kv);
-                    ldv<P::V>(qc + t * D + r, qv);
+            for (int g = 0; g < G; ++g) vv[g] = vs[(t0g + g) * DS + c];
+#pragma unroll
+            for (int g = 0; g < G; ++g) {
+                const int t = t0g + g;
+                r0[g] = r1[g] = 0.f;
+                if (BB == 0) {
+#pragma unroll
+                    for (int u = 0; u < P::NV; ++u) {
+                        const int r = P::V * (tl + P::TPC * u);
+                        float av[P::V], kv[P::V], qv[P::V];
+                        ldv<P::V>(al + t * D + r, av);
+                        ldv<P::V>(kn + t * LD + r, kv);
+                        ldv<P::V>(qc + t * LD + r, qv);
+#pragma unroll
+                        for (int e = 0; e < P::V; ++e) {
+                            S[u][e] = fmaf(av[e], S[u][e], kv[e] * vv[g]);
+                            r0[g] = fmaf(S[u][e], qv[e], r0[g]);
+                        }
+                    }
+                } else {
+                    const float ag = gs[t], bt = be[t];
+                    float kv[kKeep ? P::NV : 1][P::V], p0[P::V], p1[P::V];
+#pragma unroll
+                    for (int e = 0; e < P::V; ++e) p0[e] = p1[e] = 0.f;
+#pragma unroll
+                    for (int u = 0; u < P::NV; ++u) {
+                        const int r = P::V * (tl + P::TPC * u), uk = kKeep ? u : 0;
+                        float qv[P::V];
+                        ldv<P::V>(kn + t * LD + r, kv[uk]);
+                        ldv<P::V>(qc + t * LD + r, qv);
+#pragma unroll
+                        for (int e = 0; e < P::V; ++e) {
+                            p0[e] = fmaf(kv[uk][e], S[u][e], p0[e]);
+                            p1[e] = fmaf(qv[e], S[u][e], p1[e]);
+                        }
+                    }
 #pragma unroll
                     for (int e = 0; e < P::V; ++e) {
-                        S[u][e] = fmaf(av[e], S[u][e], kv[e] * vv);
-                        po = fmaf(S[u][e], qv[e], po);
+                        r0[g] += p0[e];
+                        r1[g] += p1[e];
+                    }
+#pragma unroll
+                    for (int o = P::TPC / 2; o > 0; o >>= 1) r0[g] += __shfl_xor_sync(0xffffffffu, r0[g], o);
+                    // S <- alpha S + kbar (beta (v - alpha kbar^T S))
+                    const float w = bt * (vv[g] - ag * r0[g]);
+#pragma unroll
+                    for (int u = 0; u < P::NV; ++u) {
+                        if (!kKeep) ldv<P::V>(kn + t * LD + P::V * (tl + P::TPC * u), kv[0]);
+#pragma unroll
+                        for (int e = 0; e < P::V; ++e) S[u][e] = fmaf(kv[kKeep ? u : 0][e], w, ag * S[u][e]);
                     }
                 }
-#pragma unroll
-                for (int o = P::TPC / 2; o > 0; o >>= 1) po += __shfl_xor_sync(0xffffffffu, po, o);
-                if (tl == 0) vs[t * DS + c] = a.scale * po;
             }
-        } else {
-#pragma unroll 2
-            for (int t = 0; t < n; ++t) {
-                const float vv = vs[t * DS + c], ag = gs[t], bt = be[t];
-                float sk = 0.f, sq = 0.f, kv[P::NV][P::V];
 #pragma unroll
-                for (int u = 0; u < P::NV; ++u) {
-                    const int r = P::V * (tl + P::TPC * u);
-                    float qv[P::V];
-                    ldv<P::V>(kn + t * LD + r, kv[u]);
-                    ldv<P::V>(qc + t * D + r, qv);
+            for (int o = P::TPC / 2; o > 0; o >>= 1)
 #pragma unroll
-                    for (int e = 0; e < P::V; ++e) {
-                        sk = fmaf(kv[u][e], S[u][e], sk);
-                        sq = fmaf(qv[e], S[u][e], sq);
-                    }
+                for (int g = 0; g < G; ++g) {
+                    if (BB == 0) r0[g] += __shfl_xor_sync(0xffffffffu, r0[g], o);
+                    else r1[g] += __shfl_xor_sync(0xffffffffu, r1[g], o);
                 }
+            if (tl == 0)
 #pragma unroll
-                for (int o = P::TPC / 2; o > 0; o >>= 1) {
-                    sk += __shfl_xor_sync(0xffffffffu, sk, o);
-                    sq += __shfl_xor_sync(0xffffffffu, sq, o);
+                for (int g = 0; g < G; ++g) {
+                    const int t = t0g + g;
+                    // (delta rule: o = S_new^T q_clean expanded in the old state)
+                    vs[t * DS + c] = BB == 0 ? a.scale * r0[g]
+                                             : a.scale * (gs[t] * r1[g] - gs[t] * be[t] * qk[t] * r0[g] +
+                                                          be[t] * qk[t] * vv[g]);
                 }
-#pragma unroll
-                for (int u = 0; u < P::NV; ++u)
-#pragma unroll
-                    for (int e = 0; e < P::V; ++e)
-                        S[u][e] = ag * (S[u][e] - bt * kv[u][e] * sk) + bt * kv[u][e] * vv;
-                // o = S_new^T q_clean expanded in the old state
-                if (tl == 0) vs[t * DS + c] = a.scale * (ag * sq - ag * bt * qk[t] * sk + bt * qk[t] * vv);
-            }
         }
         __syncthreads();
         for (int i = tid; i < n * (DS / 4); i += kThreads) {
