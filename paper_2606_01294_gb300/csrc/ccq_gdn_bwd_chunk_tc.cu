@@ -51,11 +51,13 @@ __device__ __forceinline__ void signal_issue(int id) {
     named_bar_arrive(id, kAll);
 }
 
-// 256-bit global accesses: a thread's rows of 16 or 32 floats are 32-byte sectors of their own (32-byte
-// aligned; the workspace arrays are).
+// 256-bit global accesses (32-byte aligned; the workspace arrays are).  The stores, read again by a later kernel
+// only, are the first to leave L2, where the next chunk's prefetched inputs wait.
 __device__ __forceinline__ void st_global8(float *p, const float *v) {
-    asm volatile("st.global.v8.f32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(p), "f"(v[0]), "f"(v[1]), "f"(v[2]),
-                 "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7])
+    uint64_t policy;
+    asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(policy));
+    asm volatile("st.global.L2::cache_hint.v8.f32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8}, %9;" ::"l"(p), "f"(v[0]), "f"(v[1]),
+                 "f"(v[2]), "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7]), "l"(policy)
                  : "memory");
 }
 __device__ __forceinline__ void ld_global8(const float *p, float *v) {
@@ -104,18 +106,13 @@ __device__ __forceinline__ void put8(uint8_t *tile, int i, int hf, int grp, cons
     *reinterpret_cast<uint4 *>(tile + t64_chunk(i, 4 * hf + grp)) = pack8(f);
 }
 
-// 16 consecutive values of a token row (zero past the sequence).
+// The thread's 16 bf16 columns of a [64][128] tile, raw.
 struct Raw16 {
     uint4 a, b;
 };
-__device__ __forceinline__ Raw16 load_raw16(const void *base, size_t row, int c0, bool valid) {
-    Raw16 x{make_uint4(0u, 0u, 0u, 0u), make_uint4(0u, 0u, 0u, 0u)};
-    if (valid) {
-        const uint4 *p = reinterpret_cast<const uint4 *>(static_cast<const __nv_bfloat16 *>(base) + row * kD + c0);
-        x.a = p[0];
-        x.b = p[1];
-    }
-    return x;
+__device__ __forceinline__ Raw16 get16(const uint8_t *tile, int i, int hf, int grp) {
+    return Raw16{*reinterpret_cast<const uint4 *>(tile + hf * 8192 + t64_chunk(i, 2 * grp)),
+                 *reinterpret_cast<const uint4 *>(tile + hf * 8192 + t64_chunk(i, 2 * grp + 1))};
 }
 __device__ __forceinline__ void unpack16(const Raw16 &x, float (&f)[16]) {
     float lo[8], hi[8];
@@ -127,10 +124,32 @@ __device__ __forceinline__ void unpack16(const Raw16 &x, float (&f)[16]) {
         f[8 + e] = hi[e];
     }
 }
-__device__ __forceinline__ void store_row16(void *base, size_t row, int c0, const float (&f)[16]) {
-    uint4 *p = reinterpret_cast<uint4 *>(static_cast<__nv_bfloat16 *>(base) + row * kD + c0);
-    p[0] = pack8(f);
-    p[1] = pack8(f + 8);
+
+// A [64][128] token tile (two swizzled 64-column boxes) of chunk r of (b, h).  Loads go through TMA: a
+// thread's own row of a token tensor is 32 bytes in a line of its own (rows are H D apart), and loading
+// q, k, v, dO that way held a CTA's first loads for 10 K cycles.
+__device__ __forceinline__ void load_tokens(uint8_t *tile, const CUtensorMap *m, uint64_t *bar, int b, int h, int r) {
+    tma_load_4d(tile, m, bar, 0, h, r * kC, b);
+    tma_load_4d(tile + 8192, m, bar, 64, h, r * kC, b);
+}
+__device__ __forceinline__ void store_tokens(const CUtensorMap *m, const uint8_t *tile, int b, int h, int r) {
+    tma_store_4d(m, tile, 0, h, r * kC, b);
+    tma_store_4d(m, tile + 8192, 64, h, r * kC, b);
+}
+// 2-D tiled store of one box of an fp32 [rows][128] array (make_f32_rows_map).
+__device__ __forceinline__ void tma_store_2d(const CUtensorMap *m, const void *src, int c0, int c1) {
+    asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.tile.bulk_group [%0, {%1, %2}], [%3];" ::"l"(
+                     reinterpret_cast<uint64_t>(m)),
+                 "r"(c0), "r"(c1), "r"(smem_addr(src))
+                 : "memory");
+}
+// Four (or 4 n) fp32 columns of a row of a swizzled 32-column box.
+template <int N>
+__device__ __forceinline__ void put_f32(uint8_t *box, int row, int c4, const float *v) {
+#pragma unroll
+    for (int q = 0; q < N / 4; ++q)
+        *reinterpret_cast<float4 *>(box + t64_chunk(row, c4 + q)) =
+            make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
 }
 
 // The fp32 chunk tiles that one kernel writes and the other reads in the same thread layout (R, U, W):
@@ -243,10 +262,6 @@ __device__ __forceinline__ float row_norms(const uint8_t *qt, const uint8_t *kt,
     }
     return gbwd::rnorm_of(parts_total(p0, p1, tid & 31), l2norm);
 }
-__device__ __forceinline__ void put_raw16(uint8_t *tile, int i, int hf, int grp, const Raw16 &x) {
-    *reinterpret_cast<uint4 *>(tile + hf * 8192 + t64_chunk(i, 2 * grp)) = x.a;
-    *reinterpret_cast<uint4 *>(tile + hf * 8192 + t64_chunk(i, 2 * grp + 1)) = x.b;
-}
 
 // K = 64 or 128 products over T64 tiles.  A and B: descriptors of the first K = 16 step; K-major operands
 // advance 32 B a step and `*blk` (tile bytes >> 4) every 64, MN-major ones 2 KB a step.
@@ -258,30 +273,25 @@ __device__ __forceinline__ void mma_k(uint32_t d, uint64_t A, int ablk, uint64_t
                  id, (acc || k > 0) ? 1u : 0u);
 }
 
-// The chunk one wave later finds its strided token rows in L2 (one 128-byte line a thread).
-__device__ __forceinline__ void prefetch_rows(const void *t0, const void *t1, const void *t2, const void *t3,
-                                              const GdnBwdArgs &a, int ch, int tid) {
+// L2 prefetch of the token tiles of chunk ch.
+__device__ __forceinline__ void prefetch_tokens(const CUtensorMap *m, const GdnBwdArgs &a, int ch) {
     const int r = ch % a.NC, bh = ch / a.NC, b = bh / a.H, h = bh % a.H;
-    const int row = (tid >> 1) & 63, which = tid >> 7, t = r * kC + row;
-    if (t >= a.T) return;
-    const void *src = which == 0 ? t0 : which == 1 ? t1 : which == 2 ? t2 : t3;
-    const __nv_bfloat16 *p = static_cast<const __nv_bfloat16 *>(src) +
-                             ((static_cast<size_t>(b) * a.T + t) * a.H + h) * kD + 64 * (tid & 1);
-    asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
+    tma_prefetch_l2_4d(m, 0, h, r * kC, b);
+    tma_prefetch_l2_4d(m, 64, h, r * kC, b);
 }
 
 // =====================================================================================
 // gdn_bwd_local128_kernel: one CTA per (sequence, head, chunk)
 // =====================================================================================
 namespace lk {
-constexpr uint32_t OFF_Q = 0;        // qbar
+constexpr uint32_t OFF_Q = 0;        // qbar, then dq
 constexpr uint32_t OFF_K = 16384;    // kbar
 constexpr uint32_t OFF_SK = 32768;   // S^K_r (32 KB)
-constexpr uint32_t OFF_H = 65536;    // H_r (32 KB)
-constexpr uint32_t OFF_R = 98304;    // R, then W
+constexpr uint32_t OFF_H = 65536;    // H_r (32 KB); then, with U and q_clean, Y1 and DC on their way out
+constexpr uint32_t OFF_R = 98304;    // v, then R, then W
 constexpr uint32_t OFF_U = 114688;   // U
 constexpr uint32_t OFF_QC = 131072;  // q_clean
-constexpr uint32_t OFF_D = 147456;   // D = scale dO
+constexpr uint32_t OFF_D = 147456;   // D = scale dO; then, with E D, X1 on its way out
 constexpr uint32_t OFF_ED = 163840;  // diag(E) D
 constexpr uint32_t OFF_TB = 180224;  // Tt diag(beta), then dP
 constexpr uint32_t OFF_SA = 188416;  // (Qbar Kbar^T) o causal, then P, then (W Kbar^T) o causal
@@ -289,15 +299,20 @@ constexpr uint32_t OFF_MISC = 196608;
 constexpr int F_GC = 0, F_E = 64, F_BE = 128, F_TI = 192, F_LAM = 256, F_M = 320, F_SEG = 448, F_DM = 960,
               F_RN = 1088, F_CQ = 1216, F_RED = 1280, kReds = 4, kFloats = F_RED + kReds * 256;
 constexpr int LS = 72;               // row stride (floats) of the fp32 copy of masked Sc in U's and q_clean's place
-constexpr uint32_t M_BAR = kFloats * 4, M_TMEM = M_BAR + 80, M_ABORT = M_TMEM + 4;
+constexpr uint32_t M_BAR = kFloats * 4, M_TMEM = M_BAR + 96, M_ABORT = M_TMEM + 4;
 constexpr uint32_t kSmem = OFF_MISC + M_ABORT + 4 + 1024;
 static_assert(kSmem <= 232448, "exceeds the 227 KB per-CTA limit");
-enum { BIN = 0, B1, B2, B2B, B3, B3B, B4, B5, B5B, B6, kBars };
-static_assert(8 * kBars <= 80, "barriers reach the TMEM slot");
+enum { BTOK = 0, BIN, B1, B2, B2B, B3, B3B, B4, B5, B5B, B6, kBars };
+static_assert(8 * kBars <= 96, "barriers reach the TMEM slot");
 static_assert(OFF_QC == OFF_U + 16384 && 64 * LS * 4 <= 32768, "the fp32 staging spans U and q_clean");
 // TMEM columns: Sc, then P | dP, then dP Kbar, then W Kbar^T | KH, U, Y1, DC | z, X1, the dqbar terms | (E D) H^T
 constexpr uint32_t TM_A = 0, TM_A2 = 64, TM_B = 128, TM_C = 256, TM_D = 384;
 }  // namespace lk
+
+// Box g (32 fp32 columns of 128 rows, 16 KB) of a [128][128] array on its way out: H's tile, then U and q_clean.
+__device__ __forceinline__ uint8_t *square_box(uint8_t *sm, int g) {
+    return sm + (g < 2 ? lk::OFF_H + g * 16384 : lk::OFF_U + (g - 2) * 16384);
+}
 
 // Per chunk, everything that does not need dH.  Rounds (products, then the epilogue they feed):
 //   1  Sc = Qbar Kbar^T, KH = Kbar H | Z = Qbar S^K     masked Sc, cq, R = V - E KH
@@ -306,7 +321,12 @@ constexpr uint32_t TM_A = 0, TM_A2 = 64, TM_B = 128, TM_C = 256, TM_D = 384;
 //   4  dP Kbar, X1 = P^T D                               dqc, dlambda, W; X1
 //   5  Wk = W Kbar^T | W S^K, DC = W^T Qbar              masked Wk, cz; DC
 //   6  += Wk Kbar                                        dqbar, dq, the Dm increment
-__global__ void __launch_bounds__(kAll, 1) gdn_bwd_local128_kernel(const GdnBwdArgs a) {
+__global__ void __launch_bounds__(kAll, 1)
+gdn_bwd_local128_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
+                        const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CUtensorMap map_do,
+                        const __grid_constant__ CUtensorMap map_dq, const __grid_constant__ CUtensorMap map_x1,
+                        const __grid_constant__ CUtensorMap map_y1, const __grid_constant__ CUtensorMap map_dc,
+                        const GdnBwdArgs a) {
     using namespace lk;
     extern __shared__ uint8_t smem_raw[];
     uint8_t *sm = smem_align1024(smem_raw);
@@ -321,7 +341,7 @@ __global__ void __launch_bounds__(kAll, 1) gdn_bwd_local128_kernel(const GdnBwdA
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int ch = blockIdx.x, r = ch % a.NC, bh = ch / a.NC, b = bh / a.H, h = bh % a.H;
     const int n = min(kC, a.T - r * kC);
-    const size_t t64 = static_cast<size_t>(ch) * kC * kD, sq = static_cast<size_t>(ch) * kD * kD;
+    const size_t t64 = static_cast<size_t>(ch) * kC * kD;
     int *status = a.status;
 
     if (warp == kCompute / 32) {
@@ -330,6 +350,12 @@ __global__ void __launch_bounds__(kAll, 1) gdn_bwd_local128_kernel(const GdnBwdA
             for (int i = 0; i < kBars; ++i) mbar_init(&bar[i], 1);
             *abort_flag = 0;
             fence_barrier_init();
+            mbar_arrive_expect_tx(&bar[BTOK], 4 * 16384 + 512);
+            load_tokens(sm + OFF_Q, &map_q, &bar[BTOK], b, h, r);
+            load_tokens(sm + OFF_K, &map_k, &bar[BTOK], b, h, r);
+            bulk_load(M, a.mk + static_cast<size_t>(ch) * kD, 512, &bar[BTOK]);
+            load_tokens(sm + OFF_D, &map_do, &bar[BTOK], b, h, r);
+            load_tokens(sm + OFF_R, &map_v, &bar[BTOK], b, h, r);
             mbar_arrive_expect_tx(&bar[BIN], 65536);
             bulk_load(sm + OFF_H, a.hs_img + static_cast<size_t>(ch) * 32768, 32768, &bar[BIN]);
             bulk_load(sm + OFF_SK, a.sk_img + static_cast<size_t>(ch) * 32768, 32768, &bar[BIN]);
@@ -359,15 +385,6 @@ __global__ void __launch_bounds__(kAll, 1) gdn_bwd_local128_kernel(const GdnBwdA
             mma_commit(&bar[B1]);
             mma_k<128, false, true>(tb + TM_C, dQ, 512, dSKm, 0, ID_64x128_KM, false);
             last = B1;
-        }
-        {
-            // the chunk one wave later finds its inputs in L2
-            const int nx = ch + a.wave;
-            if (lane == 0 && a.wave > 0 && nx < static_cast<int>(gridDim.x)) {
-                bulk_prefetch_l2(a.hs_img + static_cast<size_t>(nx) * 32768, 32768);
-                bulk_prefetch_l2(a.sk_img + static_cast<size_t>(nx) * 32768, 32768);
-                bulk_prefetch_l2(a.tt + static_cast<size_t>(nx) * kC * kC, kC * kC * 4);
-            }
         }
         named_bar(3, kAll);
         tc_fence_after();
@@ -407,6 +424,19 @@ __global__ void __launch_bounds__(kAll, 1) gdn_bwd_local128_kernel(const GdnBwdA
             mma_commit(&bar[B5B]);
             last = B5B;
         }
+        {
+            // the chunk one wave later finds its inputs in L2
+            const int nx = ch + a.wave;
+            if (lane == 0 && a.wave > 0 && nx < static_cast<int>(gridDim.x)) {
+                prefetch_tokens(&map_q, a, nx);
+                prefetch_tokens(&map_k, a, nx);
+                prefetch_tokens(&map_do, a, nx);
+                prefetch_tokens(&map_v, a, nx);
+                bulk_prefetch_l2(a.hs_img + static_cast<size_t>(nx) * 32768, 32768);
+                bulk_prefetch_l2(a.sk_img + static_cast<size_t>(nx) * 32768, 32768);
+                bulk_prefetch_l2(a.tt + static_cast<size_t>(nx) * kC * kC, kC * kC * 4);
+            }
+        }
         named_bar(3, kAll);
         tc_fence_after();
         if (go()) {
@@ -415,6 +445,7 @@ __global__ void __launch_bounds__(kAll, 1) gdn_bwd_local128_kernel(const GdnBwdA
             last = B6;
         }
         if (lane == 0 && *abort_flag) {
+            mbar_drain(&bar[BTOK], 0);
             mbar_drain(&bar[BIN], 0);
             if (last >= 0) mbar_drain(&bar[last], 0);
         }
@@ -428,17 +459,11 @@ __global__ void __launch_bounds__(kAll, 1) gdn_bwd_local128_kernel(const GdnBwdA
     if (warp == 0) tmem_alloc(tmem_slot, 512);
     const bool valid = i < n;
     const size_t row = (static_cast<size_t>(b) * a.T + r * kC + (valid ? i : 0)) * a.H + h;
-    const Raw16 qr = load_raw16(a.q, row, c0, valid), kr = load_raw16(a.k, row, c0, valid);
-    const Raw16 vr = load_raw16(a.v, row, c0, valid), dr = load_raw16(a.dout, row, c0, valid);
-    if (tid < kD) {
-        M[tid] = a.mk[static_cast<size_t>(ch) * kD + tid];
-        dMs[tid] = 0.f;
-    }
-    put_raw16(sm + OFF_Q, i, hf, grp, qr);
-    put_raw16(sm + OFF_K, i, hf, grp, kr);
-    if (a.wave > 0 && ch + a.wave < static_cast<int>(gridDim.x)) prefetch_rows(a.q, a.k, a.v, a.dout, a, ch + a.wave, tid);
+    if (tid < kD) dMs[tid] = 0.f;
     __syncthreads();
     const uint32_t tb = *tmem_slot, tq = tb + (static_cast<uint32_t>(32 * qd) << 16);
+    mbar_wait(&bar[BTOK], 0, abort_flag, status);
+    const Raw16 qr = get16(sm + OFF_Q, i, hf, grp), kr = get16(sm + OFF_K, i, hf, grp);
     // row norms, and (threads 0-255) the M . qbar terms of cq in the same interleaved parts
     float m0 = 0.f, m1 = 0.f;
     {
@@ -472,7 +497,7 @@ __global__ void __launch_bounds__(kAll, 1) gdn_bwd_local128_kernel(const GdnBwdA
         fst[i * 32 + ((c0 / 4 + q) ^ (i & 7))] = make_float4(x[4 * q], x[4 * q + 1], x[4 * q + 2], x[4 * q + 3]);
     {
         float d[16];
-        unpack16(dr, d);
+        unpack16(get16(sm + OFF_D, i, hf, grp), d);
 #pragma unroll
         for (int e = 0; e < 16; ++e) d[e] *= a.scale;
         put16(sm + OFF_D, i, hf, grp, d);
@@ -533,7 +558,7 @@ __global__ void __launch_bounds__(kAll, 1) gdn_bwd_local128_kernel(const GdnBwdA
         *reinterpret_cast<float4 *>(scf + i * LS + s0) = make_float4(s[0], s[1], s[2], s[3]);
         *reinterpret_cast<float4 *>(scf + i * LS + s0 + 4) = make_float4(s[4], s[5], s[6], s[7]);
         float v[16];
-        unpack16(vr, v);
+        unpack16(get16(sm + OFF_R, i, hf, grp), v);
         acc_ld16(tq + TM_B + 16 * grp, x);
         const float ei = E[i];
 #pragma unroll
@@ -616,9 +641,14 @@ __global__ void __launch_bounds__(kAll, 1) gdn_bwd_local128_kernel(const GdnBwdA
         row_part(red, grp, i, hf, part);
         float y[32];
         tmem_ld32(tq + TM_B + 32 * grp, y);
-        float *Y1 = a.y1 + sq + (32 * qd + lane) * kD + 32 * grp;
-#pragma unroll
-        for (int e = 0; e < 32; e += 8) st_global8(Y1 + e, y + e);
+        // Y1 by TMA through the tiles of H, U and q_clean, whose products are done: one 32-column box a group
+        put_f32<32>(square_box(sm, grp), 32 * qd + lane, 0, y);
+    }
+    fence_proxy_async_smem();
+    compute_sync();
+    if (tid < 4) {
+        tma_store_2d(&map_y1, square_box(sm, tid), 32 * tid, ch * kD);
+        tma_store_commit();
     }
     // ---- round 4: dqc, dlambda, W; X1
     mbar_wait(&bar[B4], 0, abort_flag, status);
@@ -639,12 +669,8 @@ __global__ void __launch_bounds__(kAll, 1) gdn_bwd_local128_kernel(const GdnBwdA
         row_part(red + 256, grp, i, hf, part);
         acc_ld16(tq + TM_C + 16 * grp, x);
     }
+    put_f32<16>(sm + OFF_D + (2 * hf + (grp >> 1)) * 8192, i, 4 * (grp & 1), x);  // X1 in the tiles of D and E D
     signal_issue(2);
-    {
-        float *X1 = a.x1 + t64 + i * kD + c0;
-        st_global8(X1, x);
-        st_global8(X1 + 8, x + 8);
-    }
     st_own16(a.w + t64, tid, z);
     // ---- round 5: masked W Kbar^T, cz; DC
     mbar_wait(&bar[B5], 0, abort_flag, status);
@@ -660,8 +686,13 @@ __global__ void __launch_bounds__(kAll, 1) gdn_bwd_local128_kernel(const GdnBwdA
         put8(sm + OFF_SA, i, hf, grp, s);
         row_part(red + 512, grp, i, hf, part);
     }
+    if (tid < 4) tma_store_wait_read();  // Y1 has left its tiles
     signal_issue(3);
     compute_sync();
+    if (tid < 4) {
+        tma_store_2d(&map_x1, sm + OFF_D + tid * 8192, 32 * tid, ch * kC);
+        tma_store_commit();
+    }
     const float cz = row_total(red + 512, i) / ti;
     if (grp == 0 && hf == 0) {
         float *vec = a.vec + static_cast<size_t>(ch) * 4 * kC;
@@ -675,10 +706,9 @@ __global__ void __launch_bounds__(kAll, 1) gdn_bwd_local128_kernel(const GdnBwdA
     {
         float y[32];
         tmem_ld32(tq + TM_B + 32 * grp, y);
-        float *dC = a.dc + sq + (32 * qd + lane) * kD + 32 * grp;
-#pragma unroll
-        for (int e = 0; e < 32; e += 8) st_global8(dC + e, y + e);
+        put_f32<32>(square_box(sm, grp), 32 * qd + lane, 0, y);
     }
+    fence_proxy_async_smem();
     {
         // the Dm increment: sum_i (W_i cq_i t_i + qbar_i cz_i) / t_i^2
         const float ct = cq / ti, t2 = ti * ti;
@@ -703,12 +733,23 @@ __global__ void __launch_bounds__(kAll, 1) gdn_bwd_local128_kernel(const GdnBwdA
     }
     tc_fence_before();
     compute_sync();
-    if (valid) {
+    if (tid < 4) {
+        tma_store_2d(&map_dc, square_box(sm, tid), 32 * tid, ch * kD);
+        tma_store_commit();
+    }
+    {
         const float rdot = a.l2norm ? row_total(red + 768, i) : 0.f;
 #pragma unroll
         for (int e = 0; e < 16; ++e) x[e] = (dqc[e] - qb[e] * rdot) * rq;
-        store_row16(a.dq, row, c0, x);
+        put16(sm + OFF_Q, i, hf, grp, x);
+        fence_proxy_async_smem();
+        compute_sync();
+        if (tid == 0) {
+            store_tokens(&map_dq, sm + OFF_Q, b, h, r);
+            tma_store_commit();
+        }
     }
+    if (tid < 4) tma_store_wait_read();
     if (tid < kD) a.dm[static_cast<size_t>(ch) * kD + tid] = -cf * dMs[tid];
     __syncthreads();
     if (warp == 0) {
@@ -721,7 +762,7 @@ __global__ void __launch_bounds__(kAll, 1) gdn_bwd_local128_kernel(const GdnBwdA
 // gdn_bwd_kv128_kernel: one CTA per (sequence, head, chunk)
 // =====================================================================================
 namespace kk {
-constexpr uint32_t OFF_K = 0;        // kbar
+constexpr uint32_t OFF_K = 0;        // kbar, then dk
 constexpr uint32_t OFF_Q = 16384;    // qbar
 constexpr uint32_t OFF_W = 32768;    // W
 constexpr uint32_t OFF_D = 49152;    // D = scale dO, then R, then dR
@@ -732,19 +773,19 @@ constexpr uint32_t OFF_DH = 114688;  // dH (32 KB), then DC_{r+1} + DC_{r+1}^T
 constexpr uint32_t OFF_H = 147456;   // H_r (32 KB)
 constexpr uint32_t OFF_TT = 180224;  // Tt
 constexpr uint32_t OFF_DP = 188416;  // dP, then M2
-constexpr uint32_t OFF_QK = 196608;  // (Qbar Kbar^T) o causal
+constexpr uint32_t OFF_QK = 196608;  // v (with the next tile), then (Qbar Kbar^T) o causal
 constexpr uint32_t OFF_WK = 204800;  // (W Kbar^T) o causal
 constexpr uint32_t OFF_DT = 212992;  // dTb, then dKK + dKK^T
 constexpr uint32_t OFF_MISC = 221184;
 constexpr int F_GC = 0, F_E = 64, F_BE = 128, F_TI = 192, F_PCS = 256, F_CS = 320, F_DB = 384, F_SEG = 448,
               F_RN = 960, F_RED = 1088, kReds = 5, kFloats = F_RED + kReds * 256;
-constexpr uint32_t M_BAR = kFloats * 4, M_TMEM = M_BAR + 80, M_ABORT = M_TMEM + 4;
+constexpr uint32_t M_BAR = kFloats * 4, M_TMEM = M_BAR + 96, M_ABORT = M_TMEM + 4;
 constexpr uint32_t kSmem = OFF_MISC + M_ABORT + 4 + 1024;
 static_assert(kSmem <= 232448, "exceeds the 227 KB per-CTA limit");
 static_assert(OFF_U == OFF_QC + 16384 && 64 * 65 * 4 <= 32768, "the dKK staging spans q_clean and U");
 static_assert(M_BAR % 8 == 0, "barrier alignment");
-enum { BIN = 0, BDC, B1, B1B, B2, B2B, B3, B4, B5, kBars };
-static_assert(8 * kBars <= 80, "barriers reach the TMEM slot");
+enum { BTOK = 0, BIN, BDC, B1, B1B, B2, B2B, B3, B4, B5, kBars };
+static_assert(8 * kBars <= 96, "barriers reach the TMEM slot");
 // TMEM columns: t, then dR, then dR H^T | S, dP, then U dH^T | KK | QK, WK, then the sum of dk's other
 // products | dTb, then M2, then dA
 constexpr uint32_t TM_T = 0, TM_S = 128, TM_P = 192, TM_KK = 256, TM_ACC = 320, TM_WK = 384, TM_X = 448;
@@ -757,7 +798,11 @@ constexpr int LS = 65;  // row stride of the dKK staging (floats)
 //   3  M2 = Tt^T dTb | dR H^T                                    M2 diag(beta)
 //   4  dA = M2 Tt^T                                              dKK + dKK^T
 //   5  += (dKK + dKK^T) Kbar + Kbar (DC + DC^T)                  dk
-__global__ void __launch_bounds__(kAll, 1) gdn_bwd_kv128_kernel(const GdnBwdArgs a) {
+__global__ void __launch_bounds__(kAll, 1)
+gdn_bwd_kv128_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
+                     const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CUtensorMap map_do,
+                     const __grid_constant__ CUtensorMap map_dv, const __grid_constant__ CUtensorMap map_dk,
+                     const GdnBwdArgs a) {
     using namespace kk;
     extern __shared__ uint8_t smem_raw[];
     uint8_t *sm = smem_align1024(smem_raw);
@@ -784,6 +829,11 @@ __global__ void __launch_bounds__(kAll, 1) gdn_bwd_kv128_kernel(const GdnBwdArgs
             *abort_flag = 0;
             fence_barrier_init();
             const size_t img = static_cast<size_t>(ch) * 32768;
+            mbar_arrive_expect_tx(&bar[BTOK], 4 * 16384);
+            load_tokens(sm + OFF_K, &map_k, &bar[BTOK], b, h, r);
+            load_tokens(sm + OFF_Q, &map_q, &bar[BTOK], b, h, r);
+            load_tokens(sm + OFF_D, &map_do, &bar[BTOK], b, h, r);
+            load_tokens(sm + OFF_QK, &map_v, &bar[BTOK], b, h, r);
             mbar_arrive_expect_tx(&bar[BIN], 16384 + 65536);
             bulk_load(sm + OFF_DH, a.dh_img + img, 32768, &bar[BIN]);
             bulk_load(sm + OFF_QC, a.qc + t64 / 2, 16384, &bar[BIN]);
@@ -821,21 +871,6 @@ __global__ void __launch_bounds__(kAll, 1) gdn_bwd_kv128_kernel(const GdnBwdArgs
             mma_commit(&bar[B1B]);
             last = B1B;
         }
-        {
-            const int nx = ch + a.wave;
-            if (lane == 0 && a.wave > 0 && nx < static_cast<int>(gridDim.x)) {
-                const size_t nimg = static_cast<size_t>(nx) * 32768, n64 = static_cast<size_t>(nx) * kC * kD;
-                bulk_prefetch_l2(a.dh_img + nimg, 32768);
-                bulk_prefetch_l2(a.u + n64, kC * kD * 4);
-                bulk_prefetch_l2(a.w + n64, kC * kD * 4);
-                bulk_prefetch_l2(a.qc + n64 / 2, kC * kD * 2);
-                bulk_prefetch_l2(a.tt + static_cast<size_t>(nx) * kC * kC, kC * kC * 4);
-                bulk_prefetch_l2(a.hs_img + nimg, 32768);
-                bulk_prefetch_l2(a.r + n64, kC * kD * 4);
-                bulk_prefetch_l2(a.x1 + n64, kC * kD * 4);
-                bulk_prefetch_l2(a.dcs_img + nimg, 32768);
-            }
-        }
         named_bar(3, kAll);
         tc_fence_after();
         if (go()) {
@@ -869,6 +904,26 @@ __global__ void __launch_bounds__(kAll, 1) gdn_bwd_kv128_kernel(const GdnBwdArgs
             mbar_arrive_expect_tx(&bar[BDC], 32768);
             bulk_load(sm + OFF_DH, a.dcs_img + static_cast<size_t>(ch) * 32768, 32768, &bar[BDC]);
         }
+        {
+            // the chunk one wave later finds its inputs in L2
+            const int nx = ch + a.wave;
+            if (lane == 0 && a.wave > 0 && nx < static_cast<int>(gridDim.x)) {
+                const size_t nimg = static_cast<size_t>(nx) * 32768, n64 = static_cast<size_t>(nx) * kC * kD;
+                prefetch_tokens(&map_k, a, nx);
+                prefetch_tokens(&map_q, a, nx);
+                prefetch_tokens(&map_do, a, nx);
+                prefetch_tokens(&map_v, a, nx);
+                bulk_prefetch_l2(a.dh_img + nimg, 32768);
+                bulk_prefetch_l2(a.u + n64, kC * kD * 4);
+                bulk_prefetch_l2(a.w + n64, kC * kD * 4);
+                bulk_prefetch_l2(a.qc + n64 / 2, kC * kD * 2);
+                bulk_prefetch_l2(a.tt + static_cast<size_t>(nx) * kC * kC, kC * kC * 4);
+                bulk_prefetch_l2(a.hs_img + nimg, 32768);
+                bulk_prefetch_l2(a.r + n64, kC * kD * 4);
+                bulk_prefetch_l2(a.x1 + n64, kC * kD * 4);
+                bulk_prefetch_l2(a.dcs_img + nimg, 32768);
+            }
+        }
         named_bar(2, kAll);
         tc_fence_after();
         if (go()) {
@@ -886,6 +941,7 @@ __global__ void __launch_bounds__(kAll, 1) gdn_bwd_kv128_kernel(const GdnBwdArgs
             last = B5;
         }
         if (lane == 0 && *abort_flag) {
+            mbar_drain(&bar[BTOK], 0);
             mbar_drain(&bar[BIN], 0);
             if (dcs) mbar_drain(&bar[BDC], 0);
             if (last >= 0) mbar_drain(&bar[last], 0);
@@ -927,15 +983,9 @@ __global__ void __launch_bounds__(kAll, 1) gdn_bwd_kv128_kernel(const GdnBwdArgs
     const int qd = warp & 3, grp = warp >> 2, hf = lane >> 4, i = 16 * qd + (lane & 15);
     const int c0 = 64 * hf + 16 * grp, s0 = 32 * hf + 8 * grp;
     if (warp == 0) tmem_alloc(tmem_slot, 512);
-    const bool valid = i < n;
-    const size_t row = (static_cast<size_t>(b) * a.T + r * kC + (valid ? i : 0)) * a.H + h;
-    const Raw16 kr = load_raw16(a.k, row, c0, valid), qr = load_raw16(a.q, row, c0, valid);
-    const Raw16 dr = load_raw16(a.dout, row, c0, valid), vr = load_raw16(a.v, row, c0, valid);
     float u[16], x[16];
     ld_own16(a.u + t64, tid, u);
     if (tid < kC) pcs[tid] = cs[tid] = db1[tid] = 0.f;
-    put_raw16(sm + OFF_Q, i, hf, grp, qr);
-    put_raw16(sm + OFF_K, i, hf, grp, kr);
     put16(sm + OFF_U, i, hf, grp, u);
     ld_own16(a.w + t64, tid, x);
     put16(sm + OFF_W, i, hf, grp, x);
@@ -943,14 +993,15 @@ __global__ void __launch_bounds__(kAll, 1) gdn_bwd_kv128_kernel(const GdnBwdArgs
         float t[8];
         ld_global8(a.tt + static_cast<size_t>(ch) * kC * kC + 8 * tid, t);
         *reinterpret_cast<uint4 *>(sm + OFF_TT + t64_chunk(tid >> 3, tid & 7)) = pack8(t);
-        unpack16(dr, x);
-#pragma unroll
-        for (int e = 0; e < 16; ++e) x[e] *= a.scale;
-        put16(sm + OFF_D, i, hf, grp, x);
     }
-    if (a.wave > 0 && ch + a.wave < static_cast<int>(gridDim.x)) prefetch_rows(a.q, a.k, a.v, a.dout, a, ch + a.wave, tid);
     __syncthreads();
     const uint32_t tb = *tmem_slot, tq = tb + (static_cast<uint32_t>(32 * qd) << 16);
+    mbar_wait(&bar[BTOK], 0, abort_flag, status);
+    const Raw16 kr = get16(sm + OFF_K, i, hf, grp), qr = get16(sm + OFF_Q, i, hf, grp), vr = get16(sm + OFF_QK, i, hf, grp);
+    unpack16(get16(sm + OFF_D, i, hf, grp), x);
+#pragma unroll
+    for (int e = 0; e < 16; ++e) x[e] *= a.scale;
+    put16(sm + OFF_D, i, hf, grp, x);
     {
         uint32_t w[16];
         const float rr = row_norms(sm + OFF_Q, sm + OFF_K, tid, a.l2norm, w);
@@ -1043,12 +1094,16 @@ __global__ void __launch_bounds__(kAll, 1) gdn_bwd_kv128_kernel(const GdnBwdArgs
         acc_ld8(tq + TM_X + 8 * grp, t);
         put8(sm + OFF_DT, i, hf, grp, t);
         signal_issue(3);
-        if (valid) store_row16(a.dv, row, c0, x);
         row_part(red + 1024, grp, i, hf, part);
 #pragma unroll
         for (int e = 0; e < 8; ++e) t[e] *= tt[e];
         col_sums<8>(t, lane);
         if (!(lane & 1)) atomicAdd(&db1[s0 + ((lane >> 1) & 7)], t[0]);
+    }
+    compute_sync();
+    if (tid == 0) {  // dv is the bf16 tile of dR (signal_issue's fence came before the barrier)
+        store_tokens(&map_dv, sm + OFF_D, b, h, r);
+        tma_store_commit();
     }
     // the reverse sums G_i = sum_{l >= i} (W_l cq_l t_l + qbar_l cz_l) / t_l^2: sixteen rows by shuffle, the
     // quadrants' totals through segs
@@ -1146,11 +1201,18 @@ __global__ void __launch_bounds__(kAll, 1) gdn_bwd_kv128_kernel(const GdnBwdArgs
     }
     tc_fence_before();
     compute_sync();
-    if (valid) {
+    {
         const float rdot = a.l2norm ? row_total(red, i) : 0.f;
 #pragma unroll
         for (int e = 0; e < 16; ++e) x[e] = (dmv[e] - x[e] * rdot) * rk;
-        store_row16(a.dk, row, c0, x);
+        put16(sm + OFF_K, i, hf, grp, x);
+        fence_proxy_async_smem();
+        compute_sync();
+        if (tid == 0) {
+            store_tokens(&map_dk, sm + OFF_K, b, h, r);
+            tma_store_commit();
+            tma_store_wait_read();
+        }
     }
     __syncthreads();
     if (warp == 0) {
@@ -1259,7 +1321,17 @@ cudaError_t launch_gdn_local128(const gbwd::GdnBwdArgs &a, cudaStream_t s) {
     cudaError_t e = cudaFuncSetAttribute(gdn_bwd_local128_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          static_cast<int>(lk::kSmem));
     if (e != cudaSuccess) return e;
-    gdn_bwd_local128_kernel<<<static_cast<unsigned>(a.B * a.H * a.NC), kAll, lk::kSmem, s>>>(a);
+    const long long chunks = static_cast<long long>(a.B) * a.H * a.NC;
+    CUtensorMap q, k, v, d, dq, x1, y1, dc;
+    if (!make_token_map(&q, a.q, 2, a.B, a.T, a.H, kD, 64, true) ||
+        !make_token_map(&k, a.k, 2, a.B, a.T, a.H, kD, 64, true) ||
+        !make_token_map(&v, a.v, 2, a.B, a.T, a.H, kD, 64, true) ||
+        !make_token_map(&d, a.dout, 2, a.B, a.T, a.H, kD, 64, true) ||
+        !make_token_map(&dq, a.dq, 2, a.B, a.T, a.H, kD, 64, true) ||
+        !make_f32_rows_map(&x1, a.x1, chunks * kC, kD, 32, kC) ||
+        !make_f32_rows_map(&y1, a.y1, chunks * kD, kD, 32, kD) || !make_f32_rows_map(&dc, a.dc, chunks * kD, kD, 32, kD))
+        return cudaErrorInvalidValue;
+    gdn_bwd_local128_kernel<<<static_cast<unsigned>(chunks), kAll, lk::kSmem, s>>>(q, k, v, d, dq, x1, y1, dc, a);
     return cudaGetLastError();
 }
 
@@ -1272,7 +1344,15 @@ cudaError_t launch_gdn_kv128(const gbwd::GdnBwdArgs &a, cudaStream_t s) {
     cudaError_t e = cudaFuncSetAttribute(gdn_bwd_kv128_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          static_cast<int>(kk::kSmem));
     if (e != cudaSuccess) return e;
-    gdn_bwd_kv128_kernel<<<static_cast<unsigned>(a.B * a.H * a.NC), kAll, kk::kSmem, s>>>(a);
+    CUtensorMap q, k, v, d, dv, dk;
+    if (!make_token_map(&q, a.q, 2, a.B, a.T, a.H, kD, 64, true) ||
+        !make_token_map(&k, a.k, 2, a.B, a.T, a.H, kD, 64, true) ||
+        !make_token_map(&v, a.v, 2, a.B, a.T, a.H, kD, 64, true) ||
+        !make_token_map(&d, a.dout, 2, a.B, a.T, a.H, kD, 64, true) ||
+        !make_token_map(&dv, a.dv, 2, a.B, a.T, a.H, kD, 64, true) ||
+        !make_token_map(&dk, a.dk, 2, a.B, a.T, a.H, kD, 64, true))
+        return cudaErrorInvalidValue;
+    gdn_bwd_kv128_kernel<<<static_cast<unsigned>(a.B * a.H * a.NC), kAll, kk::kSmem, s>>>(q, k, v, d, dv, dk, a);
     return cudaGetLastError();
 }
 
