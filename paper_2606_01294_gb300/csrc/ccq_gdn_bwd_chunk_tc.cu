@@ -152,7 +152,7 @@ __device__ __forceinline__ void put_f32(uint8_t *box, int row, int c4, const flo
             make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
 }
 
-// The fp32 chunk tiles that one kernel writes and the other reads in the same thread layout (R, U, W):
+// The fp32 chunk tiles that one kernel writes and the other reads in the same thread layout (R, U, G):
 // 32 bytes a thread, consecutive threads consecutive in memory.
 __device__ __forceinline__ void st_own16(float *tile, int tid, const float (&f)[16]) {
     st_global8(tile + 8 * tid, f);
@@ -163,26 +163,19 @@ __device__ __forceinline__ void ld_own16(const float *tile, int tid, float (&f)[
     ld_global8(tile + 8 * (kCompute + tid), f + 8);
 }
 
-// Sums over the sixteen rows of a half-warp of N columns: leaves in v[0] the sum of column lane & 15 (N = 16)
-// or (lane >> 1) & 7 (N = 8).
-template <int N>
-__device__ __forceinline__ void col_sums(float (&v)[N], int lane) {
-    int m = N;
+// Sums over the sixteen rows of a half-warp of eight columns: leaves in v[0] the sum of column (lane >> 1) & 7.
+__device__ __forceinline__ void col_sums(float (&v)[8], int lane) {
 #pragma unroll
-    for (int o = 8; o >= 1; o >>= 1) {
-        if (m > 1) {
-            m >>= 1;
-            const bool up = (lane & o) != 0;
+    for (int m = 4, o = 8; m >= 1; m >>= 1, o >>= 1) {
+        const bool up = (lane & o) != 0;
 #pragma unroll
-            for (int e = 0; e < N / 2; ++e)
-                if (e < m) {
-                    const float send = up ? v[e] : v[e + m], keep = up ? v[e + m] : v[e];
-                    v[e] = keep + __shfl_xor_sync(0xffffffffu, send, o);
-                }
-        } else {
-            v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
-        }
+        for (int e = 0; e < 4; ++e)
+            if (e < m) {
+                const float send = up ? v[e] : v[e + m], keep = up ? v[e + m] : v[e];
+                v[e] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+            }
     }
+    v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1);
 }
 
 // Row sums: the eight threads of row i add up (two by shuffle, four through red[4][64]).
@@ -296,8 +289,8 @@ constexpr uint32_t OFF_ED = 163840;  // diag(E) D
 constexpr uint32_t OFF_TB = 180224;  // Tt diag(beta), then dP
 constexpr uint32_t OFF_SA = 188416;  // (Qbar Kbar^T) o causal, then P, then (W Kbar^T) o causal
 constexpr uint32_t OFF_MISC = 196608;
-constexpr int F_GC = 0, F_E = 64, F_BE = 128, F_TI = 192, F_LAM = 256, F_M = 320, F_SEG = 448, F_DM = 960,
-              F_RN = 1088, F_CQ = 1216, F_RED = 1280, kReds = 4, kFloats = F_RED + kReds * 256;
+constexpr int F_GC = 0, F_E = 64, F_BE = 128, F_TI = 192, F_LAM = 256, F_M = 320, F_SEG = 448, F_RN = 960,
+              F_CQ = 1088, F_RED = 1152, kReds = 4, kFloats = F_RED + kReds * 256;
 constexpr int LS = 72;               // row stride (floats) of the fp32 copy of masked Sc in U's and q_clean's place
 constexpr uint32_t M_BAR = kFloats * 4, M_TMEM = M_BAR + 96, M_ABORT = M_TMEM + 4;
 constexpr uint32_t kSmem = OFF_MISC + M_ABORT + 4 + 1024;
@@ -333,7 +326,7 @@ gdn_bwd_local128_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
     const uint32_t sb = smem_addr(sm);
     float *fm = reinterpret_cast<float *>(sm + OFF_MISC);
     float *gc = fm + F_GC, *E = fm + F_E, *be = fm + F_BE, *tinv = fm + F_TI, *lam = fm + F_LAM, *M = fm + F_M;
-    float *segs = fm + F_SEG, *dMs = fm + F_DM, *rn = fm + F_RN, *cqs = fm + F_CQ, *red = fm + F_RED;
+    float *segs = fm + F_SEG, *rn = fm + F_RN, *cqs = fm + F_CQ, *red = fm + F_RED;
     uint64_t *bar = reinterpret_cast<uint64_t *>(sm + OFF_MISC + M_BAR);
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(sm + OFF_MISC + M_TMEM);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(sm + OFF_MISC + M_ABORT);
@@ -403,6 +396,10 @@ gdn_bwd_local128_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
             mma_commit(&bar[B3]);
             mma_k<128, false, false>(tb + TM_D, dED, 512, dH, 1024, ID_64x128_KK, false);
             mma_k<64, true, true>(tb + TM_B, dQCm, 0, dEDm, 0, ID_128x128_MM, false);
+            // q_clean as the kv kernel's operand tile (read before B3B: Y1 then goes over it)
+            bulk_store(a.qc + t64 / 2, sm + OFF_QC, 16384);
+            tma_store_commit();
+            tma_store_wait_read();
             mma_commit(&bar[B3B]);
             last = B3B;
         }
@@ -422,6 +419,8 @@ gdn_bwd_local128_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
             mma_k<128, false, true>(tb + TM_C, dR, 512, dSKm, 0, ID_64x128_KM, false);
             mma_k<64, true, true>(tb + TM_B, dRm, 0, dQm, 0, ID_128x128_MM, false);
             mma_commit(&bar[B5B]);
+            bulk_store(a.w_img + static_cast<size_t>(ch) * 16384, sm + OFF_R, 16384);  // W likewise
+            tma_store_commit();
             last = B5B;
         }
         {
@@ -449,6 +448,7 @@ gdn_bwd_local128_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
             mbar_drain(&bar[BIN], 0);
             if (last >= 0) mbar_drain(&bar[last], 0);
         }
+        if (lane == 0) tma_store_wait_read();
         __syncthreads();
         return;
     }
@@ -459,7 +459,6 @@ gdn_bwd_local128_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
     if (warp == 0) tmem_alloc(tmem_slot, 512);
     const bool valid = i < n;
     const size_t row = (static_cast<size_t>(b) * a.T + r * kC + (valid ? i : 0)) * a.H + h;
-    if (tid < kD) dMs[tid] = 0.f;
     __syncthreads();
     const uint32_t tb = *tmem_slot, tq = tb + (static_cast<uint32_t>(32 * qd) << 16);
     mbar_wait(&bar[BTOK], 0, abort_flag, status);
@@ -603,12 +602,6 @@ gdn_bwd_local128_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
     }
     put16(sm + OFF_QC, i, hf, grp, x);
     signal_issue(2);
-    {
-        // q_clean as the kv kernel's operand tile
-        uint8_t *img = reinterpret_cast<uint8_t *>(a.qc + t64 / 2) + hf * 8192;
-        *reinterpret_cast<uint4 *>(img + t64_chunk(i, 2 * grp)) = pack8(x);
-        *reinterpret_cast<uint4 *>(img + t64_chunk(i, 2 * grp + 1)) = pack8(x + 8);
-    }
     // ---- round 3: P, dP; E rowsum((Qc H) o D); Y1
     float gam[8];  // Gamma o causal
     {
@@ -671,7 +664,6 @@ gdn_bwd_local128_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
     }
     put_f32<16>(sm + OFF_D + (2 * hf + (grp >> 1)) * 8192, i, 4 * (grp & 1), x);  // X1 in the tiles of D and E D
     signal_issue(2);
-    st_own16(a.w + t64, tid, z);
     // ---- round 5: masked W Kbar^T, cz; DC
     mbar_wait(&bar[B5], 0, abort_flag, status);
     tc_fence_after();
@@ -710,12 +702,22 @@ gdn_bwd_local128_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
     }
     fence_proxy_async_smem();
     {
-        // the Dm increment: sum_i (W_i cq_i t_i + qbar_i cz_i) / t_i^2
+        // the reverse sums G_i = sum_{l >= i} (W_l cq_l t_l + qbar_l cz_l) / t_l^2 for dk (sixteen rows by shuffle,
+        // the quadrants' totals through segs); G of the first row is the Dm increment
         const float ct = cq / ti, t2 = ti * ti;
 #pragma unroll
         for (int e = 0; e < 16; ++e) z[e] = (z[e] * ct + qb[e] * cz) * t2;
-        col_sums<16>(z, lane);
-        atomicAdd(&dMs[c0 + (lane & 15)], z[0]);
+#pragma unroll
+        for (int o = 1; o < 16; o <<= 1)
+#pragma unroll
+            for (int e = 0; e < 16; ++e) {
+                const float y = __shfl_down_sync(0xffffffffu, z[e], o, 16);
+                if ((lane & 15) + o < 16) z[e] += y;
+            }
+        if ((lane & 15) == 0)
+#pragma unroll
+            for (int e = 0; e < 16; e += 4)
+                *reinterpret_cast<float4 *>(segs + qd * kD + c0 + e) = make_float4(z[e], z[e + 1], z[e + 2], z[e + 3]);
     }
     // ---- round 6: dqbar, dq
     mbar_wait(&bar[B6], 0, abort_flag, status);
@@ -738,6 +740,16 @@ gdn_bwd_local128_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
         tma_store_commit();
     }
     {
+        for (int s = qd + 1; s < 4; ++s)
+#pragma unroll
+            for (int e = 0; e < 16; e += 4) {
+                const float4 y = *reinterpret_cast<const float4 *>(segs + s * kD + c0 + e);
+                z[e] += y.x;
+                z[e + 1] += y.y;
+                z[e + 2] += y.z;
+                z[e + 3] += y.w;
+            }
+        st_own16(a.w + t64, tid, z);
         const float rdot = a.l2norm ? row_total(red + 768, i) : 0.f;
 #pragma unroll
         for (int e = 0; e < 16; ++e) x[e] = (dqc[e] - qb[e] * rdot) * rq;
@@ -750,7 +762,8 @@ gdn_bwd_local128_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
         }
     }
     if (tid < 4) tma_store_wait_read();
-    if (tid < kD) a.dm[static_cast<size_t>(ch) * kD + tid] = -cf * dMs[tid];
+    if (tid < kD)
+        a.dm[static_cast<size_t>(ch) * kD + tid] = -cf * ((segs[tid] + segs[kD + tid]) + (segs[2 * kD + tid] + segs[3 * kD + tid]));
     __syncthreads();
     if (warp == 0) {
         tc_fence_after();
@@ -777,8 +790,8 @@ constexpr uint32_t OFF_QK = 196608;  // v (with the next tile), then (Qbar Kbar^
 constexpr uint32_t OFF_WK = 204800;  // (W Kbar^T) o causal
 constexpr uint32_t OFF_DT = 212992;  // dTb, then dKK + dKK^T
 constexpr uint32_t OFF_MISC = 221184;
-constexpr int F_GC = 0, F_E = 64, F_BE = 128, F_TI = 192, F_PCS = 256, F_CS = 320, F_DB = 384, F_SEG = 448,
-              F_RN = 960, F_RED = 1088, kReds = 5, kFloats = F_RED + kReds * 256;
+constexpr int F_GC = 0, F_E = 64, F_BE = 128, F_TI = 192, F_PCS = 256, F_CS = 320, F_DB = 384, F_RN = 448,
+              F_RED = 576, kReds = 5, kFloats = F_RED + kReds * 256;
 constexpr uint32_t M_BAR = kFloats * 4, M_TMEM = M_BAR + 96, M_ABORT = M_TMEM + 4;
 constexpr uint32_t kSmem = OFF_MISC + M_ABORT + 4 + 1024;
 static_assert(kSmem <= 232448, "exceeds the 227 KB per-CTA limit");
@@ -809,7 +822,7 @@ gdn_bwd_kv128_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
     const uint32_t sb = smem_addr(sm);
     float *fm = reinterpret_cast<float *>(sm + OFF_MISC);
     float *gc = fm + F_GC, *E = fm + F_E, *be = fm + F_BE, *tinv = fm + F_TI, *pcs = fm + F_PCS, *cs = fm + F_CS;
-    float *db1 = fm + F_DB, *segs = fm + F_SEG, *rn = fm + F_RN, *red = fm + F_RED;
+    float *db1 = fm + F_DB, *rn = fm + F_RN, *red = fm + F_RED;
     uint64_t *bar = reinterpret_cast<uint64_t *>(sm + OFF_MISC + M_BAR);
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(sm + OFF_MISC + M_TMEM);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(sm + OFF_MISC + M_ABORT);
@@ -834,9 +847,10 @@ gdn_bwd_kv128_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
             load_tokens(sm + OFF_Q, &map_q, &bar[BTOK], b, h, r);
             load_tokens(sm + OFF_D, &map_do, &bar[BTOK], b, h, r);
             load_tokens(sm + OFF_QK, &map_v, &bar[BTOK], b, h, r);
-            mbar_arrive_expect_tx(&bar[BIN], 16384 + 65536);
+            mbar_arrive_expect_tx(&bar[BIN], 2 * 16384 + 65536);
             bulk_load(sm + OFF_DH, a.dh_img + img, 32768, &bar[BIN]);
             bulk_load(sm + OFF_QC, a.qc + t64 / 2, 16384, &bar[BIN]);
+            bulk_load(sm + OFF_W, a.w_img + static_cast<size_t>(ch) * 16384, 16384, &bar[BIN]);
             bulk_load(sm + OFF_H, a.hs_img + img, 32768, &bar[BIN]);
         }
         token_scalars(a, b, h, r, lane, gc, E, be, tinv, nullptr);
@@ -915,7 +929,7 @@ gdn_bwd_kv128_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
                 prefetch_tokens(&map_v, a, nx);
                 bulk_prefetch_l2(a.dh_img + nimg, 32768);
                 bulk_prefetch_l2(a.u + n64, kC * kD * 4);
-                bulk_prefetch_l2(a.w + n64, kC * kD * 4);
+                bulk_prefetch_l2(a.w_img + static_cast<size_t>(nx) * 16384, 16384);
                 bulk_prefetch_l2(a.qc + n64 / 2, kC * kD * 2);
                 bulk_prefetch_l2(a.tt + static_cast<size_t>(nx) * kC * kC, kC * kC * 4);
                 bulk_prefetch_l2(a.hs_img + nimg, 32768);
@@ -987,8 +1001,6 @@ gdn_bwd_kv128_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
     ld_own16(a.u + t64, tid, u);
     if (tid < kC) pcs[tid] = cs[tid] = db1[tid] = 0.f;
     put16(sm + OFF_U, i, hf, grp, u);
-    ld_own16(a.w + t64, tid, x);
-    put16(sm + OFF_W, i, hf, grp, x);
     {
         float t[8];
         ld_global8(a.tt + static_cast<size_t>(ch) * kC * kC + 8 * tid, t);
@@ -1057,7 +1069,7 @@ gdn_bwd_kv128_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
         put8(sm + OFF_DP, i, hf, grp, p);
         signal_issue(3);
         row_part(red + 768, grp, i, hf, part);
-        col_sums<8>(s, lane);
+        col_sums(s, lane);
         if (!(lane & 1)) atomicAdd(&pcs[s0 + ((lane >> 1) & 7)], s[0]);
     }
     mbar_wait(&bar[B1B], 0, abort_flag, status);
@@ -1097,33 +1109,13 @@ gdn_bwd_kv128_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
         row_part(red + 1024, grp, i, hf, part);
 #pragma unroll
         for (int e = 0; e < 8; ++e) t[e] *= tt[e];
-        col_sums<8>(t, lane);
+        col_sums(t, lane);
         if (!(lane & 1)) atomicAdd(&db1[s0 + ((lane >> 1) & 7)], t[0]);
     }
     compute_sync();
     if (tid == 0) {  // dv is the bf16 tile of dR (signal_issue's fence came before the barrier)
         store_tokens(&map_dv, sm + OFF_D, b, h, r);
         tma_store_commit();
-    }
-    // the reverse sums G_i = sum_{l >= i} (W_l cq_l t_l + qbar_l cz_l) / t_l^2: sixteen rows by shuffle, the
-    // quadrants' totals through segs
-    float g[16];
-    {
-        ld_own16(a.w + t64, tid, g);
-        unpack16(qr, x);
-        const float ti = tinv[i], ct = vec[i] / ti, cz = vec[kC + i], t2 = ti * ti;
-#pragma unroll
-        for (int e = 0; e < 16; ++e) g[e] = (g[e] * ct + x[e] * rq * cz) * t2;
-#pragma unroll
-        for (int o = 1; o < 16; o <<= 1)
-#pragma unroll
-            for (int e = 0; e < 16; ++e) {
-                const float y = __shfl_down_sync(0xffffffffu, g[e], o, 16);
-                if ((lane & 15) + o < 16) g[e] += y;
-            }
-        if ((lane & 15) == 0)
-#pragma unroll
-            for (int e = 0; e < 16; ++e) segs[qd * kD + c0 + e] = g[e];
     }
     // ---- round 3: M2
     mbar_wait(&bar[B2B], 0, abort_flag, status);
@@ -1158,7 +1150,7 @@ gdn_bwd_kv128_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
             stage[i * LS + j] = da[e];
         }
         row_part(red + 256, grp, i, hf, part);
-        col_sums<8>(kk2, lane);
+        col_sums(kk2, lane);
         if (!(lane & 1)) atomicAdd(&cs[s0 + ((lane >> 1) & 7)], kk2[0]);
         tc_fence_before();
         compute_sync();
@@ -1167,14 +1159,13 @@ gdn_bwd_kv128_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
         put8(sm + OFF_DT, i, hf, grp, da);
     }
     signal_issue(3);
-    float dmv[16];
-    ld_global8(a.dm + static_cast<size_t>(ch) * kD + c0, dmv);
-    ld_global8(a.dm + static_cast<size_t>(ch) * kD + c0 + 8, dmv + 8);
+    float dmv[16];  // Dm - c G, then dk
+    {
+        ld_own16(a.w + t64, tid, dmv);  // G (gdn_bwd_local128_kernel)
+        ld_global8(a.dm + static_cast<size_t>(ch) * kD + c0, x);
+        ld_global8(a.dm + static_cast<size_t>(ch) * kD + c0 + 8, x + 8);
 #pragma unroll
-    for (int e = 0; e < 16; ++e) {
-        float off = 0.f;
-        for (int s = qd + 1; s < 4; ++s) off += segs[s * kD + c0 + e];
-        dmv[e] -= cf * (g[e] + off);
+        for (int e = 0; e < 16; ++e) dmv[e] = x[e] - cf * dmv[e];
     }
     // ---- round 5: dk
     mbar_wait(&bar[B5], 0, abort_flag, status);

@@ -100,6 +100,7 @@ struct GdnBwdArgs {
     // chunk): H_r and S^K_r (from the forward), dH (the state pass), DC_{r+1} + DC_{r+1}^T (the suffix)
     const uint8_t *hs_img = nullptr, *sk_img = nullptr;
     uint8_t *dh_img = nullptr, *dcs_img = nullptr;
+    uint8_t *w_img = nullptr;  // W likewise (two T64 tiles of 64 rows, 16 KB); w then holds G, qc the image of Qc
     int *status = nullptr; // status word of the tensor-core products' bounded waits (TC kernels)
     int wave = 0;          // chunk CTAs resident at once: each prefetches into L2 the inputs of the
                            // chunk one wave after its own (ccq_gdn_bwd_chunk_tc.cu)
