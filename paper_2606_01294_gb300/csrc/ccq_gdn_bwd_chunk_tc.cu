@@ -244,7 +244,9 @@ __device__ __forceinline__ void load_parts(const uint8_t *tile, int row, int qtr
 __device__ __forceinline__ float lo_bf16(uint32_t w) { return __uint_as_float(w << 16); }
 __device__ __forceinline__ float hi_bf16(uint32_t w) { return __uint_as_float(w & 0xffff0000u); }
 // 1 / |row| of the raw q (threads 0-255) and k (256-511) tiles: row (tid % 256) / 4, the row's four
-// threads return the same value; w keeps the values read.
+// threads return the same value; w keeps the values read.  ODD_FIRST: the k rows' parts are added odd part of
+// each pair first, the order in which the CUDA-core kv kernel's atomics mostly arrive.
+template <bool ODD_FIRST = false>
 __device__ __forceinline__ float row_norms(const uint8_t *qt, const uint8_t *kt, int tid, int l2norm, uint32_t (&w)[16]) {
     load_parts(tid < 256 ? qt : kt, (tid & 255) >> 2, tid & 3, w);
     float p0 = 0.f, p1 = 0.f;
@@ -253,7 +255,8 @@ __device__ __forceinline__ float row_norms(const uint8_t *qt, const uint8_t *kt,
         p0 = fmaf(lo_bf16(w[c]), lo_bf16(w[c]), p0);
         p1 = fmaf(hi_bf16(w[c]), hi_bf16(w[c]), p1);
     }
-    return gbwd::rnorm_of(parts_total(p0, p1, tid & 31), l2norm);
+    const bool odd = ODD_FIRST && tid >= 256;
+    return gbwd::rnorm_of(parts_total(odd ? p1 : p0, odd ? p0 : p1, tid & 31), l2norm);
 }
 
 // K = 64 or 128 products over T64 tiles.  A and B: descriptors of the first K = 16 step; K-major operands
@@ -1016,7 +1019,7 @@ gdn_bwd_kv128_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
     put16(sm + OFF_D, i, hf, grp, x);
     {
         uint32_t w[16];
-        const float rr = row_norms(sm + OFF_Q, sm + OFF_K, tid, a.l2norm, w);
+        const float rr = row_norms<true>(sm + OFF_Q, sm + OFF_K, tid, a.l2norm, w);
         if ((tid & 3) == 0) rn[tid >> 2] = rr;
     }
     compute_sync();
