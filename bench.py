@@ -68,28 +68,47 @@ KERNEL_NAMES = {"gla": "gla_chunk_kernel", "gdn": "gdn_wy_kernel + gdn_chunk_ker
                           " gdn_bwd_local_kernel + gdn_bwd_state_tc_kernel + gdn_bwd_suffix_kernel + gdn_bwd_kv_kernel"}
 
 
-def gla_segments(B, H, T, sms):
-    """Segments per sequence the library's default split picks (ccq_capi.cu)."""
+def state_segments(B, H, T, sms):
+    """(segments per sequence, chunks per segment) of the Gated DeltaNet forward and of a training
+    step's forwards (split_sequences in ccq_capi.cu)."""
     nc = (T + 63) // 64
     ns = sms // (B * H) if B * H * 2 <= sms else 1
     ns = max(1, min(ns, nc // 8, nc))
     per = (nc + ns - 1) // ns
-    return (nc + per - 1) // per
+    return (nc + per - 1) // per, per
+
+
+def gla_segments(B, H, T, sms):
+    """Segments per sequence the library's default split of a GLA forward picks (split_gla_forward
+    in ccq_capi.cu)."""
+    nc = (T + 63) // 64
+    ns, per = state_segments(B, H, T, sms)
+    if B * H * 2 > sms:
+        return ns
+
+    def cost(n, p):
+        return 42 * nc if n == 1 else 18 * p + 48 * max(p, nc - p * (n - 1)) + 140 + 3 * n
+
+    best = cost(ns, per)
+    for n in range(max(2, ns), sms // (B * H) + 1):
+        for p in (nc // n, (nc + n - 1) // n):
+            if 3 * n <= nc and nc - p * (n - 1) >= 3 and cost(n, p) < best:
+                best, ns = cost(n, p), n
+    return ns
 
 
 def launches_per_step(kind, B, H, T, sms):
-    """Kernel launches of one step: the segmented GLA forward is three kernels, the
-    Gated DeltaNet forward two (WY, chunk) or four when segmented, the backward three,
-    and every call that returns the position count adds the one-thread-per-row count
-    update."""
-    if kind in ("glavl", "gdnvl"):  # one launch (two for GDN: WY, chunk) plus the count update
-        return 2 if kind == "glavl" else 3
-    split = gla_segments(B, H, T, sms) > 1
-    fwd = 3 if split else 1
-    gdn = 4 if split else 2
+    """Kernel launches of one step: a GLA forward is one kernel, or three when its sequences are
+    split, the Gated DeltaNet forward two (WY, chunk) or four; the GLA backward three; the decode step one
+    (the kernels write the position count)."""
+    if kind in ("glavl", "gdnvl"):  # one launch (two for GDN: WY, chunk)
+        return 1 if kind == "glavl" else 2
+    gla = 3 if gla_segments(B, H, T, sms) > 1 else 1
+    train = state_segments(B, H, T, sms)[0] > 1
+    gdn = 4 if train else 2
     # the Gated DeltaNet training step runs the forward twice (the step's forward, then the
     # backward's recompute of the forward's per-chunk quantities) and four backward kernels
-    return {"gla": fwd + 1, "gdn": gdn + 1, "decode": 1 + 1, "glabwd": fwd + 1 + 3, "gdnbwd": 2 * gdn + 1 + 4}[kind]
+    return {"gla": gla, "gdn": gdn, "decode": 1, "glabwd": (3 if train else 1) + 3, "gdnbwd": 2 * gdn + 4}[kind]
 
 
 def algorithmic_bytes(kind, B, H, T, D):

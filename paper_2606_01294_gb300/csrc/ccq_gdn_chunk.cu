@@ -461,8 +461,8 @@ gdn_chunk_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     const size_t rowbase = vl ? static_cast<size_t>(tok0) : static_cast<size_t>(b) * a.T;
     const int NCt = (T + kC - 1) / kC;
     const int cb = a.nseg > 1 ? seg * a.seg_chunks : 0;  // first chunk of this CTA
-    const int NC = a.nseg > 1 ? min(NCt, cb + a.seg_chunks) - cb : NCt;
     const bool last_seg = seg == a.nseg - 1;
+    const int NC = (last_seg ? NCt : cb + a.seg_chunks) - cb;
     // a segment starts from the states its slot of the workspace holds (ccq_gdn_segment.cu)
     const float *segst = a.nseg > 1 ? a.seg_ws + static_cast<size_t>(blockIdx.x) * kGdnSegFloats : nullptr;
     const float *S0 = segst ? segst : a.S0;
@@ -1004,6 +1004,7 @@ gdn_chunk_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
             dmprev[wt] = dmp[wt] + dmp[kD + wt];
             if (wt == 0) mbar_arrive(&bar[BAR_PREP0 + s]);
         }
+        if ((NC > 0 || vl) && a.tT && last_seg && h == 0 && wt == 0) a.tT[b] = (a.t0 ? a.t0[b] : 0) + T;
         if ((NC > 0 || vl) && a.mT && last_seg) {
             const int sl = NC > 0 ? (NC - 1) & 1 : 0;
             a.mT[static_cast<size_t>(bh) * kD + wt] = slot_f(sl, MS_MST)[wt] + dmprev[wt];

@@ -242,8 +242,8 @@ gla_chunk_wide_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_co
     const int T = a.T, H = a.H;
     const int NCt = (T + kC - 1) / kC;
     const int cb = a.nseg > 1 ? seg * a.seg_chunks : 0;  // first chunk of this CTA
-    const int NC = a.nseg > 1 ? min(NCt, cb + a.seg_chunks) - cb : NCt;
     const bool last_seg = seg == a.nseg - 1;
+    const int NC = (last_seg ? NCt : cb + a.seg_chunks) - cb;
     const float *segst = a.nseg > 1 ? a.seg_ws + static_cast<size_t>(blockIdx.x) * kSegFloats : nullptr;
     const float *S0 = segst ? segst : a.S0;
     const float *C0 = segst ? segst + kD * kD : a.C0;
@@ -771,6 +771,7 @@ gla_chunk_wide_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_co
         // represented: report it rather than return silently wrong values
         if (emax > kMaxExp2) atomicExch(status, kStatusRange);
         // final key sum
+        if (NC > 0 && a.tT && last_seg && h == 0 && wt == 0) a.tT[b] = (a.t0 ? a.t0[b] : 0) + T;
         if (NC > 0 && a.mT && last_seg) {
             const int sl = (NC - 1) & 1;
             a.mT[static_cast<size_t>(bh) * kD + wt] = slot_f(sl, MS_MST)[wt] + dmprev[wt];

@@ -63,11 +63,10 @@ gla_segment_state_kernel(const __grid_constant__ CUtensorMap map_k, const __grid
     volatile int *abort_flag = reinterpret_cast<volatile int *>(misc + M_ABORT);
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int seq = blockIdx.x / a.nseg, seg = blockIdx.x % a.nseg;
+    // (no segment starts from the last one's deltas: it has no CTA)
+    const int seq = blockIdx.x / (a.nseg - 1), seg = blockIdx.x % (a.nseg - 1);
     const int b = seq / a.H, h = seq % a.H;
-    const int NCt = (a.T + kC - 1) / kC;
-    const int cb = seg * a.seg_chunks, ce = min(NCt, cb + a.seg_chunks);
-    const int n = ce - cb;  // chunks of this segment (>= 1)
+    const int n = a.seg_chunks, ce = (seg + 1) * n;  // chunks [ce - n, ce)
     const bool gate_f32 = a.gate_dtype != 0;
     const uint32_t g_bytes = gate_f32 ? kC * kD * 4 : kC * kD * 2;
     int *status = a.status;
@@ -210,7 +209,7 @@ gla_segment_state_kernel(const __grid_constant__ CUtensorMap map_k, const __grid
     if (n >= 1) mbar_wait(&bar[2 + ((n - 1) & 1)], ((n - 1) >> 1) & 1, abort_flag, status);
     if (n >= 2) mbar_wait(&bar[2 + ((n - 2) & 1)], ((n - 2) >> 1) & 1, abort_flag, status);
     tc_fence_after();
-    float *out = a.seg_ws + static_cast<size_t>(blockIdx.x) * kSegFloats;
+    float *out = a.seg_ws + (static_cast<size_t>(seq) * a.nseg + seg) * kSegFloats;
     {
         const int lq = warp & 3, ch = warp >> 2;  // 8 warps: lane quadrant, column half
         const int row = 32 * lq + lane;
@@ -273,12 +272,13 @@ gla_segment_combine_kernel(const ChunkArgs a) {
         for (int g = 0; g < kGroup; ++g) {
             if (g < ns) {
                 const float *slot = a.seg_ws + (sq * a.nseg + s0 + g) * kSegFloats;
+                const bool delta = s0 + g + 1 < a.nseg;  // the last segment's is not needed
 #pragma unroll
                 for (int u = 0; u < 4; ++u) {
                     const int e = el[u];
-                    const bool live = e < 2 * kSS + kD;
+                    const bool live = delta && e < 2 * kSS + kD;
                     dv[g][u] = live ? slot[e] : 0.f;
-                    Dv[g][u] = (e < kSS) ? slot[2 * kSS + kD + (e >> 7)] : 1.f;
+                    Dv[g][u] = (delta && e < kSS) ? slot[2 * kSS + kD + (e >> 7)] : 1.f;
                 }
             }
         }
@@ -308,7 +308,7 @@ cudaError_t launch_gla_segments(const ChunkArgs &a, const ChunkMaps &m, cudaStre
         if (e != cudaSuccess) return e;
         attr_set = true;
     }
-    gla_segment_state_kernel<<<a.B * a.H * a.nseg, kThreads, kSmem, s>>>(m.k, m.v, m.g, a);
+    gla_segment_state_kernel<<<a.B * a.H * (a.nseg - 1), kThreads, kSmem, s>>>(m.k, m.v, m.g, a);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     const int nblk = (kSegFloats - kD + kCombineBlock - 1) / kCombineBlock;

@@ -34,9 +34,9 @@ constexpr int kCountHeads = 1 << 16;  // heads a row the upper bits are used for
 cudaError_t launch_recurrent(const RecurrentArgs &a, cudaStream_t s);
 cudaError_t launch_recurrent_block(const RecurrentArgs &a, cudaStream_t s);
 
-// tT[b] = t0[b] + T (t0 NULL: T), one thread per batch row.  The kernels leave
-// the final count to this launch, enqueued after them: tT may alias t0, and
-// every (batch, head) CTA reads t0[b] while it runs.
+// tT[b] = t0[b] + T (t0 NULL: T), one thread per batch row.  Where tT overlaps t0 the kernels leave
+// the final count to this launch, enqueued after them: every (batch, head) CTA reads t0[b] as it
+// starts.  (Elsewhere they write it themselves: a launch less, about 3 us of a call.)
 cudaError_t launch_t_update(const int64_t *t0, int64_t *tT, int B, int T, cudaStream_t s);
 // tT[s] = t0[s] + (cu[s+1] - cu[s]) (t0 NULL: 0 +) for packed sequences (device cu).
 cudaError_t launch_t_update_varlen(const int64_t *t0, int64_t *tT, const int64_t *cu, int num_seqs,
@@ -57,9 +57,10 @@ struct ChunkArgs {
     const int64_t *t0;
     __nv_bfloat16 *o;
     float *ST, *CT, *mT;
+    int64_t *tT = nullptr;  // final position counts the kernel writes (not overlapping t0), or NULL
     int *status;  // device status word (bounded-wait give-ups)
     // sequence segments (long sequences): nseg segments of seg_chunks chunks each
-    // (the last one shorter); seg_ws holds kSegFloats (GLA) or kGdnSegFloats (Gated
+    // (the last one takes the rest); seg_ws holds kSegFloats (GLA) or kGdnSegFloats (Gated
     // DeltaNet) floats per (sequence, segment).
     int nseg = 1;
     int seg_chunks = 0;
