@@ -90,13 +90,12 @@ gdn_segment_state_kernel(const __grid_constant__ CUtensorMap map_k, const __grid
     volatile int *abort_flag = reinterpret_cast<volatile int *>(misc + M_ABORT);
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    // (no segment starts from the last one's states: it has no CTA)
-    const int seq = blockIdx.x / (a.nseg - 1), seg = blockIdx.x % (a.nseg - 1);
+    const int seq = blockIdx.x / a.nst, seg = blockIdx.x % a.nst;
     const int b = seq / a.H, h = seq % a.H;
     const int T = a.T, H = a.H;
     const int NCt = (T + kC - 1) / kC;
-    const int cb = seg * a.seg_chunks;
-    const int n = a.seg_chunks;  // chunks of this segment (>= 1)
+    const int cb = seg * a.st_chunks;
+    const int n = min(a.st_chunks, a.seg_chunks * (a.nseg - 1) - cb);  // chunks of this segment (>= 1)
     const int wrow0 = seq * NCt * kC;                 // first Tb row of this sequence
     int *status = a.status;
 
@@ -414,20 +413,20 @@ gdn_segment_combine_kernel(const ChunkArgs a) {
         qv[0] = q4[0]; qv[1] = q4[1];
         dv[0] = d4[0]; dv[1] = d4[1];
     };
-    load_next(0);
-    for (int s = 0; s < a.nseg; ++s) {
+    // the states entering segment s, over what the state pass left in its slot
+    auto entering = [&](int s) {
         float *slot = a.seg_ws + (sq * a.nseg + s) * kGdnSegFloats;
-        if (s + 1 == a.nseg) {  // nothing follows the last segment: its entering states only
 #pragma unroll
-            for (int u = 0; u < 2; ++u) {
-                *reinterpret_cast<float4 *>(slot + arow * kD + c0 + 4 * u) =
-                    make_float4(hreg[4 * u], hreg[4 * u + 1], hreg[4 * u + 2], hreg[4 * u + 3]);
-                *reinterpret_cast<float4 *>(slot + 2 * kSS + arow * kD + c0 + 4 * u) =
-                    make_float4(creg[4 * u], creg[4 * u + 1], creg[4 * u + 2], creg[4 * u + 3]);
-            }
-            if (cblk == 0 && tid < kD) slot[3 * kSS + tid] = mreg;
-            break;
+        for (int u = 0; u < 2; ++u) {
+            *reinterpret_cast<float4 *>(slot + arow * kD + c0 + 4 * u) =
+                make_float4(hreg[4 * u], hreg[4 * u + 1], hreg[4 * u + 2], hreg[4 * u + 3]);
+            *reinterpret_cast<float4 *>(slot + 2 * kSS + arow * kD + c0 + 4 * u) =
+                make_float4(creg[4 * u], creg[4 * u + 1], creg[4 * u + 2], creg[4 * u + 3]);
         }
+        if (cblk == 0 && tid < kD) slot[3 * kSS + tid] = mreg;
+    };
+    load_next(0);
+    for (int s = 0; s < a.nst; ++s) {
         // stage P_s (element e = 4 (256 u + tid): row e / 128, column e % 128) and H_s
 #pragma unroll
         for (int u = 0; u < 16; ++u) {
@@ -441,7 +440,8 @@ gdn_segment_combine_kernel(const ChunkArgs a) {
         float acc[8] = {qv[0].x, qv[0].y, qv[0].z, qv[0].w, qv[1].x, qv[1].y, qv[1].z, qv[1].w};  // Q_s
         const float dcv[8] = {dv[0].x, dv[0].y, dv[0].z, dv[0].w, dv[1].x, dv[1].y, dv[1].z, dv[1].w};
         __syncthreads();
-        if (s + 2 < a.nseg) load_next(s + 1);
+        if (s + 1 < a.nst) load_next(s + 1);
+        const float dm = cblk == 0 && tid < kD ? a.seg_ws[(sq * a.nseg + s) * kGdnSegFloats + 3 * kSS + tid] : 0.f;
         const float *P = Ps + arow * kPS;
 #pragma unroll 4
         for (int bb = 0; bb < kD; bb += 4) {
@@ -456,31 +456,24 @@ gdn_segment_combine_kernel(const ChunkArgs a) {
                 for (int u = 0; u < 8; ++u) acc[u] = fmaf(pw[t], hv[u], acc[u]);
             }
         }
-        // this slot now holds the states entering segment s
-#pragma unroll
-        for (int u = 0; u < 2; ++u) {
-            *reinterpret_cast<float4 *>(slot + arow * kD + c0 + 4 * u) =
-                make_float4(hreg[4 * u], hreg[4 * u + 1], hreg[4 * u + 2], hreg[4 * u + 3]);
-            *reinterpret_cast<float4 *>(slot + 2 * kSS + arow * kD + c0 + 4 * u) =
-                make_float4(creg[4 * u], creg[4 * u + 1], creg[4 * u + 2], creg[4 * u + 3]);
-        }
+        // (with halves of one chunk segment, nst = nseg = 2, the second half starts no segment)
+        if (s == 0 || a.nst < a.nseg) entering(s);
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
             hreg[u] = acc[u];
             creg[u] += dcv[u];
         }
-        if (cblk == 0 && tid < kD) {
-            const float dm = slot[3 * kSS + tid];
-            slot[3 * kSS + tid] = mreg;
-            mreg += dm;
-        }
+        mreg += dm;
         __syncthreads();  // Ps and hcur are rewritten by the next segment
     }
+    entering(a.nseg - 1);
 }
 
 }  // namespace
 
-cudaError_t launch_gdn_segments(const ChunkArgs &a, const GdnMaps &m, cudaStream_t s) {
+cudaError_t launch_gdn_segments(const ChunkArgs &args, const GdnMaps &m, cudaStream_t s) {
+    ChunkArgs a = args;
+    state_segments(a);
     cudaError_t e = launch_gdn_wy(a, m, s);
     if (e != cudaSuccess) return e;
     static bool attr_set = false;
@@ -490,7 +483,7 @@ cudaError_t launch_gdn_segments(const ChunkArgs &a, const GdnMaps &m, cudaStream
         if (e != cudaSuccess) return e;
         attr_set = true;
     }
-    gdn_segment_state_kernel<<<a.B * a.H * (a.nseg - 1), kThreads, kSmem, s>>>(m.k, m.v, m.tb, a);
+    gdn_segment_state_kernel<<<a.B * a.H * a.nst, kThreads, kSmem, s>>>(m.k, m.v, m.tb, a);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     static bool attr_combine = false;

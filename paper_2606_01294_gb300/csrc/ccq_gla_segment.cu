@@ -7,7 +7,7 @@
 //   second moment  C_out = C_in + dC,  key sum  m_out = m_in + dm  (undecayed, App. B)
 // so three launches replace one long sequential walk:
 //   1. gla_segment_state_kernel: per segment, from a zero state, the deltas
-//      (dS, dC, dm, D) -- no read, no output.  Chunks are visited last to first so
+//      (dS, dC, dm, D) -- no read, no output, and none for the last segment.  Chunks are visited last to first so
 //      each chunk's write is scaled by the decay of the chunks after it and
 //      accumulates straight into TMEM: dS = sum_r (kbar e^{Gtot_r - G} * Dsuf_r)^T V.
 //   2. gla_segment_combine_kernel: per sequence, an exclusive scan over its
@@ -63,10 +63,10 @@ gla_segment_state_kernel(const __grid_constant__ CUtensorMap map_k, const __grid
     volatile int *abort_flag = reinterpret_cast<volatile int *>(misc + M_ABORT);
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    // (no segment starts from the last one's deltas: it has no CTA)
-    const int seq = blockIdx.x / (a.nseg - 1), seg = blockIdx.x % (a.nseg - 1);
+    const int seq = blockIdx.x / a.nst, seg = blockIdx.x % a.nst;
     const int b = seq / a.H, h = seq % a.H;
-    const int n = a.seg_chunks, ce = (seg + 1) * n;  // chunks [ce - n, ce)
+    const int cb = seg * a.st_chunks, ce = min(cb + a.st_chunks, a.seg_chunks * (a.nseg - 1));
+    const int n = ce - cb;  // chunks of this segment (>= 1)
     const bool gate_f32 = a.gate_dtype != 0;
     const uint32_t g_bytes = gate_f32 ? kC * kD * 4 : kC * kD * 2;
     int *status = a.status;
@@ -262,6 +262,27 @@ gla_segment_combine_kernel(const ChunkArgs a) {
         else if (e < 2 * kSS + kD) x = a.m0 ? a.m0[sq * kD + e - 2 * kSS] : 0.f;
         cur[u] = x;
     }
+    if (a.nst == a.nseg) {
+        // two chunk segments, the first in two halves: their deltas in slots 0 and 1
+        float *s0 = a.seg_ws + sq * a.nseg * kSegFloats, *s1 = s0 + kSegFloats;
+        float d0[4], d1[4], D0[4], D1[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int e = el[u];
+            const bool live = e < 2 * kSS + kD;
+            d0[u] = live ? s0[e] : 0.f;
+            d1[u] = live ? s1[e] : 0.f;
+            D0[u] = e < kSS ? s0[2 * kSS + kD + (e >> 7)] : 1.f;
+            D1[u] = e < kSS ? s1[2 * kSS + kD + (e >> 7)] : 1.f;
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            if (el[u] >= 2 * kSS + kD) continue;
+            s0[el[u]] = cur[u];
+            s1[el[u]] = D1[u] * (D0[u] * cur[u] + d0[u]) + d1[u];
+        }
+        return;
+    }
     // segments in groups of kGroup: every load of a group is issued before its scan steps
     // (the loads do not depend on the scan), so the group costs one memory round trip
     constexpr int kGroup = 8;
@@ -300,7 +321,9 @@ gla_segment_combine_kernel(const ChunkArgs a) {
 
 }  // namespace
 
-cudaError_t launch_gla_segments(const ChunkArgs &a, const ChunkMaps &m, cudaStream_t s) {
+cudaError_t launch_gla_segments(const ChunkArgs &args, const ChunkMaps &m, cudaStream_t s) {
+    ChunkArgs a = args;
+    state_segments(a);
     static bool attr_set = false;
     if (!attr_set) {
         cudaError_t e = cudaFuncSetAttribute(gla_segment_state_kernel,
@@ -308,7 +331,7 @@ cudaError_t launch_gla_segments(const ChunkArgs &a, const ChunkMaps &m, cudaStre
         if (e != cudaSuccess) return e;
         attr_set = true;
     }
-    gla_segment_state_kernel<<<a.B * a.H * (a.nseg - 1), kThreads, kSmem, s>>>(m.k, m.v, m.g, a);
+    gla_segment_state_kernel<<<a.B * a.H * a.nst, kThreads, kSmem, s>>>(m.k, m.v, m.g, a);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     const int nblk = (kSegFloats - kD + kCombineBlock - 1) / kCombineBlock;

@@ -65,6 +65,8 @@ struct ChunkArgs {
     int nseg = 1;
     int seg_chunks = 0;
     float *seg_ws = nullptr;
+    // the state pass's own segments (state_segments() of ccq_internal.h): nst of st_chunks chunks, the last shorter
+    int nst = 0, st_chunks = 0;
     // GLA only: when set, the chunk-start states of every chunk are saved for the
     // backward (layout below).  skip_o suppresses the output write (both backbones).
     uint8_t *ckpt = nullptr;
@@ -89,6 +91,16 @@ struct ChunkArgs {
     float *tt_out = nullptr, *hs_out = nullptr, *mk_out = nullptr;
     uint8_t *hs_img = nullptr, *sk_img = nullptr;
 };
+
+// The segments of the state pass, which the chunk kernels' last segment does not need: one for each of the
+// others.  With two chunk segments the pass would leave half the SMs idle, so it cuts the first in two (the
+// second's slot is free until the combine), which compose like any two.  B = 4, H = 16, T = 4096 (32 chunks):
+// GLA 59 -> 31 us, Gated DeltaNet 132 -> 68 us.
+inline void state_segments(ChunkArgs &a) {
+    const bool halves = a.nseg == 2 && a.seg_chunks >= 8;
+    a.nst = halves ? 2 : a.nseg - 1;
+    a.st_chunks = halves ? (a.seg_chunks + 1) / 2 : a.seg_chunks;
+}
 
 // Per (sequence, segment) workspace: S [128][128], C [128][128], m [128], D [128].
 constexpr int kSegFloats = 2 * 128 * 128 + 2 * 128;
