@@ -93,11 +93,11 @@ struct ChunkArgs {
 };
 
 // The segments of the state pass, which the chunk kernels' last segment does not need: one for each of the
-// others.  With two chunk segments the pass would leave half the SMs idle, so it cuts the first in two (the
-// second's slot is free until the combine), which compose like any two.  B = 4, H = 16, T = 4096 (32 chunks):
-// GLA 59 -> 31 us, Gated DeltaNet 132 -> 68 us.
+// others.  With two chunk segments the pass would leave half the SMs idle, so a forward that hands nothing to a
+// backward cuts the first in two (the second's slot is free until the combine), which compose like any two; a
+// backward's forward keeps the order in which one segment's key statistics sum.
 inline void state_segments(ChunkArgs &a) {
-    const bool halves = a.nseg == 2 && a.seg_chunks >= 8;
+    const bool halves = a.nseg == 2 && a.seg_chunks >= 8 && !a.ckpt && !a.skip_o;
     a.nst = halves ? 2 : a.nseg - 1;
     a.st_chunks = halves ? (a.seg_chunks + 1) / 2 : a.seg_chunks;
 }
