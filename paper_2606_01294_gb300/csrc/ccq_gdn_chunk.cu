@@ -433,6 +433,9 @@ __device__ __forceinline__ void img_row32(uint8_t *img, int row, int cc, const u
     }
 }
 
+// STATES: the states entering each chunk for the backward (ChunkArgs::hs_out and the rest), without the CCQ
+// read, the scores and the output: the chain of a chunk is D2, R, DU, U, D6, H's copy.
+template <bool STATES>
 __global__ void __launch_bounds__(kThreads, 1)
 gdn_chunk_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                  const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CUtensorMap map_tb,
@@ -487,15 +490,19 @@ gdn_chunk_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         const int s = r & 1;
         uint8_t *base = sm + s * SLOT_BYTES;
         uint64_t *bb = &bar[BAR_IN0 + s];
-        mbar_arrive_expect_tx(bb, 4 * 8192);
+        mbar_arrive_expect_tx(bb, (STATES ? 2 : 4) * 8192);
         const int tg = (cb + r) * kC;
-        tma_load_4d(base + SO_Q, &map_q, bb, 0, h, tok0 + tg, bt);
-        tma_load_4d(base + SO_Q + 8192, &map_q, bb, 64, h, tok0 + tg, bt);
+        if constexpr (!STATES) {
+            tma_load_4d(base + SO_Q, &map_q, bb, 0, h, tok0 + tg, bt);
+            tma_load_4d(base + SO_Q + 8192, &map_q, bb, 64, h, tok0 + tg, bt);
+        }
         tma_load_4d(base + SO_K, &map_k, bb, 0, h, tok0 + tg, bt);
         tma_load_4d(base + SO_K + 8192, &map_k, bb, 64, h, tok0 + tg, bt);
         if (r + 2 < NC) {  // chunk r + 2 into L2, so that its loads hit there
-            tma_prefetch_l2_4d(&map_q, 0, h, tok0 + tg + 2 * kC, bt);
-            tma_prefetch_l2_4d(&map_q, 64, h, tok0 + tg + 2 * kC, bt);
+            if constexpr (!STATES) {
+                tma_prefetch_l2_4d(&map_q, 0, h, tok0 + tg + 2 * kC, bt);
+                tma_prefetch_l2_4d(&map_q, 64, h, tok0 + tg + 2 * kC, bt);
+            }
             tma_prefetch_l2_4d(&map_k, 0, h, tok0 + tg + 2 * kC, bt);
             tma_prefetch_l2_4d(&map_k, 64, h, tok0 + tg + 2 * kC, bt);
         }
@@ -572,8 +579,8 @@ gdn_chunk_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         const int i = 16 * (warp & 3) + (lane & 15);
         const int hf = lane >> 4;
         const int row = 32 * (warp & 3) + lane;  // state row of the M = 128 layout
-        // (with a.sk_img / a.hs_img the snapshots of chunk ch of this sequence also write the operand
-        // tiles they make to the backward's arrays, with a.hs_out the fp32 H)
+        // (STATES: the snapshots of chunk ch of this sequence write the operand tiles they make, and the fp32
+        // H, to the backward's arrays)
         auto state_img = [&](int ch) { return (static_cast<size_t>(bh) * NCt + ch) * 32768; };
         auto snap_sk = [&](int ch) {
             tc_fence_after();
@@ -584,13 +591,15 @@ gdn_chunk_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
                 uint32_t w[16];
 #pragma unroll
                 for (int e = 0; e < 16; ++e) w[e] = pack_bf16(x[2 * e], x[2 * e + 1]);
-                put_row32(sm + OFF_SK + grp * 16384, row, cc, w);
-                if (a.sk_img) img_row32(a.sk_img + state_img(ch) + grp * 16384, row, cc, w);
+                if constexpr (STATES) img_row32(a.sk_img + state_img(ch) + grp * 16384, row, cc, w);
+                else put_row32(sm + OFF_SK + grp * 16384, row, cc, w);
             }
-            fence_proxy_async_smem();
-            tc_fence_before();
-            named_bar(NB_EPI, kEpiThreads);
-            if (tid == 0) mbar_arrive(&bar[BAR_SNAPK]);
+            if constexpr (!STATES) {
+                fence_proxy_async_smem();
+                tc_fence_before();
+                named_bar(NB_EPI, kEpiThreads);
+                if (tid == 0) mbar_arrive(&bar[BAR_SNAPK]);
+            }
         };
         // bf16 copy of the state H entering the next chunk; the TMEM copy is scaled by that
         // chunk's e^{gC} (hs), onto which D6 accumulates the chunk's write
@@ -600,7 +609,7 @@ gdn_chunk_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
             for (int cc = 0; cc < 2; ++cc) {
                 float x[32];
                 tmem_ld32(tq + TM_S + 64 * grp + 32 * cc, x);
-                if (a.hs_out) {
+                if constexpr (STATES) {
                     float4 *dst = reinterpret_cast<float4 *>(
                         a.hs_out + ((static_cast<size_t>(bh) * NCt + ch) * kD + row) * kD + 64 * grp + 32 * cc);
 #pragma unroll
@@ -616,7 +625,7 @@ gdn_chunk_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
                     x[2 * e + 1] = y.y;
                 }
                 put_row32(sm + OFF_HB + grp * 16384, row, cc, w);
-                if (a.hs_img) img_row32(a.hs_img + state_img(ch) + grp * 16384, row, cc, w);
+                if constexpr (STATES) img_row32(a.hs_img + state_img(ch) + grp * 16384, row, cc, w);
                 tmem_st32(tq + TM_S + 64 * grp + 32 * cc, x);
             }
             tmem_wait_st();
@@ -642,35 +651,37 @@ gdn_chunk_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
             const float qni = slot_f(s, MS_QN)[i];
             const float lt = slot_f(s, MS_LT)[i];
             const float ep = slot_f(s, MS_EP)[i];
-            // ---- W' of the CCQ mean fold
-            mbar_wait(&bar[BAR_GA1], par, abort_flag, status);
-            tc_fence_after();
             float c = 0.f;
-            {
-                float sc[32];
-                tmem_ld16x2_32<32>(tq + TM_SA, sc);
-                float pa[4] = {0.f, 0.f, 0.f, 0.f};
+            if constexpr (!STATES) {
+                // ---- W' of the CCQ mean fold
+                mbar_wait(&bar[BAR_GA1], par, abort_flag, status);
+                tc_fence_after();
+                {
+                    float sc[32];
+                    tmem_ld16x2_32<32>(tq + TM_SA, sc);
+                    float pa[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-                for (int jj = 0; jj < 32; ++jj)
-                    if (32 * hf + jj <= i) pa[jj & 3] += sc[jj];
-                float part = (pa[0] + pa[1]) + (pa[2] + pa[3]);
-                part += __shfl_xor_sync(0xffffffffu, part, 16);
-                const float cq = mqi + rqi * part;
-                c = a.centered ? cq * iti : 0.f;
-                const float cn = c * qni;
+                    for (int jj = 0; jj < 32; ++jj)
+                        if (32 * hf + jj <= i) pa[jj & 3] += sc[jj];
+                    float part = (pa[0] + pa[1]) + (pa[2] + pa[3]);
+                    part += __shfl_xor_sync(0xffffffffu, part, 16);
+                    const float cq = mqi + rqi * part;
+                    c = a.centered ? cq * iti : 0.f;
+                    const float cn = c * qni;
 #pragma unroll
-                for (int q2 = 0; q2 < 2; ++q2) {
-                    float w[8];
+                    for (int q2 = 0; q2 < 2; ++q2) {
+                        float w[8];
 #pragma unroll
-                    for (int e = 0; e < 8; ++e) {
-                        const int jj = 8 * q2 + e;
-                        const float v = grp ? sc[16 + jj] : sc[jj];
-                        w[e] = (32 * hf + 16 * grp + jj <= i) ? v - cn : 0.f;
+                        for (int e = 0; e < 8; ++e) {
+                            const int jj = 8 * q2 + e;
+                            const float v = grp ? sc[16 + jj] : sc[jj];
+                            w[e] = (32 * hf + 16 * grp + jj <= i) ? v - cn : 0.f;
+                        }
+                        store_row_chunk(sm + OFF_WM, i, 4 * hf + 2 * grp + q2, w);
                     }
-                    store_row_chunk(sm + OFF_WM, i, 4 * hf + 2 * grp + q2, w);
                 }
+                fence_proxy_async_smem();  // W' is read by G3, issued with G1 after NB_PO
             }
-            fence_proxy_async_smem();  // W' is read by G3, issued with G1 after NB_PO
             // ---- R = V - e^{gc} Kbar H0: read Kbar H0 out of the P/O accumulator
             // first, freeing it for G1
             mbar_wait(&bar[BAR_GA2], par, abort_flag, status);
@@ -679,7 +690,7 @@ gdn_chunk_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
                 float x[32];
                 tmem_ld16x2_32<32>(tq + TM_PO + 64 * grp, x);  // columns 64 grp + 32 hf ..
                 tc_fence_before();
-                named_bar_arrive(NB_PO, kSyncCount);
+                if constexpr (!STATES) named_bar_arrive(NB_PO, kSyncCount);
                 mbar_wait(&bar[BAR_WU], par, abort_flag, status);  // v of the chunk
                 const uint8_t *vt = sm + OFF_V + grp * 8192;
                 uint8_t *rt = sm + OFF_UB + grp * 8192;
@@ -700,7 +711,7 @@ gdn_chunk_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
             tc_fence_before();
             named_bar_arrive(NB_W, kSyncCount);
             // ---- q_clean (Eq. clean) into the Q tile
-            {
+            if constexpr (!STATES) {
                 uint8_t *qt = slot + SO_Q + grp * 8192;
                 const float *Mst = slot_f(s, MS_MST) + 64 * grp + 32 * hf;
                 uint4 qraw[4];
@@ -744,7 +755,7 @@ gdn_chunk_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
             // gc_i - gc_j (log2 units) of this thread's 16 key columns, and e^{gc} of the rows for
             // the output epilogue, read before the slot is released
             float ev[16];
-            {
+            if constexpr (!STATES) {
                 const float *gcv = slot_f(s, MS_SCAL) + 2;
                 const float gi = gcv[i];
 #pragma unroll
@@ -759,80 +770,84 @@ gdn_chunk_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
                 mbar_wait(&bar[BAR_GK], par, abort_flag, status);
                 snap_sk(cb + r + 1);
             }
-            // ---- Pm_ij = [j<=i] QK_ij e^{gc_i - gc_j} (one exponential of a non-positive argument)
-            mbar_wait(&bar[BAR_GC], par, abort_flag, status);
-            tc_fence_after();
-            {
-                float sc[32];
-                tmem_ld16x2_32<32>(tq + TM_SA, sc);
+            if constexpr (STATES) {
+                mbar_wait(&bar[BAR_GD], par, abort_flag, status);
+            } else {
+                // ---- Pm_ij = [j<=i] QK_ij e^{gc_i - gc_j} (one exponential of a non-positive argument)
+                mbar_wait(&bar[BAR_GC], par, abort_flag, status);
+                tc_fence_after();
+                {
+                    float sc[32];
+                    tmem_ld16x2_32<32>(tq + TM_SA, sc);
 #pragma unroll
-                for (int q2 = 0; q2 < 2; ++q2) {
-                    float w[8];
+                    for (int q2 = 0; q2 < 2; ++q2) {
+                        float w[8];
 #pragma unroll
-                    for (int e = 0; e < 8; ++e) {
-                        const int jj = 8 * q2 + e;
-                        const float v = grp ? sc[16 + jj] : sc[jj];
-                        w[e] = (32 * hf + 16 * grp + jj <= i) ? v * fast_exp2(ev[jj]) : 0.f;
-                    }
-                    store_row_chunk(sm + OFF_WM, i, 4 * hf + 2 * grp + q2, w);
-                }
-            }
-            fence_proxy_async_smem();
-            tc_fence_before();
-            named_bar_arrive(NB_MASK, kSyncCount);
-            // ---- output o_i = e^{gc_i} O1_i + O2_i (q_clean carries the read scale), staged for
-            // the copy warp's TMA store in the slot's Kd tile (its last reader, D6, completed
-            // before GD).  O1^T, O2^T are M = 128 accumulators: this thread holds value column
-            // `row` for the chunk rows 32 grp .. 32 grp + 31.  A lane pair swaps one value per two
-            // rows so that each lane writes a bf16 pair of adjacent columns: the even lane row e,
-            // the odd lane row e + 1 (half the shared-memory stores of one column per thread).
-            named_bar(NB_EPI, kEpiThreads);  // epo of this chunk visible
-            mbar_wait(&bar[BAR_GD], par, abort_flag, status);
-            tc_fence_after();
-            {
-                const bool direct = partial(r), odd = lane & 1;
-                const int c2 = row & ~1;  // first column of this lane's pair
-                // Shared addresses of the pair in tile row 0 + odd for the four swizzle classes of
-                // the even rows (row & 7 = 0, 2, 4, 6); a row adds 128 bytes.
-                const uint32_t ob = smem_addr(slot + SO_KD + (row >> 6) * 8192) + (odd ? 128u : 0u) +
-                                    (static_cast<uint32_t>(c2 & 7) << 1);
-                const uint32_t cx = (static_cast<uint32_t>(c2 & 63) >> 3) ^ (odd ? 1u : 0u);
-                uint32_t bk[4];
-#pragma unroll
-                for (int k = 0; k < 4; ++k) bk[k] = ob + ((cx ^ (2u * k)) << 4);
-#pragma unroll 1
-                for (int hh = 0; hh < 2; ++hh) {
-                    const int i0 = 32 * grp + 16 * hh;
-                    float o1[16], o2[16];
-                    tmem_ld16(tq + TM_O1 + i0, o1);
-                    tmem_ld16(tq + TM_O2 + i0, o2);
-                    const float *ep_r = epo + (r & 1) * 64 + i0;
-                    const uint32_t rb = static_cast<uint32_t>(i0) * 128u;
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        const float4 e4 = *reinterpret_cast<const float4 *>(ep_r + 4 * q);
-                        const float ev4[4] = {e4.x, e4.y, e4.z, e4.w};
-                        float ov[4];
-#pragma unroll
-                        for (int u = 0; u < 4; ++u) ov[u] = fmaf(ev4[u], o1[4 * q + u], o2[4 * q + u]);
-#pragma unroll
-                        for (int u = 0; u < 4; u += 2) {
-                            const float y = __shfl_xor_sync(0xffffffffu, odd ? ov[u] : ov[u + 1], 1);
-                            const uint32_t pr = odd ? pack_bf16(y, ov[u + 1]) : pack_bf16(ov[u], y);
-                            if (!direct) {
-                                st_shared_b32(bk[(2 * q + u / 2) & 3] + rb + (4 * q + u) * 128, pr);
-                            } else {
-                                const int tpos = (cb + r) * kC + i0 + 4 * q + u + (odd ? 1 : 0);
-                                if (tpos < T && !a.skip_o)
-                                    *reinterpret_cast<uint32_t *>(a.o + ((rowbase + tpos) * H + h) * kD + c2) = pr;
-                            }
+                        for (int e = 0; e < 8; ++e) {
+                            const int jj = 8 * q2 + e;
+                            const float v = grp ? sc[16 + jj] : sc[jj];
+                            w[e] = (32 * hf + 16 * grp + jj <= i) ? v * fast_exp2(ev[jj]) : 0.f;
                         }
+                        store_row_chunk(sm + OFF_WM, i, 4 * hf + 2 * grp + q2, w);
                     }
                 }
                 fence_proxy_async_smem();
+                tc_fence_before();
+                named_bar_arrive(NB_MASK, kSyncCount);
+                // ---- output o_i = e^{gc_i} O1_i + O2_i (q_clean carries the read scale), staged for
+                // the copy warp's TMA store in the slot's Kd tile (its last reader, D6, completed
+                // before GD).  O1^T, O2^T are M = 128 accumulators: this thread holds value column
+                // `row` for the chunk rows 32 grp .. 32 grp + 31.  A lane pair swaps one value per two
+                // rows so that each lane writes a bf16 pair of adjacent columns: the even lane row e,
+                // the odd lane row e + 1 (half the shared-memory stores of one column per thread).
+                named_bar(NB_EPI, kEpiThreads);  // epo of this chunk visible
+                mbar_wait(&bar[BAR_GD], par, abort_flag, status);
+                tc_fence_after();
+                {
+                    const bool direct = partial(r), odd = lane & 1;
+                    const int c2 = row & ~1;  // first column of this lane's pair
+                    // Shared addresses of the pair in tile row 0 + odd for the four swizzle classes of
+                    // the even rows (row & 7 = 0, 2, 4, 6); a row adds 128 bytes.
+                    const uint32_t ob = smem_addr(slot + SO_KD + (row >> 6) * 8192) + (odd ? 128u : 0u) +
+                                        (static_cast<uint32_t>(c2 & 7) << 1);
+                    const uint32_t cx = (static_cast<uint32_t>(c2 & 63) >> 3) ^ (odd ? 1u : 0u);
+                    uint32_t bk[4];
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) bk[k] = ob + ((cx ^ (2u * k)) << 4);
+#pragma unroll 1
+                    for (int hh = 0; hh < 2; ++hh) {
+                        const int i0 = 32 * grp + 16 * hh;
+                        float o1[16], o2[16];
+                        tmem_ld16(tq + TM_O1 + i0, o1);
+                        tmem_ld16(tq + TM_O2 + i0, o2);
+                        const float *ep_r = epo + (r & 1) * 64 + i0;
+                        const uint32_t rb = static_cast<uint32_t>(i0) * 128u;
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) {
+                            const float4 e4 = *reinterpret_cast<const float4 *>(ep_r + 4 * q);
+                            const float ev4[4] = {e4.x, e4.y, e4.z, e4.w};
+                            float ov[4];
+#pragma unroll
+                            for (int u = 0; u < 4; ++u) ov[u] = fmaf(ev4[u], o1[4 * q + u], o2[4 * q + u]);
+#pragma unroll
+                            for (int u = 0; u < 4; u += 2) {
+                                const float y = __shfl_xor_sync(0xffffffffu, odd ? ov[u] : ov[u + 1], 1);
+                                const uint32_t pr = odd ? pack_bf16(y, ov[u + 1]) : pack_bf16(ov[u], y);
+                                if (!direct) {
+                                    st_shared_b32(bk[(2 * q + u / 2) & 3] + rb + (4 * q + u) * 128, pr);
+                                } else {
+                                    const int tpos = (cb + r) * kC + i0 + 4 * q + u + (odd ? 1 : 0);
+                                    if (tpos < T)
+                                        *reinterpret_cast<uint32_t *>(a.o + ((rowbase + tpos) * H + h) * kD + c2) = pr;
+                                }
+                            }
+                        }
+                    }
+                    fence_proxy_async_smem();
+                }
+                tc_fence_before();
+                named_bar_arrive(NB_OUT, kSyncCount);
             }
-            tc_fence_before();
-            named_bar_arrive(NB_OUT, kSyncCount);
             // ---- H_{r+1} while G2 of chunk r+1 runs (D3, D6 of chunk r have run: GD follows them)
             if (r + 1 < NC) {
                 mbar_wait(&bar[BAR_PREP0 + (s ^ 1)], ((r + 1) >> 1) & 1, abort_flag, status);
@@ -879,7 +894,7 @@ gdn_chunk_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
             float *scal = slot_f(s, MS_SCAL);
             mbar_wait(&bar[BAR_IN0 + s], sp, abort_flag, status);
             if (r > 0) Mst[wt] = slot_f(s ^ 1, MS_MST)[wt] + dmprev[wt];
-            if (a.mk_out) a.mk_out[(static_cast<size_t>(bh) * NCt + cb + r) * kD + wt] = Mst[wt];
+            if constexpr (STATES) a.mk_out[(static_cast<size_t>(bh) * NCt + cb + r) * kD + wt] = Mst[wt];
             const float lam_cur = lam_reg;
             if (wt < 64) scal[2 + wt] = g_reg;
             {
@@ -1028,7 +1043,7 @@ gdn_chunk_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
             mbar_wait(&bar[BAR_PREP0 + s], sp, abort_flag, status);
             tc_fence_after();
             // G2 Sc = Q Kbar^T (SA is free: the Pm epilogue of chunk r-1 has read it)
-            if (lead && !*abort_flag) {
+            if (!STATES && lead && !*abort_flag) {
                 for (int k = 0; k < 8; ++k) {
                     const uint64_t ko = (k >> 2) * 512 + (k & 3) * 2;
                     mma_bf16(tbase + TM_SA, dQ + ko, dK + ko, ID_64x64_KK, k != 0);
@@ -1046,10 +1061,12 @@ gdn_chunk_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
             __syncwarp();
             // G1 P = Q S^K once Kbar H0 is out of the accumulator, G3 P += W' Kbar (W' is
             // written before NB_PO)
-            named_bar(NB_PO, kSyncCount);
-            mbar_wait(&bar[BAR_SNAPK], par, abort_flag, status);
-            tc_fence_after();
-            if (lead && !*abort_flag) {
+            if constexpr (!STATES) {
+                named_bar(NB_PO, kSyncCount);
+                mbar_wait(&bar[BAR_SNAPK], par, abort_flag, status);
+                tc_fence_after();
+            }
+            if (!STATES && lead && !*abort_flag) {
                 for (int k = 0; k < 8; ++k)
                     mma_bf16(tbase + TM_PO, dQ + (k >> 2) * 512 + (k & 3) * 2,
                              dSK + (k >> 2) * 1024 + (k & 3) * 2, ID_64x128_KK, k != 0);
@@ -1071,6 +1088,15 @@ gdn_chunk_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
             // D4 QK = Qc Kbar^T, D6 X += Kd^T U, D3 O1^T = H0^T Qc^T
             named_bar(NB_QC, kSyncCount);
             tc_fence_after();
+            if constexpr (STATES) {
+                if (lead && !*abort_flag) {
+                    for (int k = 0; k < 4; ++k) mma_bf16(tbase + TM_S, dKDm + k * 128, dUBm + k * 128, ID_128x128_MM, 1);
+                    mma_commit(&bar[BAR_GC2]);
+                    mma_commit(&bar[BAR_GD]);
+                }
+                __syncwarp();
+                continue;
+            }
             if (lead && !*abort_flag) {
                 for (int k = 0; k < 8; ++k) {
                     const uint64_t ko = (k >> 2) * 512 + (k & 3) * 2;
@@ -1111,12 +1137,14 @@ gdn_chunk_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
             if (r + 2 < NC) {
                 mbar_wait(&bar[BAR_GC2], r & 1, abort_flag, status);
                 if (lead && !*abort_flag) issue_in(r + 2);
+                if (STATES && lead) mbar_arrive(&bar[BAR_OST0 + s]);  // D6 has read the Kd tile
                 __syncwarp();
             }
+            if constexpr (STATES) continue;
             named_bar(NB_OUT, kSyncCount);  // O of chunk r staged
             if (lead) {
                 uint8_t *st = sm + s * SLOT_BYTES + SO_KD;
-                if (!partial(r) && !a.skip_o) {
+                if (!partial(r)) {
                     tma_store_4d(&map_o, st, 0, h, tok0 + (cb + r) * kC, bt);
                     tma_store_4d(&map_o, st + 8192, 64, h, tok0 + (cb + r) * kC, bt);
                     tma_store_commit();
@@ -1165,16 +1193,21 @@ cudaError_t launch_gdn_wy(const ChunkArgs &a, const GdnMaps &m, cudaStream_t s) 
 
 namespace ccq {
 
-cudaError_t launch_gdn_chunk_only(const ChunkArgs &a, const GdnMaps &m, cudaStream_t s) {
+template <bool STATES>
+static cudaError_t launch_chunk(const ChunkArgs &a, const GdnMaps &m, cudaStream_t s) {
     static bool attr_set = false;
     if (!attr_set) {
-        cudaError_t e = cudaFuncSetAttribute(gdn_chunk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        cudaError_t e = cudaFuncSetAttribute(gdn_chunk_kernel<STATES>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              static_cast<int>(kSmemBytes));
         if (e != cudaSuccess) return e;
         attr_set = true;
     }
-    gdn_chunk_kernel<<<a.B * a.H * a.nseg, kThreads, kSmemBytes, s>>>(m.q, m.k, m.v, m.tb, m.o, a);
+    gdn_chunk_kernel<STATES><<<a.B * a.H * a.nseg, kThreads, kSmemBytes, s>>>(m.q, m.k, m.v, m.tb, m.o, a);
     return cudaGetLastError();
+}
+
+cudaError_t launch_gdn_chunk_only(const ChunkArgs &a, const GdnMaps &m, cudaStream_t s) {
+    return a.skip_o ? launch_chunk<true>(a, m, s) : launch_chunk<false>(a, m, s);
 }
 
 cudaError_t launch_gdn_chunk(const ChunkArgs &a, const GdnMaps &m, cudaStream_t s) {

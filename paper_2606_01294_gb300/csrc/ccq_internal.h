@@ -68,7 +68,8 @@ struct ChunkArgs {
     // the state pass's own segments (state_segments() of ccq_internal.h): nst of st_chunks chunks, the last shorter
     int nst = 0, st_chunks = 0;
     // GLA only: when set, the chunk-start states of every chunk are saved for the
-    // backward (layout below).  skip_o suppresses the output write (both backbones).
+    // backward (layout below).  skip_o suppresses the output (Gated DeltaNet: with the arrays below, only the
+    // states are formed).
     uint8_t *ckpt = nullptr;
     int skip_o = 0;
     // Packed variable-length sequences (cu != NULL): the batch index b is the sequence, B the
