@@ -83,7 +83,7 @@ struct GdnBwdArgs {
     float *tt;   // [64][64] Tt
     float *sk;   // [D][D]   chunk's Kbar^T Kbar, then S^K_r
     float *mk;   // [D]      chunk's sum Kbar, then M_r
-    float *hs;   // [D][D]   H_r (the state entering the chunk)
+    float *hs;   // [D][D]   H_r (the state entering the chunk); bf16, D = 128: [D / 8][D][8] (ChunkArgs::hs_out)
     float *dh;   // [D][D]   adjoint of H_{r+1} (the state leaving the chunk)
     float *dc;   // [D][D]   chunk's increment of DC, then DC_{r+1}
     float *dm;   // [D]      chunk's increment of Dm, then Dm_{r+1}

@@ -145,12 +145,13 @@ gdn_bwd_state_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_
         const uint32_t bsb = sb + buf * BUF_BYTES;
         float hv[32];  // this thread's part of H_r, in flight until dH_{r+1} is read
         {
-            const float4 *src = reinterpret_cast<const float4 *>(a.hs + (ci * kD + row) * kD + 64 * half + 32 * th);
+            const float *src = a.hs + (ci * 16 + 8 * half + 4 * th) * kD * 8 + row * 8;  // ChunkArgs::hs_out's layout
 #pragma unroll
-            for (int e = 0; e < 8; ++e) {
-                const float4 v = src[e];
-                hv[4 * e] = v.x; hv[4 * e + 1] = v.y; hv[4 * e + 2] = v.z; hv[4 * e + 3] = v.w;
-            }
+            for (int q = 0; q < 4; ++q)
+                asm volatile("ld.global.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                             : "=f"(hv[8 * q]), "=f"(hv[8 * q + 1]), "=f"(hv[8 * q + 2]), "=f"(hv[8 * q + 3]),
+                               "=f"(hv[8 * q + 4]), "=f"(hv[8 * q + 5]), "=f"(hv[8 * q + 6]), "=f"(hv[8 * q + 7])
+                             : "l"(src + q * kD * 8));
         }
         if (it > 0) {
             // chunk r+1's three products are done: dH is updated, the shared tiles and buffer

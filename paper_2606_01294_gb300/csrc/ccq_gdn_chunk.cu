@@ -609,11 +609,14 @@ gdn_chunk_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
             for (int cc = 0; cc < 2; ++cc) {
                 float x[32];
                 tmem_ld32(tq + TM_S + 64 * grp + 32 * cc, x);
-                if constexpr (STATES) {
-                    float4 *dst = reinterpret_cast<float4 *>(
-                        a.hs_out + ((static_cast<size_t>(bh) * NCt + ch) * kD + row) * kD + 64 * grp + 32 * cc);
+                if constexpr (STATES) {  // consecutive rows, 32 bytes each (ChunkArgs::hs_out)
+                    float *dst = a.hs_out + ((static_cast<size_t>(bh) * NCt + ch) * 16 + 8 * grp + 4 * cc) * kD * 8 + row * 8;
 #pragma unroll
-                    for (int e = 0; e < 8; ++e) dst[e] = make_float4(x[4 * e], x[4 * e + 1], x[4 * e + 2], x[4 * e + 3]);
+                    for (int q8 = 0; q8 < 4; ++q8)
+                        asm volatile("st.global.v8.f32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(dst + q8 * kD * 8),
+                                     "f"(x[8 * q8]), "f"(x[8 * q8 + 1]), "f"(x[8 * q8 + 2]), "f"(x[8 * q8 + 3]),
+                                     "f"(x[8 * q8 + 4]), "f"(x[8 * q8 + 5]), "f"(x[8 * q8 + 6]), "f"(x[8 * q8 + 7])
+                                     : "memory");
                 }
                 const uint64_t hs2 = f2_make(hs, hs);
                 uint32_t w[16];

@@ -86,7 +86,7 @@ struct ChunkArgs {
     // Gated DeltaNet, for the backward (no packed sequences): when set, the forward writes per
     // chunk ch = (b H + h) NC + r of every (sequence, head) what the backward reads: in fp32
     // tt_out[ch][64][64] = Tt = (I + A)^{-1} (the WY kernel), and of the states entering the chunk
-    // hs_out[ch][Dk][Dv] = H_r and mk_out[ch][Dk] = M_r (the chunk kernel); and as the byte images of
+    // hs_out[ch][Dv / 8][Dk][8] = H_r and mk_out[ch][Dk] = M_r (the chunk kernel); and as the byte images of
     // its bf16 operand tiles (two T64 tiles of 128 rows, 32 KB a chunk, 32-byte aligned) hs_img = H_r
     // and sk_img = S^K_r.
     float *tt_out = nullptr, *hs_out = nullptr, *mk_out = nullptr;
