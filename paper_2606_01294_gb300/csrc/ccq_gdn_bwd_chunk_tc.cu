@@ -346,6 +346,9 @@ gdn_bwd_local128_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
             for (int i = 0; i < kBars; ++i) mbar_init(&bar[i], 1);
             *abort_flag = 0;
             fence_barrier_init();
+        }
+        grid_wait();
+        if (lane == 0) {
             mbar_arrive_expect_tx(&bar[BTOK], 4 * 16384 + 512);
             load_tokens(sm + OFF_Q, &map_q, &bar[BTOK], b, h, r);
             load_tokens(sm + OFF_K, &map_k, &bar[BTOK], b, h, r);
@@ -460,6 +463,7 @@ gdn_bwd_local128_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
     const int qd = warp & 3, grp = warp >> 2, hf = lane >> 4, i = 16 * qd + (lane & 15);
     const int c0 = 64 * hf + 16 * grp, s0 = 32 * hf + 8 * grp;
     if (warp == 0) tmem_alloc(tmem_slot, 512);
+    grid_wait();
     const bool valid = i < n;
     const size_t row = (static_cast<size_t>(b) * a.T + r * kC + (valid ? i : 0)) * a.H + h;
     __syncthreads();
@@ -844,6 +848,9 @@ gdn_bwd_kv128_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
             for (int i = 0; i < kBars; ++i) mbar_init(&bar[i], 1);
             *abort_flag = 0;
             fence_barrier_init();
+        }
+        grid_wait();
+        if (lane == 0) {
             const size_t img = static_cast<size_t>(ch) * 32768;
             mbar_arrive_expect_tx(&bar[BTOK], 4 * 16384);
             load_tokens(sm + OFF_K, &map_k, &bar[BTOK], b, h, r);
@@ -1000,6 +1007,7 @@ gdn_bwd_kv128_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
     const int qd = warp & 3, grp = warp >> 2, hf = lane >> 4, i = 16 * qd + (lane & 15);
     const int c0 = 64 * hf + 16 * grp, s0 = 32 * hf + 8 * grp;
     if (warp == 0) tmem_alloc(tmem_slot, 512);
+    grid_wait();
     float u[16], x[16];
     ld_own16(a.u + t64, tid, u);
     if (tid < kC) pcs[tid] = cs[tid] = db1[tid] = 0.f;
@@ -1229,6 +1237,7 @@ __global__ void __launch_bounds__(256) gdn_bwd_suffix128_kernel(const GdnBwdArgs
     __shared__ float tile[2][2][32][33];
     const int bh = blockIdx.x / (kSufPairs + 1), pr = blockIdx.x % (kSufPairs + 1), tid = threadIdx.x, NC = a.NC;
     const size_t ch0 = static_cast<size_t>(bh) * NC;
+    grid_wait();
     if (pr == kSufPairs) {
         if (tid >= kD) return;
         float acc = a.dmT ? a.dmT[static_cast<size_t>(bh) * kD + tid] : 0.f;
@@ -1325,13 +1334,12 @@ cudaError_t launch_gdn_local128(const gbwd::GdnBwdArgs &a, cudaStream_t s) {
         !make_f32_rows_map(&x1, a.x1, chunks * kC, kD, 32, kC) ||
         !make_f32_rows_map(&y1, a.y1, chunks * kD, kD, 32, kD) || !make_f32_rows_map(&dc, a.dc, chunks * kD, kD, 32, kD))
         return cudaErrorInvalidValue;
-    gdn_bwd_local128_kernel<<<static_cast<unsigned>(chunks), kAll, lk::kSmem, s>>>(q, k, v, d, dq, x1, y1, dc, a);
-    return cudaGetLastError();
+    return launch_after(gdn_bwd_local128_kernel, static_cast<unsigned>(chunks), kAll, lk::kSmem, s, q, k, v, d, dq, x1, y1,
+                        dc, a);
 }
 
 cudaError_t launch_gdn_suffix128(const gbwd::GdnBwdArgs &a, cudaStream_t s) {
-    gdn_bwd_suffix128_kernel<<<static_cast<unsigned>(a.B * a.H * (kSufPairs + 1)), 256, 0, s>>>(a);
-    return cudaGetLastError();
+    return launch_after(gdn_bwd_suffix128_kernel, static_cast<unsigned>(a.B * a.H * (kSufPairs + 1)), 256, 0, s, a);
 }
 
 cudaError_t launch_gdn_kv128(const gbwd::GdnBwdArgs &a, cudaStream_t s) {
@@ -1346,8 +1354,8 @@ cudaError_t launch_gdn_kv128(const gbwd::GdnBwdArgs &a, cudaStream_t s) {
         !make_token_map(&dv, a.dv, 2, a.B, a.T, a.H, kD, 64, true) ||
         !make_token_map(&dk, a.dk, 2, a.B, a.T, a.H, kD, 64, true))
         return cudaErrorInvalidValue;
-    gdn_bwd_kv128_kernel<<<static_cast<unsigned>(a.B * a.H * a.NC), kAll, kk::kSmem, s>>>(q, k, v, d, dv, dk, a);
-    return cudaGetLastError();
+    return launch_after(gdn_bwd_kv128_kernel, static_cast<unsigned>(a.B * a.H * a.NC), kAll, kk::kSmem, s, q, k, v, d, dv,
+                        dk, a);
 }
 
 }  // namespace ccq

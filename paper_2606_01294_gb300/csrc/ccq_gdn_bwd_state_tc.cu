@@ -103,6 +103,7 @@ gdn_bwd_state_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_
         fence_barrier_init();
     }
     if (warp == 0) tmem_alloc(tmem_slot, kTmemCols);
+    grid_wait();
     __syncthreads();
     tc_fence_after();
     const uint32_t tbase = *tmem_slot;
@@ -369,8 +370,7 @@ cudaError_t launch_gdn_dstate_tc(const gbwd::GdnBwdArgs &a, const void *k, cudaS
         return cudaErrorInvalidValue;
     int *status = device_status_word();
     if (!status) return cudaErrorInvalidValue;
-    gdn_bwd_state_tc_kernel<<<a.B * a.H * 2, kThreads, kSmem, s>>>(mk, mx, my, a, status);
-    return cudaGetLastError();
+    return launch_after(gdn_bwd_state_tc_kernel, a.B * a.H * 2, kThreads, kSmem, s, mk, mx, my, a, status);
 }
 
 }  // namespace ccq

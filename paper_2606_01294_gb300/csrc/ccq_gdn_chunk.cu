@@ -481,6 +481,7 @@ gdn_chunk_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         fence_barrier_init();
     }
     if (warp == 0) tmem_alloc(tmem_slot, kTmemCols);
+    grid_wait();
     __syncthreads();
     tc_fence_after();
     const uint32_t tbase = *tmem_slot;
@@ -1205,8 +1206,8 @@ static cudaError_t launch_chunk(const ChunkArgs &a, const GdnMaps &m, cudaStream
         if (e != cudaSuccess) return e;
         attr_set = true;
     }
-    gdn_chunk_kernel<STATES><<<a.B * a.H * a.nseg, kThreads, kSmemBytes, s>>>(m.q, m.k, m.v, m.tb, m.o, a);
-    return cudaGetLastError();
+    // after the WY kernel, or the combine of the segments' states
+    return launch_after(gdn_chunk_kernel<STATES>, a.B * a.H * a.nseg, kThreads, kSmemBytes, s, m.q, m.k, m.v, m.tb, m.o, a);
 }
 
 cudaError_t launch_gdn_chunk_only(const ChunkArgs &a, const GdnMaps &m, cudaStream_t s) {

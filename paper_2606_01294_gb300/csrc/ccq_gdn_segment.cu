@@ -105,6 +105,7 @@ gdn_segment_state_kernel(const __grid_constant__ CUtensorMap map_k, const __grid
         fence_barrier_init();
     }
     if (warp == 0) tmem_alloc(tslot, 512);
+    grid_wait();
     __syncthreads();
     tc_fence_after();
     const uint32_t tbase = *tslot;
@@ -381,6 +382,7 @@ constexpr int kCombineSmem = (kD * kPS + kD * kCols) * 4;
 __global__ void __launch_bounds__(256)
 gdn_segment_combine_kernel(const ChunkArgs a) {
     extern __shared__ float csm[];
+    grid_wait();
     float *Ps = csm;               // [128][kPS]
     float *hcur = csm + kD * kPS;  // [128][16]
     const int nblk = kD / kCols;
@@ -483,8 +485,7 @@ cudaError_t launch_gdn_segments(const ChunkArgs &args, const GdnMaps &m, cudaStr
         if (e != cudaSuccess) return e;
         attr_set = true;
     }
-    gdn_segment_state_kernel<<<a.B * a.H * a.nst, kThreads, kSmem, s>>>(m.k, m.v, m.tb, a);
-    e = cudaGetLastError();
+    e = launch_after(gdn_segment_state_kernel, a.B * a.H * a.nst, kThreads, kSmem, s, m.k, m.v, m.tb, a);
     if (e != cudaSuccess) return e;
     static bool attr_combine = false;
     if (!attr_combine) {
@@ -493,8 +494,7 @@ cudaError_t launch_gdn_segments(const ChunkArgs &args, const GdnMaps &m, cudaStr
         if (e != cudaSuccess) return e;
         attr_combine = true;
     }
-    gdn_segment_combine_kernel<<<a.B * a.H * (kD / kCols), 256, kCombineSmem, s>>>(a);
-    e = cudaGetLastError();
+    e = launch_after(gdn_segment_combine_kernel, a.B * a.H * (kD / kCols), 256, kCombineSmem, s, a);
     if (e != cudaSuccess) return e;
     return launch_gdn_chunk_only(a, m, s);
 }

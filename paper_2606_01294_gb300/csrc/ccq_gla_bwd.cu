@@ -713,6 +713,7 @@ gla_bwd_state_kernel(const __grid_constant__ CUtensorMap map_qg, const __grid_co
         fence_barrier_init();
     }
     if (warp == 0) tmem_alloc(tmem_slot, 128);
+    grid_wait();
     __syncthreads();
     tc_fence_after();
     const uint32_t tbase = *tmem_slot;
@@ -950,6 +951,7 @@ gla_bwd_kv_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
         tma_load_4d(sm + OFF_KD, &map_g, ba, 0, h, c0, b);
     }
     if (warp == 0) tmem_alloc(tmem_slot, 512);
+    grid_wait();
     __syncthreads();
     if (warp == kLoadWarp) {
         if (lane == 0) {
@@ -1195,11 +1197,10 @@ cudaError_t launch_gla_bwd(const BwdArgs &a, const BwdMaps &m, cudaStream_t s) {
                                                           m.dzr, a);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    gla_bwd_state_kernel<<<a.B * a.H * 2, kThreads, st::kSmem, s>>>(m.qg, m.dO, m.dzr, m.q, a);
-    e = cudaGetLastError();
+    e = launch_after(gla_bwd_state_kernel, a.B * a.H * 2, kThreads, st::kSmem, s, m.qg, m.dO, m.dzr, m.q, a);
     if (e != cudaSuccess) return e;
-    gla_bwd_kv_kernel<<<chunks, kThreadsLoad, kv::kSmem, s>>>(m.k, m.v, m.dO, m.g, m.qg, m.dkc, m.gq, m.dk, m.dv, a);
-    return cudaGetLastError();
+    return launch_after(gla_bwd_kv_kernel, chunks, kThreadsLoad, kv::kSmem, s, m.k, m.v, m.dO, m.g, m.qg, m.dkc, m.gq,
+                        m.dk, m.dv, a);
 }
 
 }  // namespace ccq

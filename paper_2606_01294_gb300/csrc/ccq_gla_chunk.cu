@@ -210,6 +210,7 @@ gla_chunk_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         fence_barrier_init();
     }
     if (warp == 0) tmem_alloc(tmem_slot, kTmemCols);
+    grid_wait();
     __syncthreads();
     tc_fence_after();
     const uint32_t tbase = *tmem_slot;
@@ -915,6 +916,9 @@ cudaError_t launch_gla_chunk(const ChunkArgs &a, const ChunkMaps &m, cudaStream_
     // without checkpoints (4K: 268 -> 253 us) and slower with segments or checkpoint copies.
     if (a.nseg == 1 && a.ckpt == nullptr)
         gla_chunk_kernel<true><<<a.B * a.H, kThreadsCopy, kSmemBytes, s>>>(m.q, m.k, m.v, m.g, m.o, a);
+    else if (a.nseg > 1)  // after the combine of the segments' states
+        return launch_after(gla_chunk_kernel<false>, a.B * a.H * a.nseg, kThreadsNoCopy, kSmemBytes, s, m.q, m.k, m.v,
+                            m.g, m.o, a);
     else
         gla_chunk_kernel<false><<<a.B * a.H * a.nseg, kThreadsNoCopy, kSmemBytes, s>>>(m.q, m.k, m.v, m.g, m.o, a);
     return cudaGetLastError();

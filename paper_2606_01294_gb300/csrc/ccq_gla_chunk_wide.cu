@@ -257,6 +257,7 @@ gla_chunk_wide_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_co
         fence_barrier_init();
     }
     if (warp == 0) tmem_alloc(tmem_slot, kTmemCols);
+    grid_wait();
     __syncthreads();
     tc_fence_after();
     const uint32_t tbase = *tmem_slot;

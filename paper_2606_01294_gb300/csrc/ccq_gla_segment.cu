@@ -250,6 +250,7 @@ gla_segment_combine_kernel(const ChunkArgs a) {
     const int seq = blockIdx.x / nblk, blk = blockIdx.x % nblk;
     const size_t sq = static_cast<size_t>(seq);
     constexpr int kSS = kD * kD;  // S block, then C block, then m
+    grid_wait();
     float cur[4];
     int el[4];
 #pragma unroll
@@ -335,8 +336,7 @@ cudaError_t launch_gla_segments(const ChunkArgs &args, const ChunkMaps &m, cudaS
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     const int nblk = (kSegFloats - kD + kCombineBlock - 1) / kCombineBlock;
-    gla_segment_combine_kernel<<<a.B * a.H * nblk, 256, 0, s>>>(a);
-    e = cudaGetLastError();
+    e = launch_after(gla_segment_combine_kernel, a.B * a.H * nblk, 256, 0, s, a);
     if (e != cudaSuccess) return e;
     return launch_gla_chunk(a, m, s);
 }
