@@ -47,10 +47,10 @@
 //   gla_bwd_kv_kernel    one CTA per chunk (parallel): dk (write part, the
 //                        CCQ inter term K (DC + DC^T), Dm), dv, dgk.
 // 64-row products are M = 64 MMAs whose rows 16q..16q+15 sit in TMEM lanes
-// 32q..32q+15, so in the chunk-parallel kernels (256 compute threads, two warps
-// per lane quadrant, plus a warp that issues the input copies) thread (warp w,
+// 32q..32q+15, so in the chunk-parallel kernels (two or four compute warps per
+// lane quadrant, plus a warp that issues the input copies) thread (warp w,
 // lane l) owns row 16 (w % 4) + l % 16, column half l / 16 of a 64-column load,
-// and -- for 128-column products -- the 32-column slice w / 4 of each half; in
+// and -- for 128-column products -- slice w / 4 (32 or 16 columns) of each half; in
 // the state pass (256 threads) thread t owns state row t % 128 and the 32-column
 // slice t / 128 of its CTA's column half.
 #include <cuda.h>
@@ -68,18 +68,22 @@ namespace {
 constexpr int kC = 64;
 constexpr int kD = 128;
 constexpr int kThreads = 256;     // the state pass: two warps per TMEM lane quadrant
-constexpr int kThreadsPar = 256;  // the chunk-parallel kernels: two warps per TMEM lane quadrant,
-constexpr int kLoadWarp = kThreadsPar / 32;       // then one warp that issues the input copies
-constexpr int kThreadsLoad = kThreadsPar + 32;
-// Barrier of the kThreadsPar compute threads (the load warp leaves once its copies are issued).
-__device__ __forceinline__ void compute_sync() { named_bar(1, kThreadsPar); }
+// The chunk-parallel kernels: compute threads (q: two warps per TMEM lane quadrant, kv: four), then one warp that
+// issues the input copies.  Device times of a training step at B = 4, H = 16, T = 4096: q 264 us with two, 279
+// with four (its row sums, whose order the bf16 roundings of c1 and cz hang on, are done twice or in turn); kv 253
+// with two, 240 with four.
+constexpr int kThreadsQ = 256, kThreadsKv = 512;
+// Barrier of the compute threads (the load warp leaves once its copies are issued).
+template <int THREADS>
+__device__ __forceinline__ void compute_sync() {
+    named_bar(1, THREADS);
+}
 constexpr float kLog2e = 1.4426950408889634f;
 
 constexpr uint32_t ID_64x64_KK = make_idesc(64, 64, 0, 0);
 constexpr uint32_t ID_64x128_KK = make_idesc(64, 128, 0, 0);
 constexpr uint32_t ID_64x128_KM = make_idesc(64, 128, 0, 1);
 constexpr uint32_t ID_64x128_MM = make_idesc(64, 128, 1, 1);
-constexpr uint32_t ID_128x128_MM = make_idesc(128, 128, 1, 1);
 constexpr uint32_t ID_128x64_MK = make_idesc(128, 64, 1, 0);
 
 __device__ __forceinline__ void store_row_chunk(uint8_t *tile, int row, int chunk, const float *w) {
@@ -91,22 +95,19 @@ __device__ __forceinline__ void store_row_chunk(uint8_t *tile, int row, int chun
     *reinterpret_cast<uint4 *>(tile + t64_chunk(row, chunk)) = u;
 }
 
-__device__ __forceinline__ void load_row_chunk(const uint8_t *tile, int row, int chunk, float (&f)[8]) {
-    unpack_bf16x8(*reinterpret_cast<const uint4 *>(tile + t64_chunk(row, chunk)), f);
-}
-
-// Chunk preparation of the chunk-parallel kernels (all 256 threads).  Normalises
-// the k rows (and the q rows when q_tile is set) of the chunk in place -- two
-// threads per row for q and k, four for k alone -- and turns the raw gates
+// Chunk preparation of the chunk-parallel kernels (all compute threads).  Normalises
+// the k rows (and the q rows when q_tile is set) of the chunk in place -- 256
+// threads, two per row for q and k, four for k alone -- and turns the raw gates
 // landed at kd_tile (a plain [64][128] array, bf16 or fp32; the fp32 one also
 // covers eg_tile) into the tiles Kd = kbar e^{Gmid-G} and EG = e^{G-Gmid} (G the
 // in-chunk cumulative log gate over token quarters, gq4 a [4][128] scratch; Gmid
 // its value after token 31).  Outputs per row: rq (1/|q|), mq (M_r . qbar),
 // rk (1/|k|); per key dim (when non-null): f = e^{Gc-Gmid}, emid = e^{Gmid}.
+template <int THREADS>
 __device__ void prep_chunk(uint8_t *q_tile, uint8_t *k_tile, uint8_t *kd_tile, uint8_t *eg_tile,
                               bool gate_f32, bool l2norm, const float *Mr, float *rq, float *mq, float *rk,
                               float *gq4, float *f, float *emid, int pt) {
-    {
+    if (pt < 256) {
         const int tpr = q_tile ? 2 : 4;  // threads per row
         const int rr = pt / tpr, part = pt % tpr;
         const bool isq = q_tile != nullptr && rr < 64;
@@ -167,23 +168,34 @@ __device__ void prep_chunk(uint8_t *q_tile, uint8_t *k_tile, uint8_t *kd_tile, u
             }
         }
     }
-    compute_sync();
-    const int p = pt & 63, qt = pt >> 6, d0 = 2 * p;
-    uint64_t g2[16];  // cumulative gates of dims d0, d0 + 1 as fp32 pairs
+    // A thread takes two dims of a token quarter, with 512 threads half of the quarter's rows: rows 0 - 7, or rows
+    // 8 - 15 and the sums (beside the norms of the first 256).
+    constexpr int kRows = 16 * 256 / THREADS;
+    if (THREADS == 256) compute_sync<THREADS>();
+    const int p = pt & 63, qt = (pt >> 6) & 3, d0 = 2 * p, row0 = 16 * qt + (pt >> 8) * kRows;
+    const bool sums = THREADS == 256 || pt >= 256;
+    uint64_t g2[kRows];  // cumulative gates of dims d0, d0 + 1 as fp32 pairs
     uint64_t r2 = 0;
+    auto gate = [&](int j) {
+        return gate_f32 ? *reinterpret_cast<const uint64_t *>(kd_tile + (j * kD + d0) * 4)
+                        : f2_from_bf16x2(*reinterpret_cast<const uint32_t *>(kd_tile + (j * kD + d0) * 2));
+    };
+    if (THREADS > 256 && sums) {
 #pragma unroll
-    for (int jj = 0; jj < 16; ++jj) {
-        const int j = 16 * qt + jj;
-        const uint64_t x2 = gate_f32 ? *reinterpret_cast<const uint64_t *>(kd_tile + (j * kD + d0) * 4)
-                                     : f2_from_bf16x2(*reinterpret_cast<const uint32_t *>(kd_tile + (j * kD + d0) * 2));
-        r2 = f2_add(r2, x2);
+        for (int jj = 0; jj < kRows; ++jj) r2 = f2_add(r2, gate(16 * qt + jj));
+    }
+#pragma unroll
+    for (int jj = 0; jj < kRows; ++jj) {
+        r2 = f2_add(r2, gate(row0 + jj));
         g2[jj] = r2;
     }
     const float2 rv = f2_split(r2);
     const float r0 = rv.x, r1 = rv.y;
-    gq4[qt * kD + d0] = r0;
-    gq4[qt * kD + d0 + 1] = r1;
-    compute_sync();  // every raw gate read, quarter sums visible
+    if (sums) {
+        gq4[qt * kD + d0] = r0;
+        gq4[qt * kD + d0 + 1] = r1;
+    }
+    compute_sync<THREADS>();  // every row normalised, every raw gate read, quarter sums visible
     float off0 = 0.f, off1 = 0.f;
 #pragma unroll
     for (int q = 0; q < 3; ++q)
@@ -194,7 +206,7 @@ __device__ void prep_chunk(uint8_t *q_tile, uint8_t *k_tile, uint8_t *kd_tile, u
     const float gm0 = gq4[d0] + gq4[kD + d0], gm1 = gq4[d0 + 1] + gq4[kD + d0 + 1];  // Gmid
     const uint64_t o2 = f2_make((off0 - gm0) * kLog2e, (off1 - gm1) * kLog2e);
     const uint64_t l2e = f2_make(kLog2e, kLog2e);
-    if (qt == 3) {
+    if (qt == 3 && sums) {
         if (f) {
             f[d0] = fast_exp2((off0 + r0 - gm0) * kLog2e);
             f[d0 + 1] = fast_exp2((off1 + r1 - gm1) * kLog2e);
@@ -205,13 +217,13 @@ __device__ void prep_chunk(uint8_t *q_tile, uint8_t *k_tile, uint8_t *kd_tile, u
         }
     }
     const uint32_t tcol = (d0 >> 6) * 8192;
-    uint32_t kraw[16];  // every k pair before any tile store
+    uint32_t kraw[kRows];  // every k pair before any tile store
 #pragma unroll
-    for (int jj = 0; jj < 16; ++jj)
-        kraw[jj] = *reinterpret_cast<const uint32_t *>(k_tile + tcol + t64_offset(16 * qt + jj, d0 & 63));
+    for (int jj = 0; jj < kRows; ++jj)
+        kraw[jj] = *reinterpret_cast<const uint32_t *>(k_tile + tcol + t64_offset(row0 + jj, d0 & 63));
 #pragma unroll
-    for (int jj = 0; jj < 16; ++jj) {
-        const int j = 16 * qt + jj;
+    for (int jj = 0; jj < kRows; ++jj) {
+        const int j = row0 + jj;
         const uint32_t off = tcol + t64_offset(j, d0 & 63);
         const float2 x = f2_split(f2_fma(g2[jj], l2e, o2));
         *reinterpret_cast<uint32_t *>(kd_tile + off) =
@@ -219,14 +231,15 @@ __device__ void prep_chunk(uint8_t *q_tile, uint8_t *k_tile, uint8_t *kd_tile, u
         *reinterpret_cast<uint32_t *>(eg_tile + off) = pack_bf16(fast_exp2(x.x), fast_exp2(x.y));
     }
     fence_proxy_async_smem();
-    compute_sync();
+    compute_sync<THREADS>();
 }
 
-// Masked row of a 64 x 64 score tile: w_j = [j <= i] (sc_j - c) for the 32
-// columns [32 hf, 32 hf + 32) this thread holds; also returns the masked sum.
+// Masked row of a 64 x 64 score tile: w_j = [j <= i] (sc_j - c) for NQ times 8 of the 32 columns
+// [32 hf, 32 hf + 32) this thread holds, from 8 FIRST on.
+template <int FIRST = 0, int NQ = 4>
 __device__ __forceinline__ void masked_row(uint8_t *tile, int i, int hf, const float (&sc)[32], float c) {
 #pragma unroll
-    for (int q4 = 0; q4 < 4; ++q4) {
+    for (int q4 = FIRST; q4 < FIRST + NQ; ++q4) {
         float w[8];
 #pragma unroll
         for (int e = 0; e < 8; ++e) {
@@ -235,6 +248,21 @@ __device__ __forceinline__ void masked_row(uint8_t *tile, int i, int hf, const f
         }
         store_row_chunk(tile, i, 4 * hf + q4, w);
     }
+}
+
+// Columns [c, c + 16) (lanes 0-15) and [c + 64, c + 80) (lanes 16-31) of a 64-row product.
+__device__ __forceinline__ void acc_ld16(uint32_t taddr, float (&v)[16]) {
+    uint32_t r[16];
+    asm volatile(
+        "tcgen05.ld.sync.aligned.16x32bx2.x16.b32 "
+        "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16], 64;\n\t"
+        "tcgen05.wait::ld.sync.aligned;"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+          "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+        : "r"(taddr)
+        : "memory");
+#pragma unroll
+    for (int e = 0; e < 16; ++e) v[e] = __uint_as_float(r[e]);
 }
 
 __device__ __forceinline__ float masked_sum(int i, int hf, const float (&sc)[32]) {
@@ -274,7 +302,7 @@ static_assert(M_BAR + 8 * kBars <= M_TMEM, "barriers reach the TMEM slot");
 constexpr uint32_t TM_SC = 0, TM_T1 = 64, TM_Z = 128, TM_DQ = 256;
 }  // namespace qk
 
-__global__ void __launch_bounds__(kThreadsLoad, 1)
+__global__ void __launch_bounds__(kThreadsQ + 32, 1)
 gla_bwd_q_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                  const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CUtensorMap map_do,
                  const __grid_constant__ CUtensorMap map_g, const __grid_constant__ CUtensorMap map_dq,
@@ -319,7 +347,7 @@ gla_bwd_q_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     // (q, k, gates, M_r), then, once the compute threads are released, the rest, which
     // lands while that preparation runs.  Issuing stalls as the copy engine fills, so no
     // compute thread waits for it.
-    if (warp == kLoadWarp && lane == 0) {
+    if (warp == kThreadsQ / 32 && lane == 0) {
         for (int i = 0; i < kBars; ++i) mbar_init(&bar[i], 1);
         *abort_flag = 0;
         fence_barrier_init();
@@ -334,8 +362,8 @@ gla_bwd_q_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         bulk_load(misc + M_MR, rec + 65536, 512, ba);
     }
     if (warp == 0) tmem_alloc(tmem_slot, 512);
-    if (tid < kThreadsPar)
-        for (int e = tid; e < 8192 / 16; e += kThreadsPar)
+    if (tid < kThreadsQ)
+        for (int e = tid; e < 8192 / 16; e += kThreadsQ)
             reinterpret_cast<uint4 *>(sm + OFF_BC)[e] = make_uint4(0u, 0u, 0u, 0u);
     if (tid < kC) {
         const int n = c0 + tid;
@@ -343,7 +371,7 @@ gla_bwd_q_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         itauv[tid] = 1.f / static_cast<float>(tseq0 + n + 1);
     }
     __syncthreads();
-    if (warp == kLoadWarp) {
+    if (warp == kThreadsQ / 32) {
         if (lane == 0) {
             uint64_t *bb = &bar[BAR_INB];
             tma_load_4d(sm + OFF_V, &map_v, bb, 0, h, c0, b);
@@ -390,7 +418,7 @@ gla_bwd_q_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     const uint64_t dBC = make_desc(sb + OFF_BC, 16, 1024);
 
     mbar_wait(&bar[BAR_IN], 0, abort_flag, status);
-    prep_chunk(sm + OFF_Q, sm + OFF_K, sm + OFF_KD, sm + OFF_EG, gate_f32, a.l2norm, Mr, rqv, mqv, rkv, gq4,
+    prep_chunk<kThreadsQ>(sm + OFF_Q, sm + OFF_K, sm + OFF_KD, sm + OFF_EG, gate_f32, a.l2norm, Mr, rqv, mqv, rkv, gq4,
                fv, emv, tid);
     mbar_wait(&bar[BAR_INB], 0, abort_flag, status);
     tc_fence_before();
@@ -434,7 +462,7 @@ gla_bwd_q_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     }
     fence_proxy_async_smem();
     tc_fence_before();
-    compute_sync();
+    compute_sync<kThreadsQ>();
     if (tid == 0 && !*abort_flag) {
         tc_fence_after();
         for (int k = 0; k < 4; ++k)  // Zi += W2 Kbar, Dq += P1 Kd
@@ -506,7 +534,7 @@ gla_bwd_q_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
             red[grp * 128 + i] = dl;
             red[grp * 128 + 64 + i] = mdz;
         }
-        compute_sync();
+        compute_sync<kThreadsQ>();
         if (grp == 0 && hf == 0) {
             dl = red[i] + red[128 + i];
             mdzv[i] = red[64 + i] + red[192 + i];
@@ -516,7 +544,7 @@ gla_bwd_q_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     }
     fence_proxy_async_smem();
     tc_fence_before();
-    compute_sync();
+    compute_sync<kThreadsQ>();
     if (tid == 0 && !*abort_flag) {
         tma_store_4d(&map_qg, sm + OFF_V, 0, h, c0, b);
         tma_store_4d(&map_qg, sm + OFF_V + 8192, 64, h, c0, b);
@@ -556,7 +584,7 @@ gla_bwd_q_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     }
     fence_proxy_async_smem();
     tc_fence_before();
-    compute_sync();
+    compute_sync<kThreadsQ>();
     if (tid == 0 && !*abort_flag) {
         tc_fence_after();
         for (int k = 0; k < 4; ++k)  // u += W3 Kbar
@@ -621,7 +649,7 @@ gla_bwd_q_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
 #pragma unroll
             for (int q4 = 0; q4 < 4; ++q4) store_row_chunk(kt, i, 4 * h2 + q4, x + 8 * q4);
         }
-        compute_sync();
+        compute_sync<kThreadsQ>();
         dot = red[i] + red[128 + i];
         const uint64_t ndot = f2_make(-dot, -dot), rq2 = f2_make(rq, rq);
 #pragma unroll
@@ -640,7 +668,7 @@ gla_bwd_q_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     }
     fence_proxy_async_smem();
     tc_fence_before();
-    compute_sync();
+    compute_sync<kThreadsQ>();
     if (tid == 0 && !*abort_flag) {
         tma_store_4d(&map_dq, sm + OFF_Q, 0, h, c0, b);
         tma_store_4d(&map_dq, sm + OFF_Q + 8192, 64, h, c0, b);
@@ -650,7 +678,7 @@ gla_bwd_q_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         tma_store_wait_read();  // shared memory outlives the stores' reads
     }
     tc_fence_before();
-    compute_sync();
+    compute_sync<kThreadsQ>();
     if (warp == 0) {
         tc_fence_after();
         tmem_dealloc(tbase, 512);
@@ -908,7 +936,7 @@ static_assert(M_BAR + 8 * kBars <= M_TMEM, "barriers reach the TMEM slot");
 constexpr uint32_t TM_KC = 0, TM_T1 = 128, TM_SA = 192, TM_DK = 256, TM_DV = 384;
 }  // namespace kv
 
-__global__ void __launch_bounds__(kThreadsLoad, 1)
+__global__ void __launch_bounds__(kThreadsKv + 32, 1)
 gla_bwd_kv_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
                   const __grid_constant__ CUtensorMap map_do, const __grid_constant__ CUtensorMap map_g,
                   const __grid_constant__ CUtensorMap map_qg, const __grid_constant__ CUtensorMap map_dkc,
@@ -922,7 +950,7 @@ gla_bwd_kv_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
     float *vec = reinterpret_cast<float *>(misc + M_VEC);
     float *rkv = reinterpret_cast<float *>(misc + M_RK);
     float *gq4 = reinterpret_cast<float *>(misc + M_GQ4);
-    float *red = reinterpret_cast<float *>(misc + M_RED);  // [2 groups][128] partial sums
+    float *red = reinterpret_cast<float *>(misc + M_RED);  // partial sums: [4][64], then [2][128]
     float *dG = reinterpret_cast<float *>(sm + OFF_DG);
     uint64_t *bar = reinterpret_cast<uint64_t *>(misc + M_BAR);
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(misc + M_TMEM);
@@ -939,7 +967,7 @@ gla_bwd_kv_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
 
     // The load warp issues k and the gates (the row norms and the gate prefix) first, then,
     // once the compute threads are released, the rest.
-    if (warp == kLoadWarp && lane == 0) {
+    if (warp == kThreadsKv / 32 && lane == 0) {
         for (int i = 0; i < kBars; ++i) mbar_init(&bar[i], 1);
         *abort_flag = 0;
         fence_barrier_init();
@@ -953,7 +981,7 @@ gla_bwd_kv_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
     if (warp == 0) tmem_alloc(tmem_slot, 512);
     grid_wait();
     __syncthreads();
-    if (warp == kLoadWarp) {
+    if (warp == kThreadsKv / 32) {
         if (lane == 0) {
             uint64_t *bb = &bar[BAR_INB];
             tma_load_4d(sm + OFF_V, &map_v, bb, 0, h, c0, b);
@@ -968,8 +996,10 @@ gla_bwd_kv_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
             tma_load_4d(sm + OFF_GQ + 8192, &map_gq, bb, 64, h, c0, b);
             bulk_load(sm + OFF_DS, a.state_img + static_cast<size_t>(blockIdx.x) * 65536, 65536, bb);
             bulk_load(misc + M_VEC, a.state_vec + static_cast<size_t>(blockIdx.x) * 3 * kD, 1536, bb);
-            // the chunk one wave later finds its inputs in L2
+            // the chunk one wave later finds its inputs in L2, asked for once this chunk's have landed (asked
+            // for beside them: 246 us against 240)
             const int nx = blockIdx.x + a.wave;
+            mbar_wait(bb, 0, abort_flag, status);
             if (a.wave > 0 && nx < static_cast<int>(gridDim.x)) {
                 const int bh2 = nx / NC, r2 = nx % NC, b2 = bh2 / H, h2 = bh2 % H, c2 = r2 * kC;
                 const CUtensorMap *maps[6] = {&map_k, &map_v, &map_do, &map_qg, &map_dkc, &map_gq};
@@ -1001,7 +1031,7 @@ gla_bwd_kv_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
     const uint64_t dSA = make_desc(sb + OFF_SA, 16, 1024);
 
     mbar_wait(&bar[BAR_IN], 0, abort_flag, status);
-    prep_chunk(nullptr, sm + OFF_K, sm + OFF_KD, sm + OFF_EG, gate_f32, a.l2norm, nullptr, nullptr, nullptr,
+    prep_chunk<kThreadsKv>(nullptr, sm + OFF_K, sm + OFF_KD, sm + OFF_EG, gate_f32, a.l2norm, nullptr, nullptr, nullptr,
                rkv, gq4, nullptr, nullptr, tid);
     mbar_wait(&bar[BAR_INB], 0, abort_flag, status);
     if (tid == 0 && !*abort_flag) {
@@ -1025,16 +1055,19 @@ gla_bwd_kv_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
     }
     mbar_wait(&bar[BAR_R1], 0, abort_flag, status);
     tc_fence_after();
-    if (grp == 0) {
+    if (grp < 2) {  // each group half of the columns
         float t1[32];
         tmem_ld16x2_32<32>(tq + TM_T1, t1);
-        masked_row(sm + OFF_P1, i, hf, t1, 0.f);  // P1[t][j] = [j <= t] do_t . v_j
+        // P1[t][j] = [j <= t] do_t . v_j
+        if (grp == 0) masked_row<0, 2>(sm + OFF_P1, i, hf, t1, 0.f);
+        else masked_row<2, 2>(sm + OFF_P1, i, hf, t1, 0.f);
     } else {
         float sa[32];
         tmem_ld16x2_32<32>(tq + TM_SA, sa);
         // SA[j][t] = [t >= j] Kd_j . QG_t (row i is key j)
 #pragma unroll
         for (int q4 = 0; q4 < 4; ++q4) {
+            if (q4 >> 1 != (grp & 1)) continue;
             float w[8];
 #pragma unroll
             for (int e = 0; e < 8; ++e) {
@@ -1046,7 +1079,7 @@ gla_bwd_kv_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
     }
     fence_proxy_async_smem();
     tc_fence_before();
-    compute_sync();
+    compute_sync<kThreadsKv>();
     if (tid == 0 && !*abort_flag) {
         tc_fence_after();
         for (int k = 0; k < 4; ++k)  // dkw += P1^T QG, dv += SA dO
@@ -1067,17 +1100,17 @@ gla_bwd_kv_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
         const uint8_t *dkct = sm + OFF_DKC + hf * 8192;
         const uint8_t *gqt = sm + OFF_GQ + hf * 8192;
         float *dgrow = dG + i * kDgStride + 64 * hf;
-        const int h2 = grp;  // this group's 32-column slice of each 128-column product
-        uint64_t dkb[16];    // fp32 pairs over consecutive columns
+        // this group: columns [16 grp, + 16) of each half of a 128-column product
+        uint64_t dkb[8];  // fp32 pairs over consecutive columns
         float dot;
         {
-            float x[32], y[32];
-            tmem_ld16x2_32<64>(tq + TM_DK + 32 * h2, x);
-            tmem_ld16x2_32<64>(tq + TM_KC + 32 * h2, y);
+            float x[16], y[16];
+            acc_ld16(tq + TM_DK + 16 * grp, x);
+            acc_ld16(tq + TM_KC + 16 * grp, y);
             uint64_t dot2 = 0;
 #pragma unroll
-            for (int q4 = 0; q4 < 4; ++q4) {
-                const int cc = 4 * h2 + q4;
+            for (int q4 = 0; q4 < 2; ++q4) {
+                const int cc = 2 * grp + q4;
                 const uint32_t off = t64_chunk(i, cc);
                 const uint4 er = *reinterpret_cast<const uint4 *>(egt + off);
                 const uint4 kr = *reinterpret_cast<const uint4 *>(kt + off);
@@ -1106,20 +1139,20 @@ gla_bwd_kv_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
             dot = dv.x + dv.y;
         }
         dot += __shfl_xor_sync(0xffffffffu, dot, 16);
-        if (hf == 0) red[grp * 128 + i] = dot;
+        if (hf == 0) red[grp * 64 + i] = dot;
         uint8_t *vt = sm + OFF_V + hf * 8192;
         {
-            float x[32];
-            tmem_ld16x2_32<64>(tq + TM_DV + 32 * h2, x);
+            float x[16];
+            acc_ld16(tq + TM_DV + 16 * grp, x);
 #pragma unroll
-            for (int q4 = 0; q4 < 4; ++q4) store_row_chunk(vt, i, 4 * h2 + q4, x + 8 * q4);
+            for (int q4 = 0; q4 < 2; ++q4) store_row_chunk(vt, i, 2 * grp + q4, x + 8 * q4);
         }
-        compute_sync();
-        dot = red[i] + red[128 + i];
+        compute_sync<kThreadsKv>();
+        dot = (red[i] + red[64 + i]) + (red[128 + i] + red[192 + i]);
         const uint64_t ndot = f2_make(-dot, -dot), rk2 = f2_make(rk, rk);
 #pragma unroll
-        for (int q4 = 0; q4 < 4; ++q4) {
-            const int cc = 4 * h2 + q4;
+        for (int q4 = 0; q4 < 2; ++q4) {
+            const int cc = 2 * grp + q4;
             const uint4 kr = *reinterpret_cast<const uint4 *>(kt + t64_chunk(i, cc));
             const uint32_t kw[4] = {kr.x, kr.y, kr.z, kr.w};
             uint32_t ow[4];
@@ -1133,7 +1166,7 @@ gla_bwd_kv_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
     }
     fence_proxy_async_smem();
     tc_fence_before();
-    compute_sync();
+    compute_sync<kThreadsKv>();
     if (tid == 0 && !*abort_flag) {
         tma_store_4d(&map_dk, sm + OFF_K, 0, h, c0, b);
         tma_store_4d(&map_dk, sm + OFF_K + 8192, 64, h, c0, b);
@@ -1144,31 +1177,36 @@ gla_bwd_kv_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
     {
         // dgk_t = sum_{s >= t in the chunk} dG_s + rowsum(dS_{r+1} * S_{r+1}): column
         // d, tokens in reverse, in two 32-row halves (half hh = rows [32 hh, 32 hh + 32))
+        // (256 threads: the order of the sums stays)
         const int d = tid & 127, hh = tid >> 7;
         float x[32], tot = 0.f;
+        if (hh < 2) {
 #pragma unroll
-        for (int u = 0; u < 32; ++u) {
-            x[u] = dG[(32 * hh + u) * kDgStride + d];
-            tot += x[u];
+            for (int u = 0; u < 32; ++u) {
+                x[u] = dG[(32 * hh + u) * kDgStride + d];
+                tot += x[u];
+            }
+            red[hh * 128 + d] = tot;
         }
-        red[hh * 128 + d] = tot;
-        compute_sync();
-        float acc = vec[kD + d] + vec[2 * kD + d] + (hh == 0 ? red[128 + d] : 0.f);
-        const int nvalid = min(kC, T - c0);
+        compute_sync<kThreadsKv>();
+        if (hh < 2) {
+            float acc = vec[kD + d] + vec[2 * kD + d] + (hh == 0 ? red[128 + d] : 0.f);
+            const int nvalid = min(kC, T - c0);
 #pragma unroll
-        for (int u = 31; u >= 0; --u) {
-            acc += x[u];
-            const int t = 32 * hh + u;
-            if (t < nvalid) {
-                const size_t o = ((static_cast<size_t>(b) * T + c0 + t) * H + h) * kD + d;
-                if (gate_f32) static_cast<float *>(a.dgk)[o] = acc;
-                else static_cast<__nv_bfloat16 *>(a.dgk)[o] = __float2bfloat16_rn(acc);
+            for (int u = 31; u >= 0; --u) {
+                acc += x[u];
+                const int t = 32 * hh + u;
+                if (t < nvalid) {
+                    const size_t o = ((static_cast<size_t>(b) * T + c0 + t) * H + h) * kD + d;
+                    if (gate_f32) static_cast<float *>(a.dgk)[o] = acc;
+                    else static_cast<__nv_bfloat16 *>(a.dgk)[o] = __float2bfloat16_rn(acc);
+                }
             }
         }
     }
     if (tid == 0) tma_store_wait_read();  // shared memory outlives the stores' reads
     tc_fence_before();
-    compute_sync();
+    compute_sync<kThreadsKv>();
     if (warp == 0) {
         tc_fence_after();
         tmem_dealloc(tbase, 512);
@@ -1193,13 +1231,13 @@ cudaError_t launch_gla_bwd(const BwdArgs &a, const BwdMaps &m, cudaStream_t s) {
     }
     const int nc = (a.T + kC - 1) / kC;
     const int chunks = a.B * a.H * nc;
-    gla_bwd_q_kernel<<<chunks, kThreadsLoad, qk::kSmem, s>>>(m.q, m.k, m.v, m.dO, m.g, m.dq, m.qg, m.dkc, m.gq,
+    gla_bwd_q_kernel<<<chunks, kThreadsQ + 32, qk::kSmem, s>>>(m.q, m.k, m.v, m.dO, m.g, m.dq, m.qg, m.dkc, m.gq,
                                                           m.dzr, a);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     e = launch_after(gla_bwd_state_kernel, a.B * a.H * 2, kThreads, st::kSmem, s, m.qg, m.dO, m.dzr, m.q, a);
     if (e != cudaSuccess) return e;
-    return launch_after(gla_bwd_kv_kernel, chunks, kThreadsLoad, kv::kSmem, s, m.k, m.v, m.dO, m.g, m.qg, m.dkc, m.gq,
+    return launch_after(gla_bwd_kv_kernel, chunks, kThreadsKv + 32, kv::kSmem, s, m.k, m.v, m.dO, m.g, m.qg, m.dkc, m.gq,
                         m.dk, m.dv, a);
 }
 
