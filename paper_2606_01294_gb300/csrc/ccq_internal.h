@@ -24,11 +24,11 @@ struct RecurrentArgs {
     void *o;
     float *ST, *CT, *mT;
     // Decode step: the position counts to advance in place (tT = t0), or NULL.  While the kernel runs the bits
-    // from kCountBits up of a row's count hold how many of its heads are done (ccq_recurrent.cu).
+    // from kCountBits up of a row's count hold how many of its heads have read it (ccq_recurrent.cu).
     int64_t *t_inplace = nullptr;
 };
-constexpr int kCountBits = 40;
-constexpr int kCountHeads = 1 << 16;  // heads a row the upper bits are used for
+constexpr int kCountBits = 52;
+constexpr int kCountHeads = 1 << 11;  // heads a row the twelve bits count (a launch of its own advances t above)
 
 // T = 1: the decode step; else launch_recurrent_block.
 cudaError_t launch_recurrent(const RecurrentArgs &a, cudaStream_t s);
