@@ -112,7 +112,8 @@ CCQ_API void ccq_default_params(ccq_params *p);
  *   o         [B,T,H,Dv] in in_dtype.
  * Supported: Dk = Dv in {64, 128}; T >= 0; B, H >= 1.  in_dtype BF16 runs the
  * chunkwise tensor-core kernel for Dk = Dv = 128 and the recurrent kernel
- * otherwise; FP32 always runs the recurrent kernel (fp32 arithmetic).
+ * otherwise; FP32 always runs the recurrent kernel (fp32 arithmetic; the
+ * backbone state token by token, the CCQ read in blocks of 32 tokens).
  * Gate range of the chunkwise kernels.  A chunk's decays are applied as factors
  * measured from reference tokens inside the chunk.  The default kernel (AUTO,
  * CHUNKWISE) has one reference, the chunk midpoint; it is exact (up to rounding)
@@ -181,7 +182,8 @@ CCQ_API ccq_status ccq_gdn_workspace_size(int B, int T, int H, int Dk, int Dv, c
  *   backbone  0 = GLA (gate: log alpha [B,H,Dk] in gate_dtype),
  *             1 = Gated DeltaNet (gate: log alpha [B,H] fp32; beta [B,H] fp32).
  *   q, k      [B,H,Dk]; v [B,H,Dv]; lambda [B,H] fp32; o [B,H,Dv] (in_dtype).
- *   S [B,H,Dk,Dv], C [B,H,Dk,Dk], m [B,H,Dk] fp32 and t [B] int64, read and written.
+ *   S [B,H,Dk,Dv], C [B,H,Dk,Dk], m [B,H,Dk] fp32 and t [B] int64 (0 <= t < 2^52),
+ *             read and written; t holds nothing of use while the step runs.
  */
 CCQ_API ccq_status ccq_decode_step(int backbone, const void *q, const void *k, const void *v,
                            const void *gate, const float *beta, const float *lambda,
@@ -270,12 +272,13 @@ CCQ_API ccq_status ccq_gla_bwd_workspace_size(int B, int T, int H, int Dk, int D
  *   workspace at least ccq_gdn_bwd_workspace_size() bytes (16-byte aligned): per
  *             64-token chunk of every (sequence, head), the chunk's forward states,
  *             state adjoints and intermediate tiles in fp32 (for bf16 inputs with
- *             Dk = 128, followed by the chunkwise forward's own workspace).
+ *             Dk = 128 partly as bf16 operand tiles, and followed by the chunkwise
+ *             forward's own workspace).
  * Supported: Dk = Dv in {64, 128}, bf16 or fp32 inputs.  The per-chunk forward quantities
  * the adjoint needs (the UT factor (I + A)^{-1}, the entering S^K, M and H of every chunk)
  * come, for bf16 inputs with Dk = 128, from the chunkwise tensor-core forward kernels of
- * ccq_gdn_fwd (which write them in fp32 and no output; their segment split follows
- * p->seq_split), and otherwise from three CUDA-core passes.  The products of the adjoint's
+ * ccq_gdn_fwd (which write them as fp32 arrays and bf16 operand tiles, and no output; their
+ * segment split follows p->seq_split), and otherwise from three CUDA-core passes.  The products of the adjoint's
  * per-chunk kernels run, for bf16 inputs, on the tensor cores (bf16 operands, fp32 accumulation;
  * their element-wise parts stay fp32) and, for fp32 inputs, on the CUDA cores in fp32; its reverse
  * pass over the state adjoint runs, for bf16 inputs with Dk = 128, on the tensor cores, and

@@ -14,8 +14,9 @@
 //   - a seventeenth warp issues the products (six rounds in the local kernel, five in the kv one), in an
 //     order that lets the next epilogue start on the first half of a round while the rest runs.
 // What bounds them: one CTA fits an SM (about 200 KB of tiles, all of TMEM), so a chunk is the latency of its
-// load, its rounds and its epilogues.  Measured on GB300 (B = 4, H = 16, T = 4096, 4096 chunks): see the
-// two kernels below.
+// load, its rounds and its epilogues (local: 1.9 GB of DRAM traffic at 4.0 TB/s, kv 1.6 GB at 3.6).  Measured on
+// GB300 (B = 4, H = 16, T = 4096, 4096 chunks; device times): local 2420 -> 476 us, kv 2770 -> 450 us against the
+// kernels of that file, suffix 279 -> 79 us; the training step 6.55 -> 1.89 ms.
 //
 // Thread layout: 512 compute threads.  Warp w, lane l: TMEM quadrant qd = w % 4, column group grp = w / 4;
 // in a 64-row product the thread holds row i = 16 qd + l % 16 and, with hf = l / 16, columns

@@ -1,5 +1,6 @@
 // ccq_gdn_bwd_kernels.cuh -- CCQ-Gated-DeltaNet backward kernels (fp32 tiles; the per-chunk kernels'
-// products on the tensor cores for bf16 inputs).
+// products on the tensor cores for bf16 inputs) of fp32 inputs and of Dk = Dv = 64; bf16 inputs with
+// Dk = Dv = 128 take the kernels of ccq_gdn_bwd_chunk_tc.cu and ccq_gdn_bwd_state_tc.cu for the same adjoint.
 //
 // Reverse mode of the CCQ read (Eq. clean, Eq. read, the undecayed running sums of Sec. 3.2)
 // with the Gated DeltaNet write as the backbone, chunked as Algorithm 1 chunks the forward.

@@ -1,6 +1,6 @@
 // ccq_gdn_bwd_tc.cuh -- the tensor-core product of the CCQ-Gated-DeltaNet backward's per-chunk
 // kernels (gdn_bwd_local_kernel and gdn_bwd_kv_kernel, instantiated with TC = true for bf16
-// inputs).
+// inputs; on the device for D = 64, since D = 128 has kernels of its own in ccq_gdn_bwd_chunk_tc.cu).
 //
 // Those kernels keep their operands as fp32 tiles in shared memory (row strides D + 1 and 65) and
 // evaluate some thirty small products a chunk,
