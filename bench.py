@@ -58,14 +58,14 @@ def varlen_lengths(n):
     return np.random.default_rng(VARLEN_SEED).integers(100, 4001, size=n).tolist()
 KERNEL_SOURCES = {"gla": "ccq_gla_chunk.cu", "gdn": "ccq_gdn_chunk.cu", "decode": "ccq_recurrent.cu",
                   "glavl": "ccq_gla_chunk.cu", "gdnvl": "ccq_gdn_chunk.cu",
-                  "glabwd": "ccq_gla_bwd.cu", "gdnbwd": ("ccq_gdn_bwd_kernels.cuh", "ccq_gdn_bwd_tc.cuh")}
+                  "glabwd": "ccq_gla_bwd.cu", "gdnbwd": ("ccq_gdn_bwd_chunk_tc.cu", "ccq_gdn_bwd_state_tc.cu")}
 KERNEL_NAMES = {"gla": "gla_chunk_kernel", "gdn": "gdn_wy_kernel + gdn_chunk_kernel",
                 "glavl": "gla_chunk_kernel (packed sequences)", "gdnvl": "gdn_wy_kernel + gdn_chunk_kernel (packed sequences)",
                 "decode": "decode_kernel",
                 "glabwd": "whole step: forward (saving checkpoints) + gla_bwd_q_kernel + gla_bwd_state_kernel"
                           " + gla_bwd_kv_kernel",
                 "gdnbwd": "whole step: forward (gdn_wy_kernel + gdn_chunk_kernel), the backward's forward recompute,"
-                          " gdn_bwd_local_kernel + gdn_bwd_state_tc_kernel + gdn_bwd_suffix_kernel + gdn_bwd_kv_kernel"}
+                          " gdn_bwd_local128_kernel + gdn_bwd_state_tc_kernel + gdn_bwd_suffix128_kernel + gdn_bwd_kv128_kernel"}
 
 
 def state_segments(B, H, T, sms):
@@ -176,25 +176,22 @@ STEP_KERNELS = {
     "decode_b256": ["decode_kernel"],
     "gla_bf16_4k_fwdbwd": ["gla_segment_state_kernel", "gla_segment_combine_kernel", "gla_chunk_kernel",
                            "gla_bwd_q_kernel", "gla_bwd_state_kernel", "gla_bwd_kv_kernel"],
-    # (the forward kernels run twice: the forward itself, then the backward's recompute of the
-    # forward's per-chunk quantities; segment-parallel at B = 4, H = 16)
+    # (the forward kernels run twice: the forward itself, then, forming only the states, for the
+    # backward; segment-parallel at B = 4, H = 16)
     "gdn_bf16_4k_fwdbwd": ["gdn_segment_state_kernel", "gdn_segment_combine_kernel", "gdn_wy_kernel",
-                           "gdn_chunk_kernel", "gdn_bwd_local_kernel", "gdn_bwd_state_tc_kernel",
-                           "gdn_bwd_suffix_kernel", "gdn_bwd_kv_kernel"],
+                           "gdn_chunk_kernel", "gdn_bwd_local128_kernel", "gdn_bwd_state_tc_kernel",
+                           "gdn_bwd_suffix128_kernel", "gdn_bwd_kv128_kernel"],
     "gla_bf16_varlen64": ["gla_chunk_kernel"],
     "gdn_bf16_varlen64": ["gdn_wy_kernel", "gdn_chunk_kernel"],
 }
-# (each step also runs the one-thread-per-row position update: 8 bytes per batch row, not counted)
 KERNEL_FILES = {"gla_chunk_kernel": "ccq_gla_chunk.cu", "gla_segment_state_kernel": "ccq_gla_segment.cu",
                 "gla_segment_combine_kernel": "ccq_gla_segment.cu", "gdn_wy_kernel": "ccq_gdn_chunk.cu",
                 "gdn_chunk_kernel": "ccq_gdn_chunk.cu",
-                "gdn_segment_state_kernel": "ccq_gdn_segment.cu", "gdn_segment_combine_kernel": "ccq_gdn_segment.cu", "recurrent": "ccq_recurrent.cu",
+                "gdn_segment_state_kernel": "ccq_gdn_segment.cu", "gdn_segment_combine_kernel": "ccq_gdn_segment.cu",
                 "decode_kernel": "ccq_recurrent.cu", "gla_bwd_state_kernel": "ccq_gla_bwd.cu",
                 "gla_bwd_q_kernel": "ccq_gla_bwd.cu", "gla_bwd_kv_kernel": "ccq_gla_bwd.cu",
                 "gdn_bwd_state_tc_kernel": "ccq_gdn_bwd_state_tc.cu",
-                **{f"gdn_bwd_{n}_kernel": "ccq_gdn_bwd_kernels.cuh"
-                   for n in ("prep", "prefix", "fstate", "dstate", "suffix")},
-                **{f"gdn_bwd_{n}_kernel": ("ccq_gdn_bwd_kernels.cuh", "ccq_gdn_bwd_tc.cuh") for n in ("local", "kv")}}
+                **{f"gdn_bwd_{n}128_kernel": "ccq_gdn_bwd_chunk_tc.cu" for n in ("local", "suffix", "kv")}}
 
 
 SHARED_DEVICE_SOURCES = ("sm100_ptx.cuh", "ccq_internal.h")  # inlined into every kernel
