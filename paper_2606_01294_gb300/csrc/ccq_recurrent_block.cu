@@ -284,9 +284,10 @@ __global__ void __launch_bounds__(kThreads, 1) recurrent_block_kernel(const Recu
                     cs += w;
 #pragma unroll
                     for (int u = 0; u < U; ++u) {
-                        const float kv = kn[j * LD + d0 + dl + u];
+                        // (selected, not left to the zero score: a later token's key may be infinite or NaN)
+                        const float kv = j <= lane ? kn[j * LD + d0 + dl + u] : 0.f;
                         z[u] = fmaf(w, kv, z[u]);
-                        ms[u] += j <= lane ? kv : 0.f;
+                        ms[u] += kv;
                     }
                 }
 #pragma unroll

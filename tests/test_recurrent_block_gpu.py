@@ -1,0 +1,33 @@
+"""GPU checks of the fp32 forward in blocks of 32 tokens (ccq_recurrent_block.cu) where its blocks must not show:
+values that are not finite reach no earlier token."""
+import pytest
+import torch
+
+from paper_2606_01294_gb300 import ccq
+from paper_2606_01294_gb300 import inputs as gen
+from tests.helpers import GDN, GLA, TOL, compare, gpu_forward, oracle_forward
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(autouse=True)
+def _status():
+    yield
+    ccq.device_status()
+
+
+@pytest.mark.parametrize("backbone", [GLA, GDN])
+@pytest.mark.parametrize("dtype,d", [(torch.float32, 64), (torch.float32, 128), (torch.bfloat16, 64)])
+@pytest.mark.parametrize("B,H", [(1, 2), (2, 10), (2, 19), (7, 11)])  # eight, four, two CTAs a sequence and one
+@pytest.mark.parametrize("name", ["q", "k", "v", "gate", "lam"])
+@pytest.mark.parametrize("bad", [float("nan"), float("inf")])
+def test_later_tokens_leave_earlier_outputs(backbone, dtype, d, B, H, name, bad):
+    """A value at token 37 that is not finite (a right-padded batch whose padding was never written): the outputs
+    of tokens 0 to 36, whole block and started block, are bit for bit those of the finite inputs."""
+    T, at = 50, 37
+    P = gen.make_inputs(backbone, B, T, H, d, d, dtype=dtype, seed=91, lam="trained", keys="structured")
+    want, _ = gpu_forward(backbone, P, algo="recurrent")
+    P[name] = P[name].clone()
+    P[name][:, at:] = bad
+    got, _ = gpu_forward(backbone, P, algo="recurrent")
+    assert torch.equal(got[:, :at], want[:, :at])
