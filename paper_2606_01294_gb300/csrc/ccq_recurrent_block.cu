@@ -406,7 +406,8 @@ __global__ void __launch_bounds__(kThreads, 1) recurrent_block_kernel(const Recu
 #pragma unroll
                     for (int o = P::TPC / 2; o > 0; o >>= 1) r0[g] += __shfl_xor_sync(0xffffffffu, r0[g], o);
                     // S <- alpha S + kbar (beta (v - alpha kbar^T S))
-                    const float w = bt * (vv[g] - ag * r0[g]);
+                    // (past the sequence S stays as it is, where 0 times an infinite kbar^T S would not leave it)
+                    const float w = t < n ? bt * (vv[g] - ag * r0[g]) : 0.f;
 #pragma unroll
                     for (int u = 0; u < P::NV; ++u) {
                         if (!kKeep) ldv<P::V>(kn + t * LD + P::V * (tl + P::TPC * u), kv[0]);

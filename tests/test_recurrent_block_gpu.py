@@ -1,5 +1,5 @@
 """GPU checks of the fp32 forward in blocks of 32 tokens (ccq_recurrent_block.cu) where its blocks must not show:
-values that are not finite reach no earlier token."""
+values that are not finite reach no earlier token, and the rows past the sequence change no state."""
 import pytest
 import torch
 
@@ -31,3 +31,20 @@ def test_later_tokens_leave_earlier_outputs(backbone, dtype, d, B, H, name, bad)
     P[name][:, at:] = bad
     got, _ = gpu_forward(backbone, P, algo="recurrent")
     assert torch.equal(got[:, :at], want[:, :at])
+
+
+@pytest.mark.parametrize("backbone", [GLA, GDN])
+@pytest.mark.parametrize("dtype,d", [(torch.float32, 64), (torch.float32, 128), (torch.bfloat16, 64)])
+@pytest.mark.parametrize("B,H", [(1, 2), (2, 10), (2, 19), (7, 11)])
+@pytest.mark.parametrize("T", [1, 33, 46])
+def test_rows_past_the_sequence_leave_an_infinite_state(backbone, dtype, d, B, H, T):
+    """An infinite value in column 5 of the last token: the state's column is infinite after it (kbar v, whose every
+    entry is non-zero), and the part of the block past the sequence keeps it so; the other columns are finite."""
+    P = gen.make_inputs(backbone, B, T, H, d, d, dtype=dtype, seed=93, lam="trained")
+    P["v"] = P["v"].clone()
+    P["v"][:, -1, :, 5] = float("inf")
+    _, S = gpu_forward(backbone, P, algo="recurrent")
+    rest = [c for c in range(d) if c != 5]
+    assert bool(torch.isinf(S.S[..., 5]).all()) and bool(torch.isfinite(S.S[..., rest]).all())
+    want = torch.sign(P["k"][:, -1].float()).cuda()
+    assert torch.equal(torch.sign(S.S[..., 5]), want)
