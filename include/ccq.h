@@ -182,8 +182,7 @@ CCQ_API ccq_status ccq_gdn_workspace_size(int B, int T, int H, int Dk, int Dv, c
  *   backbone  0 = GLA (gate: log alpha [B,H,Dk] in gate_dtype),
  *             1 = Gated DeltaNet (gate: log alpha [B,H] fp32; beta [B,H] fp32).
  *   q, k      [B,H,Dk]; v [B,H,Dv]; lambda [B,H] fp32; o [B,H,Dv] (in_dtype).
- *   S [B,H,Dk,Dv], C [B,H,Dk,Dk], m [B,H,Dk] fp32 and t [B] int64 (0 <= t < 2^52),
- *             read and written; t holds nothing of use while the step runs.
+ *   S [B,H,Dk,Dv], C [B,H,Dk,Dk], m [B,H,Dk] fp32 and t [B] int64, read and written.
  */
 CCQ_API ccq_status ccq_decode_step(int backbone, const void *q, const void *k, const void *v,
                            const void *gate, const float *beta, const float *lambda,

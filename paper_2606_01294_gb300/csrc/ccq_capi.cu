@@ -1082,10 +1082,8 @@ ccq_status ccq_decode_step(int backbone, const void *q, const void *k, const voi
     ra.q = q; ra.k = k; ra.v = v; ra.gate = gate; ra.beta = beta; ra.lambda = lambda;
     ra.S0 = S; ra.C0 = C; ra.m0 = m; ra.t0 = t;
     ra.o = o; ra.ST = S; ra.CT = C; ra.mT = m;
-    const bool in_kernel = H <= kCountHeads;  // else a launch of its own
-    if (in_kernel) ra.t_inplace = t;
     st = run_recurrent(ra, static_cast<cudaStream_t>(stream));
-    return st != CCQ_OK || in_kernel ? st : finish_t(t, t, B, 1, static_cast<cudaStream_t>(stream));
+    return st != CCQ_OK ? st : finish_t(t, t, B, 1, static_cast<cudaStream_t>(stream));
 }
 
 ccq_status ccq_device_status(void *stream) {

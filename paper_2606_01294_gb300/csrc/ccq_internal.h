@@ -23,20 +23,16 @@ struct RecurrentArgs {
     const int64_t *t0;
     void *o;
     float *ST, *CT, *mT;
-    // Decode step: the position counts to advance in place (tT = t0), or NULL.  While the kernel runs the bits
-    // from kCountBits up of a row's count hold how many of its heads have read it (ccq_recurrent.cu).
-    int64_t *t_inplace = nullptr;
 };
-constexpr int kCountBits = 52;
-constexpr int kCountHeads = 1 << 11;  // heads a row the twelve bits count (a launch of its own advances t above)
 
 // T = 1: the decode step; else launch_recurrent_block.
 cudaError_t launch_recurrent(const RecurrentArgs &a, cudaStream_t s);
 cudaError_t launch_recurrent_block(const RecurrentArgs &a, cudaStream_t s);
 
-// tT[b] = t0[b] + T (t0 NULL: T), one thread per batch row.  Where tT overlaps t0 the kernels leave
-// the final count to this launch, enqueued after them: every (batch, head) CTA reads t0[b] as it
-// starts.  (Elsewhere they write it themselves: a launch less, about 3 us of a call.)
+// tT[b] = t0[b] + T (t0 NULL: T), one thread per batch row.  Where tT overlaps t0 (the decode step always) the
+// kernels leave the final count to this launch, enqueued after them: every (batch, head) CTA reads t0[b] as it
+// starts, and nothing but the end of the launch says that all have.  It waits for the kernel before it by itself
+// (launch_after).  (Elsewhere they write it themselves: a launch less, about 3 us of a call.)
 cudaError_t launch_t_update(const int64_t *t0, int64_t *tT, int B, int T, cudaStream_t s);
 // tT[s] = t0[s] + (cu[s+1] - cu[s]) (t0 NULL: 0 +) for packed sequences (device cu).
 cudaError_t launch_t_update_varlen(const int64_t *t0, int64_t *tT, const int64_t *cu, int num_seqs,

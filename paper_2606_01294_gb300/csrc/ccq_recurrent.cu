@@ -22,6 +22,7 @@
 #include <stdint.h>
 
 #include "ccq_internal.h"
+#include "sm100_ptx.cuh"
 
 namespace ccq {
 
@@ -124,19 +125,8 @@ decode_kernel(RecurrentArgs a) {
             scal[4] = a.beta[row];
         }
     }
-    int64_t t0 = a.t0 ? (a.t_inplace ? *reinterpret_cast<const volatile int64_t *>(a.t0 + b) : a.t0[b]) : 0;
-    if (a.t_inplace) t0 &= (int64_t{1} << kCountBits) - 1;
-    const int64_t t = t0 + 1;
+    const int64_t t = (a.t0 ? a.t0[b] : 0) + 1;
     __syncthreads();
-    // The count of a batch row is shared by its heads, each a CTA of its own that reads it above, so the CTA that
-    // arrives last writes it: the arrivals are counted in the count's own upper bits, which need no memory
-    // of the library's and leave no state behind.  (A launch of its own for the update cost a small decode step
-    // 6 of 24 us.)
-    if (a.t_inplace && tid == 0) {
-        unsigned long long *tp = reinterpret_cast<unsigned long long *>(a.t_inplace + b);
-        const unsigned long long before = atomicAdd(tp, 1ull << kCountBits);
-        if (static_cast<int>(before >> kCountBits) == a.H - 1) atomicExch(tp, static_cast<unsigned long long>(t));
-    }
     if (warp < 2) {
         const float *x = warp == 0 ? qs : ks;
         float s = 0.f;
@@ -302,6 +292,7 @@ cudaError_t launch_bb(const RecurrentArgs &a, cudaStream_t s) {
 
 __global__ void t_update_kernel(const int64_t *t0, int64_t *tT, int B, int T) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    grid_wait();
     if (i < B) tT[i] = (t0 ? t0[i] : 0) + T;
 }
 
@@ -314,8 +305,7 @@ __global__ void t_update_varlen_kernel(const int64_t *t0, int64_t *tT, const int
 
 cudaError_t launch_t_update(const int64_t *t0, int64_t *tT, int B, int T, cudaStream_t s) {
     if (!tT || B == 0) return cudaSuccess;
-    t_update_kernel<<<(B + 255) / 256, 256, 0, s>>>(t0, tT, B, T);
-    return cudaGetLastError();
+    return launch_after(t_update_kernel, (B + 255) / 256, 256, 0, s, t0, tT, B, T);
 }
 
 cudaError_t launch_t_update_varlen(const int64_t *t0, int64_t *tT, const int64_t *cu, int num_seqs,
