@@ -129,7 +129,8 @@ CCQ_API void ccq_default_params(ccq_params *p);
  *   workspace  caller-owned device scratch of at least ccq_gla_workspace_size()
  *              bytes (16-byte aligned) when that size is non-zero (long sequences
  *              split into segments); may be NULL otherwise.  Contents undefined on
- *              return.
+ *              return.  On less, a forward with seq_split = 0 cuts into longer segments
+ *              (of eight chunks or more) or none, if the workspace holds that split.
  * Returns CCQ_OK or an error code; launches asynchronously on `stream`.
  */
 CCQ_API ccq_status ccq_gla_fwd(const void *q, const void *k, const void *v, const void *gk,

@@ -280,6 +280,10 @@ static bool gla_chunk_selected(const ccq_params &p, ccq_dtype in_dtype, int Dk, 
     return in_dtype == CCQ_BF16 && Dk == 128 && T > 0 && p.algo != CCQ_ALGO_RECURRENT;
 }
 
+static size_t gla_segment_bytes(int B, int H, int nseg) {
+    return nseg > 1 ? static_cast<size_t>(B) * H * nseg * kSegFloats * sizeof(float) : 0;
+}
+
 ccq_status ccq_gla_workspace_size(int B, int T, int H, int Dk, int Dv, ccq_dtype in_dtype,
                                   const ccq_params *p, size_t *bytes) {
     Common c;
@@ -290,7 +294,7 @@ ccq_status ccq_gla_workspace_size(int B, int T, int H, int Dk, int Dv, ccq_dtype
     if (gla_chunk_selected(c.p, in_dtype, Dk, T)) {
         int ns, per;
         split_gla_forward(c.p, B, T, H, &ns, &per);  // no fewer than a checkpoint forward needs
-        if (ns > 1) *bytes = static_cast<size_t>(B) * H * ns * kSegFloats * sizeof(float);
+        *bytes = gla_segment_bytes(B, H, ns);
     }
     return CCQ_OK;
 }
@@ -327,10 +331,19 @@ static ccq_status gla_fwd_impl(const void *q, const void *k, const void *v, cons
         return fail(CCQ_ERR_UNSUPPORTED, "checkpoints come from the chunkwise kernel (algo recurrent given)");
     if (chunk_ok && c.p.algo != CCQ_ALGO_RECURRENT) {
         int nseg = 1, seg_chunks = 0;
-        if (ckpt) split_sequences(c.p, B, T, H, &nseg, &seg_chunks);
-        else split_gla_forward(c.p, B, T, H, &nseg, &seg_chunks);
+        split_sequences(c.p, B, T, H, &nseg, &seg_chunks);
+        if (!ckpt) {
+            // the finer split where the workspace holds it: its need rises and falls with T, so a workspace made for
+            // the longest T of several may not (the coarser split's outputs have the same accuracy)
+            int ns, per;
+            split_gla_forward(c.p, B, T, H, &ns, &per);
+            if (workspace && aligned16(workspace) && workspace_bytes >= gla_segment_bytes(B, H, ns)) {
+                nseg = ns;
+                seg_chunks = per;
+            }
+        }
         if (nseg > 1) {
-            const size_t need = static_cast<size_t>(B) * H * nseg * kSegFloats * sizeof(float);
+            const size_t need = gla_segment_bytes(B, H, nseg);
             if (!workspace || workspace_bytes < need)
                 return fail(CCQ_ERR_INVALID_ARG, "workspace of %zu bytes required (got %zu)", need,
                             workspace ? workspace_bytes : static_cast<size_t>(0));
@@ -1011,12 +1024,6 @@ ccq_status ccq_fwd_varlen(int backbone, const void *q, const void *k, const void
                              static_cast<cudaStream_t>(stream));
     st = check_varlen(backbone, cu_seqlens, num_seqs, H, true, &mx);
     if (st != CCQ_OK) return st;
-    size_t need = 0;
-    st = ccq_fwd_varlen_workspace_size(backbone, cu_seqlens, num_seqs, H, Dk, Dv, in_dtype, p, &need);
-    if (st != CCQ_OK) return st;
-    if (need && (!workspace || workspace_bytes < need))
-        return fail(CCQ_ERR_INVALID_ARG, "workspace of %zu bytes required (got %zu)", need,
-                    workspace ? workspace_bytes : static_cast<size_t>(0));
     const size_t esz = in_dtype == CCQ_BF16 ? 2 : 4, gsz = gate_dtype == CCQ_BF16 ? 2 : 4;
     const size_t h = static_cast<size_t>(H);
     ccq_params pin;
