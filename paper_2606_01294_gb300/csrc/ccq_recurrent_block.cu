@@ -25,6 +25,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "ccq_internal.h"
 
 namespace ccq {
@@ -466,33 +468,66 @@ __global__ void __launch_bounds__(kThreads, 1) recurrent_block_kernel(const Recu
 }
 
 template <int D, int BB, int NS>
-cudaError_t launch_ns(const RecurrentArgs &a, cudaStream_t st) {
-    constexpr size_t smem = Shape<D, NS>::kFloats * sizeof(float);
-    cudaError_t e = cudaFuncSetAttribute(recurrent_block_kernel<D, BB, NS>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
-    if (e != cudaSuccess) return e;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(static_cast<unsigned>(a.B * a.H * NS));
-    cfg.blockDim = dim3(kThreads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
+struct Launch {
+    static constexpr size_t kSmem = Shape<D, NS>::kFloats * sizeof(float);
     cudaLaunchAttribute at;
-    at.id = cudaLaunchAttributeClusterDimension;
-    at.val.clusterDim.x = NS;
-    at.val.clusterDim.y = at.val.clusterDim.z = 1;
-    cfg.attrs = &at;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, recurrent_block_kernel<D, BB, NS>, a);
+    cudaLaunchConfig_t cfg = {};
+
+    Launch(long long seqs, cudaStream_t st) {
+        cfg.gridDim = dim3(static_cast<unsigned>(seqs * NS));
+        cfg.blockDim = dim3(kThreads);
+        cfg.dynamicSmemBytes = kSmem;
+        cfg.stream = st;
+        at.id = cudaLaunchAttributeClusterDimension;
+        at.val.clusterDim.x = NS;
+        at.val.clusterDim.y = at.val.clusterDim.z = 1;
+        cfg.attrs = &at;
+        cfg.numAttrs = 1;
+    }
+    static cudaError_t allow() {
+        return cudaFuncSetAttribute(recurrent_block_kernel<D, BB, NS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    static_cast<int>(kSmem));
+    }
+};
+
+template <int D, int BB, int NS>
+cudaError_t launch_ns(const RecurrentArgs &a, cudaStream_t st) {
+    cudaError_t e = Launch<D, BB, NS>::allow();
+    if (e != cudaSuccess) return e;
+    Launch<D, BB, NS> l(static_cast<long long>(a.B) * a.H, st);
+    return cudaLaunchKernelEx(&l.cfg, recurrent_block_kernel<D, BB, NS>, a);
 }
 
-// The CTAs of a (batch, head): as many as keep the grid within the 152 SMs (one CTA an SM: two of the larger
-// ones do not fit its shared memory), since a block's cost falls with them.
+// The clusters of NS CTAs that the current device runs at once, at one CTA an SM (the larger ones do not share
+// one).  0 where it cannot be asked.
+template <int D, int BB, int NS>
+int resident() {
+    static std::atomic<int> known[64];  // by device, 1 + the count
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
+    int n = known[dev].load(std::memory_order_relaxed) - 1;
+    if (n < 0) {
+        Launch<D, BB, NS> l(1, nullptr);
+        if (Launch<D, BB, NS>::allow() != cudaSuccess ||
+            cudaOccupancyMaxActiveClusters(&n, recurrent_block_kernel<D, BB, NS>, &l.cfg) != cudaSuccess) {
+            cudaGetLastError();
+            return 0;
+        }
+        known[dev].store(n + 1, std::memory_order_relaxed);
+    }
+    return n;
+}
+
+// The CTAs of a (batch, head): as many as keep every cluster resident, since a block's cost falls with them and a
+// second round of clusters doubles it.  The clusters that fit are fewer than the SMs by count, as one lies within a
+// GPC: on GB300 15 of eight CTAs, 36 of four, 76 of two.  d = 128, T = 256, GLA: 83 us a sequence on eight CTAs,
+// 120 on four, 193 on two, 256 on one; sixteen sequences 120 us on four CTAs each, 164 on eight.
 template <int D, int BB>
 cudaError_t launch_d(const RecurrentArgs &a, cudaStream_t st) {
     const long long seqs = static_cast<long long>(a.B) * a.H;
-    if (seqs * 8 <= 152) return launch_ns<D, BB, 8>(a, st);
-    if (seqs * 4 <= 152) return launch_ns<D, BB, 4>(a, st);
-    if (seqs * 2 <= 152) return launch_ns<D, BB, 2>(a, st);
+    if (seqs <= resident<D, BB, 8>()) return launch_ns<D, BB, 8>(a, st);
+    if (seqs <= resident<D, BB, 4>()) return launch_ns<D, BB, 4>(a, st);
+    if (seqs <= resident<D, BB, 2>()) return launch_ns<D, BB, 2>(a, st);
     return launch_ns<D, BB, 1>(a, st);
 }
 

@@ -48,3 +48,14 @@ def test_rows_past_the_sequence_leave_an_infinite_state(backbone, dtype, d, B, H
     assert bool(torch.isinf(S.S[..., 5]).all()) and bool(torch.isfinite(S.S[..., rest]).all())
     want = torch.sign(P["k"][:, -1].float()).cuda()
     assert torch.equal(torch.sign(S.S[..., 5]), want)
+
+
+@pytest.mark.parametrize("backbone", [GLA, GDN])
+@pytest.mark.parametrize("dtype,d", [(torch.float32, 64), (torch.float32, 128), (torch.bfloat16, 64)])
+@pytest.mark.parametrize("B,H", [(1, 15), (1, 16), (3, 12), (1, 37), (4, 19), (7, 11), (17, 9)])
+def test_sequence_counts_where_the_cluster_size_changes(backbone, dtype, d, B, H):
+    """15 and 16, 36 and 37, 76 and 77 sequences, where the clusters of eight, four and two CTAs stop fitting the
+    device at once, and more sequences than SMs."""
+    P = gen.make_inputs(backbone, B, 45, H, d, d, dtype=dtype, seed=94, lam="trained", keys="structured")
+    o, S = gpu_forward(backbone, P, algo="recurrent")
+    compare(o, S, oracle_forward(backbone, P), TOL[dtype], f"B={B} H={H}")
