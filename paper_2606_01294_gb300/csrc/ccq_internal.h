@@ -8,7 +8,7 @@
 
 namespace ccq {
 
-// Arguments of the decode step (ccq_recurrent.cu) and of the fp32 forward over a sequence
+// Arguments of the token-by-token kernels (ccq_recurrent.cu) and of the fp32 forward in blocks of tokens
 // (ccq_recurrent_block.cu).  dtype codes
 // follow ccq_dtype (0 = bf16, 1 = fp32).
 struct RecurrentArgs {
@@ -25,9 +25,10 @@ struct RecurrentArgs {
     float *ST, *CT, *mT;
 };
 
-// T = 1: the decode step; else launch_recurrent_block.
+// T = 1: the decode step; else launch_recurrent_block where recurrent_block_pays(), or token by token.
 cudaError_t launch_recurrent(const RecurrentArgs &a, cudaStream_t s);
 cudaError_t launch_recurrent_block(const RecurrentArgs &a, cudaStream_t s);
+bool recurrent_block_pays(const RecurrentArgs &a);
 
 // tT[b] = t0[b] + T (t0 NULL: T), one thread per batch row.  Where tT overlaps t0 (the decode step always) the
 // kernels leave the final count to this launch, enqueued after them: every (batch, head) CTA reads t0[b] as it

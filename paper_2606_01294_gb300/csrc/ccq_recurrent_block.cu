@@ -25,6 +25,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <algorithm>
 #include <atomic>
 
 #include "ccq_internal.h"
@@ -523,12 +524,35 @@ int resident() {
 // GPC: on GB300 15 of eight CTAs, 36 of four, 76 of two.  d = 128, T = 256, GLA: 83 us a sequence on eight CTAs,
 // 120 on four, 193 on two, 256 on one; sixteen sequences 120 us on four CTAs each, 164 on eight.
 template <int D, int BB>
+int cluster_ctas(long long seqs) {
+    return seqs <= resident<D, BB, 8>() ? 8 : seqs <= resident<D, BB, 4>() ? 4 : seqs <= resident<D, BB, 2>() ? 2 : 1;
+}
+
+template <int D, int BB>
 cudaError_t launch_d(const RecurrentArgs &a, cudaStream_t st) {
-    const long long seqs = static_cast<long long>(a.B) * a.H;
-    if (seqs <= resident<D, BB, 8>()) return launch_ns<D, BB, 8>(a, st);
-    if (seqs <= resident<D, BB, 4>()) return launch_ns<D, BB, 4>(a, st);
-    if (seqs <= resident<D, BB, 2>()) return launch_ns<D, BB, 2>(a, st);
-    return launch_ns<D, BB, 1>(a, st);
+    switch (cluster_ctas<D, BB>(static_cast<long long>(a.B) * a.H)) {
+        case 8: return launch_ns<D, BB, 8>(a, st);
+        case 4: return launch_ns<D, BB, 4>(a, st);
+        case 2: return launch_ns<D, BB, 2>(a, st);
+        default: return launch_ns<D, BB, 1>(a, st);
+    }
+}
+
+// The longest sequence for which the token-by-token kernel is the faster one.  A first block costs what `first`
+// tokens there do (measured at 1 to 4096 sequences and 2 to 40 tokens; the columns: eight, four, two CTAs a sequence
+// and one): with d = 128 and GLA the kernels meet at 12 us with one sequence, at 16 with 20, at 32 with 100, and
+// with more sequences than SMs both take proportionally longer.  With d = 64 two CTAs of the token-by-token kernel
+// share an SM at little cost, so it loses by a round of one CTA an SM (the only one, or the last of few), and over
+// many rounds the states' traffic costs the blocks more.  A further block costs 13 to 16 tokens.
+template <int D, int BB>
+int token_limit(const RecurrentArgs &a) {
+    constexpr int first[2][2][4] = {{{4, 5, 7, 22}, {3, 4, 5, 17}}, {{4, 6, 10, 17}, {3, 5, 7, 13}}};
+    const long long seqs = static_cast<long long>(a.B) * a.H, sms = std::max(1, resident<D, BB, 1>());
+    const long long rounds = (seqs + sms - 1) / sms;
+    const int ns = cluster_ctas<D, BB>(seqs);
+    int limit = first[D == 128][BB][ns == 8 ? 0 : ns == 4 ? 1 : ns == 2 ? 2 : 3];
+    if (D == 64 && ns == 1) limit += rounds >= 10 ? 5 : rounds & 1 ? -static_cast<int>(limit / (2 * rounds)) : 0;
+    return limit + (D == 128 && rounds == 1 ? 16 : 13) * (std::max(a.T - 1, 0) / kL);
 }
 
 }  // namespace
@@ -536,6 +560,11 @@ cudaError_t launch_d(const RecurrentArgs &a, cudaStream_t st) {
 cudaError_t launch_recurrent_block(const RecurrentArgs &a, cudaStream_t s) {
     if (a.Dk == 128) return a.backbone == 0 ? launch_d<128, 0>(a, s) : launch_d<128, 1>(a, s);
     return a.backbone == 0 ? launch_d<64, 0>(a, s) : launch_d<64, 1>(a, s);
+}
+
+bool recurrent_block_pays(const RecurrentArgs &a) {
+    if (a.Dk == 128) return a.T > (a.backbone == 0 ? token_limit<128, 0>(a) : token_limit<128, 1>(a));
+    return a.T > (a.backbone == 0 ? token_limit<64, 0>(a) : token_limit<64, 1>(a));
 }
 
 }  // namespace ccq

@@ -59,3 +59,23 @@ def test_sequence_counts_where_the_cluster_size_changes(backbone, dtype, d, B, H
     P = gen.make_inputs(backbone, B, 45, H, d, d, dtype=dtype, seed=94, lam="trained", keys="structured")
     o, S = gpu_forward(backbone, P, algo="recurrent")
     compare(o, S, oracle_forward(backbone, P), TOL[dtype], f"B={B} H={H}")
+
+
+@pytest.mark.parametrize("backbone", [GLA, GDN])
+@pytest.mark.parametrize("dtype,d", [(torch.float32, 64), (torch.float32, 128), (torch.bfloat16, 64)])
+@pytest.mark.parametrize("B,H,lengths", [(1, 2, (0, 2, 3, 4, 5)), (2, 10, (4, 5, 6, 7)), (2, 19, (5, 6, 7, 8, 10, 11)),
+                                         (7, 11, (8, 9, 10, 11, 12, 13, 14, 17, 18)), (10, 16, (17, 18, 22, 23, 33, 37, 38))])
+def test_short_sequences_token_by_token_or_in_blocks(backbone, dtype, d, B, H, lengths):
+    """Either side of the lengths where the token-by-token kernel hands over to the blocks, resumed in place; one
+    kernel's state goes on in the other's."""
+    prev = gen.make_inputs(backbone, B, 3, H, d, d, dtype=dtype, seed=98, lam="trained")
+    _, S0 = gpu_forward(backbone, prev, algo="recurrent")
+    st = {n: getattr(S0, n).cpu().numpy() for n in ("S", "C", "m", "t")}
+    for T in lengths:
+        P = gen.make_inputs(backbone, B, T, H, d, d, dtype=dtype, seed=99 + T, lam="trained", keys="structured")
+        S = ccq.CCQState(S0.S.clone(), S0.C.clone(), S0.m.clone(), S0.t.clone())
+        o, _ = gpu_forward(backbone, P, S, algo="recurrent", final_state=S)
+        if T == 0:
+            assert all(torch.equal(getattr(S, n), getattr(S0, n)) for n in ("S", "C", "m", "t"))
+        else:
+            compare(o, S, oracle_forward(backbone, P, st), TOL[dtype], f"B={B} H={H} T={T}")
