@@ -220,7 +220,8 @@ __global__ void __launch_bounds__(kThreads, 1) recurrent_block_kernel(const Recu
                     qn[(warp + 8 * r) * LD + lane + 32 * e] = xq[r][e] * rq;
                     kn[(warp + 8 * r) * LD + lane + 32 * e] = xk[r][e] * rk;
                 }
-                if (lane == 0) cq[warp + 8 * r] = mq[r] * rq;
+                // (a row whose square overflows has qbar = 0, so m . qbar = 0 whatever m . q is)
+                if (lane == 0) cq[warp + 8 * r] = rq > 0.f ? mq[r] * rq : 0.f;
             }
         }
         __syncthreads();

@@ -79,3 +79,18 @@ def test_short_sequences_token_by_token_or_in_blocks(backbone, dtype, d, B, H, l
             assert all(torch.equal(getattr(S, n), getattr(S0, n)) for n in ("S", "C", "m", "t"))
         else:
             compare(o, S, oracle_forward(backbone, P, st), TOL[dtype], f"B={B} H={H} T={T}")
+
+
+@pytest.mark.parametrize("backbone", [GLA, GDN])
+@pytest.mark.parametrize("dtype,d", [(torch.float32, 64), (torch.bfloat16, 128)])
+def test_query_whose_square_overflows(backbone, dtype, d):
+    """|q|^2 above fp32's range normalises to a zero query, and its output is zero, token by token as in blocks, also
+    where m . q itself overflows."""
+    for T in (3, 40):
+        P = gen.make_inputs(backbone, 1, T, 2, d, d, dtype=dtype, seed=101, lam="trained")
+        P["k"] = P["k"].abs()  # m . q: a sum of positive terms
+        want, _ = gpu_forward(backbone, P, algo="recurrent")
+        P["q"] = P["q"].clone()
+        P["q"][:, -1] = 1e38
+        got, _ = gpu_forward(backbone, P, algo="recurrent")
+        assert torch.equal(got[:, :-1], want[:, :-1]) and not got[:, -1].any()
