@@ -99,8 +99,8 @@ def gla_segments(B, H, T, sms):
 
 def launches_per_step(kind, B, H, T, sms):
     """Kernel launches of one step: a GLA forward is one kernel, or three when its sequences are
-    split, the Gated DeltaNet forward two (WY, chunk) or four; the GLA backward three; the decode step one
-    (the kernels write the position count)."""
+    split, the Gated DeltaNet forward two (WY, chunk) or four (these write the position count); the GLA
+    backward three; the decode step two (it updates the position count in place, in a launch of its own)."""
     if kind in ("glavl", "gdnvl"):  # one launch (two for GDN: WY, chunk)
         return 1 if kind == "glavl" else 2
     gla = 3 if gla_segments(B, H, T, sms) > 1 else 1
@@ -108,7 +108,7 @@ def launches_per_step(kind, B, H, T, sms):
     gdn = 4 if train else 2
     # the Gated DeltaNet training step runs the forward twice (the step's forward, then the
     # backward's recompute of the forward's per-chunk quantities) and four backward kernels
-    return {"gla": gla, "gdn": gdn, "decode": 1, "glabwd": (3 if train else 1) + 3, "gdnbwd": 2 * gdn + 4}[kind]
+    return {"gla": gla, "gdn": gdn, "decode": 2, "glabwd": (3 if train else 1) + 3, "gdnbwd": 2 * gdn + 4}[kind]
 
 
 def algorithmic_bytes(kind, B, H, T, D):
@@ -173,7 +173,7 @@ STEP_KERNELS = {
     "gla_bf16_20k": ["gla_segment_state_kernel", "gla_segment_combine_kernel", "gla_chunk_kernel"],
     "gdn_bf16_20k": ["gdn_wy_kernel", "gdn_segment_state_kernel", "gdn_segment_combine_kernel",
                      "gdn_chunk_kernel"],
-    "decode_b256": ["decode_kernel"],
+    "decode_b256": ["decode_kernel"],  # and the count update, 16 bytes a batch row
     "gla_bf16_4k_fwdbwd": ["gla_segment_state_kernel", "gla_segment_combine_kernel", "gla_chunk_kernel",
                            "gla_bwd_q_kernel", "gla_bwd_state_kernel", "gla_bwd_kv_kernel"],
     # (the forward kernels run twice: the forward itself, then, forming only the states, for the

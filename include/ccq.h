@@ -113,7 +113,8 @@ CCQ_API void ccq_default_params(ccq_params *p);
  * Supported: Dk = Dv in {64, 128}; T >= 0; B, H >= 1.  in_dtype BF16 runs the
  * chunkwise tensor-core kernel for Dk = Dv = 128 and the recurrent kernel
  * otherwise; FP32 always runs the recurrent kernel (fp32 arithmetic; the
- * backbone state token by token, the CCQ read in blocks of 32 tokens).
+ * backbone state token by token, the CCQ read in blocks of 32 tokens except
+ * for short sequences).
  * Gate range of the chunkwise kernels.  A chunk's decays are applied as factors
  * measured from reference tokens inside the chunk.  The default kernel (AUTO,
  * CHUNKWISE) has one reference, the chunk midpoint; it is exact (up to rounding)

@@ -226,7 +226,7 @@ __device__ __forceinline__ void token_scalars(const GdnBwdArgs &a, int b, int h,
 
 // Sums over a row's columns in eight interleaved parts (columns p, p + 8, ..., each summed in order, then
 // the parts in order): four neighbouring threads take two parts each.  The order is that of row_sums() in
-// ccq_gdn_bwd_kernels.cuh, so that a row rounds to the same bf16 operands in either kernel.
+// ccq_gdn_bwd_kernels.cuh.
 __device__ __forceinline__ float parts_total(float p0, float p1, int lane) {
     float s = 0.f;
 #pragma unroll
@@ -245,8 +245,10 @@ __device__ __forceinline__ void load_parts(const uint8_t *tile, int row, int qtr
 __device__ __forceinline__ float lo_bf16(uint32_t w) { return __uint_as_float(w << 16); }
 __device__ __forceinline__ float hi_bf16(uint32_t w) { return __uint_as_float(w & 0xffff0000u); }
 // 1 / |row| of the raw q (threads 0-255) and k (256-511) tiles: row (tid % 256) / 4, the row's four
-// threads return the same value; w keeps the values read.  ODD_FIRST: the k rows' parts are added odd part of
-// each pair first, the order in which the CUDA-core kv kernel's atomics mostly arrive.
+// threads return the same value; w keeps the values read.  ODD_FIRST (the kv kernel): the k rows' parts are added odd
+// part of each pair first, as the generic kv kernel mostly adds them by atomics, so a row's kbar can round to
+// another bf16 there than in the local kernel.  Neither order is the more accurate one; the gradients' errors
+// against 64 bits are the same with either.
 template <bool ODD_FIRST = false>
 __device__ __forceinline__ float row_norms(const uint8_t *qt, const uint8_t *kt, int tid, int l2norm, uint32_t (&w)[16]) {
     load_parts(tid < 256 ? qt : kt, (tid & 255) >> 2, tid & 3, w);

@@ -457,6 +457,7 @@ gdn_chunk_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     const int bh = blockIdx.x / a.nseg, seg = blockIdx.x % a.nseg, b = bh / a.H, h = bh % a.H;
     const int H = a.H;
     // packed sequences: sequence b is rows tok0 .. tok0 + T of a [1][a.T][H][D] tensor
+    // (the offsets, their chunk bases and t0 are older than the WY kernel, so they are read before grid_wait())
     const bool vl = a.cu != nullptr;
     const int tok0 = vl ? static_cast<int>(a.cu[b]) : 0;
     const int T = vl ? static_cast<int>(a.cu[b + 1] - a.cu[b]) : a.T;

@@ -966,7 +966,8 @@ gla_bwd_kv_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
     int *status = a.status;
 
     // The load warp issues k and the gates (the row norms and the gate prefix) first, then,
-    // once the compute threads are released, the rest.
+    // once the compute threads are released, the rest.  (k and the gates are inputs, older than the q kernel that
+    // the chain starts with, so they need not wait for the kernel before.)
     if (warp == kThreadsKv / 32 && lane == 0) {
         for (int i = 0; i < kBars; ++i) mbar_init(&bar[i], 1);
         *abort_flag = 0;

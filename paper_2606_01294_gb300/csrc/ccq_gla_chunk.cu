@@ -201,7 +201,7 @@ gla_chunk_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     const float *m0 = segst ? segst + 2 * kD * kD : a.m0;
     const bool gate_f32 = a.gate_dtype != 0;
     const uint32_t g_bytes = gate_f32 ? kC * kD * 4 : kC * kD * 2;
-    const int64_t tseq0 = a.t0 ? a.t0[b] : 0;  // position before the sequence
+    const int64_t tseq0 = a.t0 ? a.t0[b] : 0;  // position before the sequence (older than the segments' kernels)
     int *status = a.status;
 
     if (tid == 0) {

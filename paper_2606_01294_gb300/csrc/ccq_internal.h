@@ -117,8 +117,9 @@ __host__ __device__ inline size_t ckpt_head_bytes(int T) {
 
 // Launches a kernel that waits by itself (grid_wait) for the kernel before it in the stream, so that its CTAs
 // are set up as that one's last CTAs leave, before its completion is flushed.  Every kernel of such a chain
-// waits, so a kernel also comes after all that precede the one it waits for; a chain's first kernel is launched
-// plainly.  Measured on GB300 against plain launches: Gated DeltaNet forward 4K (two kernels) 405.6 -> 401.9 us,
+// waits, so a kernel also comes after all that precede the one it waits for.  A chain's first kernel is launched
+// plainly and none triggers its dependents early, so what is older than the chain may be read before the wait: with
+// an early trigger, or a first kernel launched this way, such a read would be a race.  Measured on GB300 against plain launches: Gated DeltaNet forward 4K (two kernels) 405.6 -> 401.9 us,
 // 20K (four) 438 -> 429, training step 1941 -> 1917; GLA training step 899 -> 889.  (With
 // griddepcontrol.launch_dependents at the start of the kernels before, so that CTAs start still earlier: 414,
 // 441, 1940 and 905 us.)

@@ -16,10 +16,12 @@
 // the column's output (and, for the delta rule, kbar^T S) is a shuffle sum inside the warp -- no barrier.
 // The next block's inputs are in flight during the walk.
 //
-// What bounds it: the walk's chain of a token (shared-memory reads, multiply-adds, shuffles) and, before the walk
-// of a block, its scores and queries.  fp32, d = 64, B = 1, H = 2, T = 256: 49 us, 0.19 us a token; a
-// kernel that took every token through the whole of Algorithm 2 (six block barriers and a global load each,
-// one CTA per (batch, head)) took 277 us, 1.08 us a token.
+// What bounds it: latency, over a block's stages one after the other -- norms, scores, queries, the sum of C, two
+// cluster barriers -- with a CTA's eight warps alone on an SM, and only last the walk's chain of a token (shared-memory
+// reads, multiply-adds, shuffles).  GLA, d = 64, eight CTAs a sequence: a block of 32 tokens takes 5.3 us, of which the
+// walk is 1.4 (a block of two tokens takes that much less); the delta rule 8.4 and 4.6.  fp32, d = 64, B = 1, H = 2,
+// T = 256: 47 us, where the token-by-token kernel (six block barriers and a global load a token, one CTA per (batch,
+// head)) takes 277.  Short sequences stay with that kernel (recurrent_block_pays()).
 #include <cooperative_groups.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>

@@ -132,8 +132,9 @@ __device__ __forceinline__ void named_bar_arrive(int id, int count) {
 
 // ---------------------------------------------------------------- dependent launches
 
-// A kernel launched by launch_after() (ccq_internal.h) may start while the one before it in the stream
-// still runs: it waits here, before it touches global memory, until that one has completed.
+// A kernel launched by launch_after() (ccq_internal.h) starts as the last CTAs of the one before it in the stream leave,
+// before that one's stores are visible: it waits here until it has completed.  Before the wait a kernel reads
+// only what is older than its chain's first kernel (inputs, the offsets of packed sequences), and writes nothing.
 __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 // ---------------------------------------------------------------- TMA

@@ -103,3 +103,20 @@ def test_gdn_backward_workspace_at_sixteen_bytes(T):
     for n in ("dq", "dk", "dv", "dg", "dbeta", "dlambda", "dS0", "dC0", "dm0"):
         assert rel_err(g[n], ref["dlam" if n == "dlambda" else n]) <= TOL[torch.bfloat16], n
     assert int(w[at + room.numel():].sum()) == 0 and int(w[:at].sum()) == 0
+
+
+@pytest.mark.parametrize("gates", [0.0, -1e-5, -1e-3])
+@pytest.mark.parametrize("T", [700, 1000])
+def test_gla_short_split_with_gates_near_zero(gates, T):
+    """States that hardly forget keep what the segments' boundaries round off: outputs and final states of the split
+    walk, the unsplit one and two segments, each against the oracle.  S is a sum of products of two bf16 operands, one of them
+    of a bf16-rounded unit key (3 x 2^-9 of its norm); C and m of rounded unit keys (2 x 2^-9)."""
+    P = gen.make_inputs(GLA, 1, T, 16, 128, 128, dtype=torch.bfloat16, seed=63, lam="trained", keys="structured",
+                        gates=gates)
+    ref = oracle_forward(GLA, P)
+    for split in (0, 1, 2):
+        o, S = gpu_forward(GLA, P, seq_split=split)
+        compare(o, S, ref, TOL[torch.bfloat16], f"T={T} gates={gates} split={split}")
+        for n, bound in (("S", 3 * 2.0 ** -9), ("C", 2 * 2.0 ** -9), ("m", 2 * 2.0 ** -9)):
+            d = getattr(S, n).double().cpu() - torch.as_tensor(ref[n])
+            assert float(d.norm()) <= bound * float(torch.as_tensor(ref[n]).norm()), (n, split)
